@@ -150,11 +150,11 @@ typedef struct pv3d_eval_opts {
 /*
  * Stage timings (profile bit 0) and work counts (profile bit 1) of the last
  * pv3d_evaluate run with opts->profile set.  Stages: 0 light window and module setup, 1 binning
- * (triangle bins, scan, receiver lists), 2 tiles (fused path: the depth tests
+ * (triangle bins, scan, receiver lists), 2 tiles (fused path: the coverage bits
  * of the tiles taken one per warp; map path: tile rasterisation into the map),
- * 3 the tiles with many receivers or triangles (fused path, one per block,
- * rasterised in shared memory when they keep many triangles), 4 PV model
- * (with the texel gathers on the map path), 5 Kahan energy sums.  stage_ms
+ * 3 the tiles with many receivers or triangles (fused path, one per block), 4
+ * shaded samples per cell and PV model (map path: texel gathers and PV model),
+ * 5 Kahan energy sums.  stage_ms
  * sums CUDA-event intervals over the waves, recorded on the evaluation's stream.
  */
 typedef struct pv3d_profile {
@@ -163,21 +163,22 @@ typedef struct pv3d_profile {
     float stage_ms[8];
     float device_ms;
     int32_t reserved0;
-    int64_t sample_tests;      /* sample depth tests performed against rasterised tiles */
-    int64_t texel_visits;      /* texel-centre coverage tests */
-    int64_t texel_writes;      /* fragments: (texel read by a sample, triangle covering its centre) pairs
-                                  (rasterised dense tiles: every covered texel) */
-    int64_t tris_culled;       /* (triangle, tile) pairs skipped: on or behind every receiver plane */
+    int64_t sample_tests;      /* samples decided in tiles that are not lit throughout (map path: depth tests) */
+    int64_t texel_visits;      /* texels drawn as coverage (map path: texel-centre coverage tests) */
+    int64_t texel_writes;      /* those, and the texels at which a triangle's depth was compared with a
+                                  receiver plane (map path: fragments) */
+    int64_t tris_culled;       /* (triangle, tile) pairs skipped: behind every receiver plane */
     int64_t nonempty_tiles;
     int64_t binned_tris;
-    int64_t candidates;        /* receiver samples enumerated by the tile kernel (marking and testing) */
-    int64_t dense_tiles;       /* tiles rasterised at every texel */
-    int64_t sample_tiles;      /* tiles tested sample by sample against their few triangles (not rasterised) */
-    int64_t pair_tests;        /* (sample, triangle) coverage tests made by the sample-driven test */
+    int64_t candidates;        /* samples of the cells looked at (map path: samples enumerated by the marking) */
+    int64_t dense_tiles;       /* map path: tiles rasterised at every texel */
+    int64_t sample_tiles;      /* tiles in which no triangle was drawn (all behind the receivers) */
+    int64_t pair_tests;        /* (sample, triangle) depth tests at texels that a triangle's crossing of a
+                                  receiver plane leaves open */
     int64_t heavy_tiles;       /* tiles with many receivers or triangles, taken one per block (stage 3) */
     int64_t heavy_sample_tests;   /* their share of sample_tests */
     int64_t heavy_texel_writes;   /* their share of texel_writes */
-    int64_t heavy_why[3];      /* heavy tiles by cause: too many receivers, binned triangles, kept triangles */
+    int64_t heavy_why[3];      /* heavy tiles by cause: too many receivers, binned triangles, kept or open triangles */
 } pv3d_profile;
 
 /*

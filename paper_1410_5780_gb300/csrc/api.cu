@@ -113,9 +113,9 @@ struct pv3d_ctx {
     uint32_t next_id = 1;
     // workspace pools
     DevBuf lp, win, ms, ms_p, ms_pu, ms_beam, ms_iu, ss_i, sq_p, sq_pu, kahan_str, js_p, js_pu, js_bin, heat, sa_p, sa_pu,
-        kahan_arr, cs_cnt, cs_bits, t_far, t_cnt, t_off, t_cur, t_slot, t_rcnt, t_plane, t_roff, t_rcur, nonempty, heavy, bins, pairs, recv, map,
+        kahan_arr, cs_cnt, cov, touch, t_far, t_cnt, t_off, t_cur, t_slot, t_rcnt, t_plane, t_roff, t_rcur, nonempty, heavy, bins, pairs, recv, map,
         big, block_sums, ctr, waves, jobs, kahan_mod, kahan_cell, staging;
-    int64_t bin_cap = 0, map_cap_tiles = 0, big_cap = 0, recv_cap = 0;
+    int64_t bin_cap = 0, map_cap_tiles = 0, big_cap = 0, recv_cap = 0, cov_cap = 0;
     uint64_t bufgen = 0;  // bumped whenever a pool is reallocated (captured graphs hold its pointers)
     // captured wave graph: the kernels read the wave from fixed descriptor slots
     DevBuf wave_slot, jobs_slot;
@@ -1136,13 +1136,12 @@ static WaveDev pack_wave(std::vector<JobDev>& jobs, size_t first, size_t last, i
         W.tot_ss += (int64_t)J.k * (J.n_str ? J.n_sub_tot : 0);
         W.tot_sq += (int64_t)J.k * J.n_str;
         W.tot_heat += (int64_t)J.heat_az * J.heat_zen;
-        if (J.out_bits) W.want_bits = 1;
     }
     return W;
 }
 
 static int ensure_workspace(pv3d_ctx* c, int64_t js, int64_t te, int64_t ms, int64_t cs, int tile, bool fused,
-                            bool want_bits, int64_t ss = 0, int64_t sq = 0, int64_t sa = 0)
+                            int64_t ss = 0, int64_t sq = 0, int64_t sa = 0)
 {
     int rc;
     if (sa > 0 && ((rc = ensure(c, c->sa_p, sa * 4)) || (rc = ensure(c, c->sa_pu, sa * 4)))) return rc;
@@ -1163,7 +1162,14 @@ static int ensure_workspace(pv3d_ctx* c, int64_t js, int64_t te, int64_t ms, int
         (rc = ensure(c, c->t_rcur, te * 4)) || (rc = ensure(c, c->nonempty, te * 4)) || (rc = ensure(c, c->heavy, te * 4)) ||
         (rc = ensure(c, c->block_sums, scan_tiles * 24)) || (rc = ensure(c, c->ctr, sizeof(Counters))))
         return rc;
-    if (fused && want_bits && (rc = ensure(c, c->cs_bits, cs * 8))) return rc;
+    if (fused) {
+        // tile records (one plane's bits and a header each, 16-byte units): one
+        // for every tile, or 256 MiB, or one for every second module of a
+        // wave, whichever is the least that holds; grown on overflow
+        const int64_t rec = (int64_t)tile * tile / 128 + 8;
+        c->cov_cap = std::max<int64_t>(c->cov_cap, std::min<int64_t>(te * rec + 4096, std::max<int64_t>(ms * rec / 2, 1 << 24)));
+        if ((rc = ensure(c, c->cov, (size_t)c->cov_cap * 16)) || (rc = ensure(c, c->touch, ms * 16))) return rc;
+    }
     if (c->bin_cap == 0) c->bin_cap = 1 << 22;
     if (c->big_cap == 0) c->big_cap = 1 << 18;
     if (c->recv_cap == 0) c->recv_cap = 1 << 20;
@@ -1198,7 +1204,8 @@ static Buffers buffers_of(pv3d_ctx* c)
     B.js_pu = (float*)c->js_pu.p;
     B.js_bin = (int32_t*)c->js_bin.p;
     B.cs_cnt = (uint32_t*)c->cs_cnt.p;
-    B.cs_bits = (unsigned long long*)c->cs_bits.p;
+    B.cov = (uint32_t*)c->cov.p;
+    B.touch = (uint4*)c->touch.p;
     B.t_far = (uint32_t*)c->t_far.p;
     B.t_cnt = (uint32_t*)c->t_cnt.p;
     B.t_off = (uint32_t*)c->t_off.p;
@@ -1476,13 +1483,14 @@ static int evaluate_plain(pv3d_ctx* c, uint32_t gen_id, const pv3d_eval_opts* o,
     const int extras = (es.strings ? 1 : 0) | (es.heat ? 2 : 0) | (es.arrays ? 4 : 0);
     Counters hc{};
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((rc = ensure_workspace(c, mjs, mte, mms, mcs, es.tile, es.fused, d_bits != nullptr, mss, msq, msa)))
+        if ((rc = ensure_workspace(c, mjs, mte, mms, mcs, es.tile, es.fused, mss, msq, msa)))
             return rc;
         for (auto& W : waves) {
             W.bin_cap = c->bin_cap;
             W.map_cap_tiles = c->map_cap_tiles;
             W.big_cap = c->big_cap;
             W.recv_cap = c->recv_cap;
+            W.cov_cap = c->cov_cap;
         }
         if ((rc = stage_descriptors(c, waves, jobs, st))) return rc;
         CUDA_TRY(c, cudaMemsetAsync(c->ctr.p, 0, sizeof(Counters), st));
@@ -1515,6 +1523,7 @@ static int evaluate_plain(pv3d_ctx* c, uint32_t gen_id, const pv3d_eval_opts* o,
         if (hc.overflow & 2u) c->map_cap_tiles = (int64_t)(hc.need_tiles * 5 / 4 + 16);
         if (hc.overflow & 4u) c->big_cap = (int64_t)(hc.need_big * 5 / 4 + 1024);
         if (hc.overflow & 8u) c->recv_cap = (int64_t)(hc.need_recv * 5 / 4 + 1024);
+        if (hc.overflow & 16u) c->cov_cap = (int64_t)(hc.need_cov * 5 / 4 + 4096);
     }
     float ms = 0;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
@@ -1989,7 +1998,6 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
     std::vector<pv3d_ctx::Request*> in_wave;
     std::vector<int> ks;
     int64_t scratch = 0;
-    bool want_bits = false;
     int extras = 0;  // string (1) and array (4) kernels in the wave
     const size_t na = c->active.size();
     for (size_t q = 0; q < na; ++q) {
@@ -2007,7 +2015,6 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
                                 nullptr, 0, 0, (float2*)r.karr.p, r.d_ap, r.d_apu));
         in_wave.push_back(&r);
         ks.push_back(k);
-        want_bits = want_bits || r.d_bits;
         extras |= (r.es.strings ? 1 : 0) | (r.es.arrays ? 4 : 0);
     }
     c->rr = (c->rr + jobs.size()) % std::max<size_t>(na, 1);
@@ -2022,11 +2029,12 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
         std::lock_guard<std::mutex> g(c->gpu_mu);
         cudaSetDevice(c->device);
         cudaStream_t st = c->serve_stream;
-        rc = ensure_workspace(c, W.tot_js, W.tot_te, W.tot_ms, W.tot_cs, c->opts.tile, true, want_bits, W.tot_ss,
-                              W.tot_sq, W.tot_sa);
+        rc = ensure_workspace(c, W.tot_js, W.tot_te, W.tot_ms, W.tot_cs, c->opts.tile, true, W.tot_ss, W.tot_sq,
+                              W.tot_sa);
         if (!rc) {
             W.bin_cap = c->bin_cap; W.map_cap_tiles = c->map_cap_tiles;
             W.big_cap = c->big_cap; W.recv_cap = c->recv_cap;
+            W.cov_cap = c->cov_cap;
             rc = stage_descriptors(c, waves, jobs, st);
         }
         if (!rc && cudaMemsetAsync(c->ctr.p, 0, sizeof(Counters), st) != cudaSuccess) rc = PV3D_E_DEVICE;
@@ -2042,6 +2050,7 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
             if (hc.overflow & 1u) c->bin_cap = (int64_t)(hc.need_bins * 5 / 4 + 1024);
             if (hc.overflow & 4u) c->big_cap = (int64_t)(hc.need_big * 5 / 4 + 1024);
             if (hc.overflow & 8u) c->recv_cap = (int64_t)(hc.need_recv * 5 / 4 + 1024);
+            if (hc.overflow & 16u) c->cov_cap = (int64_t)(hc.need_cov * 5 / 4 + 4096);
             for (auto* r : in_wave) {
                 const GenH& g = c->gens.at(r->gen_id);
                 cudaMemsetAsync(r->kmod.p, 0, (size_t)g.M * 2 * sizeof(float2), st);
@@ -2233,7 +2242,7 @@ extern "C" void pv3d_destroy(pv3d_ctx* c)
     release_buf(c->wave_slot);
     release_buf(c->jobs_slot);
     DevBuf* bufs[] = {&c->lp, &c->win, &c->ms, &c->ms_p, &c->ms_pu, &c->ms_beam, &c->ms_iu, &c->ss_i, &c->sq_p,
-                      &c->sq_pu, &c->kahan_str, &c->js_p, &c->js_pu, &c->js_bin, &c->heat, &c->sa_p, &c->sa_pu, &c->kahan_arr, &c->cs_cnt, &c->cs_bits, &c->t_far,
+                      &c->sq_pu, &c->kahan_str, &c->js_p, &c->js_pu, &c->js_bin, &c->heat, &c->sa_p, &c->sa_pu, &c->kahan_arr, &c->cs_cnt, &c->cov, &c->touch, &c->t_far,
                       &c->t_cnt, &c->t_off, &c->t_cur, &c->t_slot, &c->t_rcnt, &c->t_plane, &c->t_roff, &c->t_rcur, &c->nonempty, &c->heavy,
                       &c->bins, &c->pairs, &c->recv, &c->map, &c->big,
                       &c->block_sums, &c->ctr, &c->waves, &c->jobs, &c->kahan_mod, &c->kahan_cell, &c->staging};

@@ -16,19 +16,18 @@
 //   k_bin_big     same for triangles that span many tiles, one warp each
 //   k_scan_*      bin offsets, the list of non-empty tiles, receiver offsets
 //   k_scatter, k_recv_fill   write the bins and receiver lists
-//   k_tile_warp   one warp per non-empty tile: the depth test of every sample
-//                 that reads the tile against the tile's kept triangles (those
-//                 in front of its receivers' planes), sub-block masks, one atomic
-//                 per sample row for the cell tallies -- the same decision as a
-//                 test against the tile's stored nearest depth (Fig. 3: the
-//                 depth buffer keeps the surface nearest the sun)
-//   k_raster_test one CTA per tile that a warp cannot take (many receivers or
-//                 triangles): block-wide sample-driven test, or a shared-memory
-//                 depth tile (texel-centre coverage, atomicMin of
-//                 order-preserving depth keys) and the test of its samples
-//   k_pv          per (step, module), one per lane: irradiance per cell,
-//                 substring currents, bypass-diode maximum power point
-//                 (Section 2, step 4)
+//   k_tile_warp   one warp per non-empty tile: one bit per texel and receiver
+//                 plane, covered by something in front of that plane (Fig. 3:
+//                 the depth buffer keeps the surface nearest the sun -- the
+//                 samples of a plane need to know only whether that surface is
+//                 in front of them), and the few texels where a triangle
+//                 crosses the plane and depths must be compared
+//   k_raster_test one CTA per tile that a warp cannot take (many triangles)
+//   k_pv          per (step, module), one per lane: the maximum power point of
+//                 modules over lit tiles, the list of the others
+//   k_cells       per listed module, one warp: shaded samples per cell from
+//                 the tiles' bits, irradiance per cell, substring currents,
+//                 bypass-diode maximum power point (Section 2, step 4)
 //   k_string, k_array   series strings and strings in parallel (when asked)
 //   k_gen_step, k_heat  sky map of the effective shading (when asked)
 //   k_epilogue    Kahan-compensated FP32 sums over the wave's steps in step
@@ -36,7 +35,7 @@
 //                 (beam loss, when asked)
 // A job may cover one window group of a generator (its own light window);
 // the generator's other modules then enter its map as occluder meshlets.
-// The map path replaces the tile kernels + k_pv by k_raster_map (tiles stored
+// The map path replaces the tile kernels, k_pv and k_cells by k_raster_map (tiles stored
 // to an HBM shadow map with 16-byte stores) + k_sample (texel gathers, ballot
 // tallies, PV model).  Outside the waves: the clear-sky sun table and ideal
 // tracker poses (k_sun_table, k_gather_sun, k_ideal_poses) and the diffuse
@@ -67,14 +66,8 @@ __device__ __forceinline__ float okey_inv(uint32_t k)
 
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 
-// Per-(step, cell) shaded-sample tallies, one byte per entry e (a count is at
-// most n^2 <= 225), four bytes to a 32-bit word: the tile kernels add to a
-// byte with a word atomic (no carry can leave the byte), the PV kernels read
-// bytes.
-__device__ __forceinline__ void tally_add(uint32_t* words, int64_t e, uint32_t cnt)
-{
-    atomicAdd(&words[e >> 2], cnt << (8 * (int)(e & 3)));
-}
+// Per-(step, cell) shaded samples, one byte per entry e (a count is at most
+// n^2 <= 225).
 __device__ __forceinline__ uint32_t tally_get(const uint32_t* words, int64_t e)
 {
     return reinterpret_cast<const uint8_t*>(words)[e];
@@ -251,7 +244,38 @@ __device__ __forceinline__ bool behind_key(float d, float bias, uint32_t key, fl
 // k_clear: reset the wave's accumulators (sizes read from the wave descriptor,
 // so the whole wave can be replayed from one captured graph)
 // ---------------------------------------------------------------------------
-__global__ void k_clear(const WaveDev* __restrict__ W, Buffers B)
+
+// Zero n bytes from p by the whole grid: 16 bytes at a time between the first
+// and the last 16-byte boundary.
+__device__ __forceinline__ void clear_bytes(void* p, int64_t n, int64_t i0, int64_t stride)
+{
+    uint8_t* b = static_cast<uint8_t*>(p);
+    const int64_t head = min(n, (int64_t)((16u - (uint32_t)((uintptr_t)b & 15u)) & 15u)), quads = (n - head) / 16;
+    const int64_t tail = head + 16 * quads;
+    uint4* q = reinterpret_cast<uint4*>(b + head);
+    for (int64_t i = i0; i < quads; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t i = i0; i < head + n - tail; i += stride) b[i < head ? i : tail + i - head] = 0;
+}
+
+// Zero the rows of a per-cell output of job J (E bytes a cell; out_cstride
+// cells a row, of which the job's n_cells).
+template <int E>
+__device__ __forceinline__ void clear_rows(uint8_t* p, const JobDev& J, int64_t i0, int64_t stride)
+{
+    p += (int64_t)J.out_row0 * J.out_cstride * E;
+    if (J.out_cstride == J.n_cells) {
+        clear_bytes(p, (int64_t)J.k * J.n_cells * E, i0, stride);
+    } else {
+        for (int64_t i = i0; i < (int64_t)J.k * J.n_cells; i += stride) {
+            const int64_t r = i / J.n_cells;
+            uint8_t* q = p + (r * J.out_cstride + i - r * J.n_cells) * E;
+            if (E == 8) *reinterpret_cast<unsigned long long*>(q) = 0ull;
+            else *q = 0;
+        }
+    }
+}
+
+__global__ void k_clear(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs, Buffers B)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -261,6 +285,10 @@ __global__ void k_clear(const WaveDev* __restrict__ W, Buffers B)
         B.ctr->raster_next = 0u;
         B.ctr->n_heavy = 0u;
         B.ctr->n_pairs = 0ull;
+        B.ctr->cov_next = 0ull;
+        B.ctr->n_touch = 0u;
+        B.ctr->n_first = 0u;
+        B.ctr->n_rest = 0u;
         B.ctr->heavy_next = 0u;
     }
     const int64_t nw = 4 * W->tot_js, nt = W->tot_te;
@@ -271,11 +299,13 @@ __global__ void k_clear(const WaveDev* __restrict__ W, Buffers B)
         B.t_rcnt[i] = 0u;
         B.t_plane[i] = kPlaneNone;
     }
-    if (W->fused) {
-        const int64_t nc = W->tot_cs, nw = (nc + 3) / 4;  // tallies, and their words
-        for (int64_t i = i0; i < nw; i += stride) B.cs_cnt[i] = 0u;
-        if (W->want_bits)
-            for (int64_t i = i0; i < nc; i += stride) B.cs_bits[i] = 0ull;
+    // fused path: the outputs per cell start at zero, k_cells writes the cells
+    // that may be shaded
+    for (int q = 0; W->fused && q < W->n_jobs; ++q) {
+        const JobDev& J = jobs[q];
+        if (J.kahan_cell) clear_bytes(reinterpret_cast<uint8_t*>(B.cs_cnt) + J.cs_base, (int64_t)J.k * J.n_cells, i0, stride);
+        if (J.out_counts) clear_rows<1>(J.out_counts, J, i0, stride);
+        if (J.out_bits) clear_rows<8>(reinterpret_cast<uint8_t*>(J.out_bits), J, i0, stride);
     }
 }
 
@@ -428,8 +458,18 @@ __device__ __forceinline__ TileRange module_tiles(const ModStep& s, const Module
     t.tx1 = max(0, min(R - 1, (int)floorf(xmax))) >> sh;
     t.ty0 = max(0, min(R - 1, (int)floorf(ymin))) >> sh;
     t.ty1 = max(0, min(R - 1, (int)floorf(ymax))) >> sh;
+    if ((R >> sh) == 0) t.ty1 = t.ty0 - 1;  // a map smaller than a tile has none
     t.dmax = dmax;
     return t;
+}
+
+// Threads that share a (step, module) item's tiles: a warp when the wave has
+// too few items to fill the grid otherwise (a module may touch a hundred tiles:
+// for two modules over a day of suns, R = 1024, a thread each made the set-up
+// kernels 105 us, a warp each 32 us).
+__device__ __forceinline__ int mod_group(int64_t tot)
+{
+    return tot * 32 <= (int64_t)gridDim.x * blockDim.x ? 32 : 1;
 }
 
 __global__ void k_modsetup(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs, Buffers B)
@@ -438,8 +478,9 @@ __global__ void k_modsetup(const WaveDev* __restrict__ W, const JobDev* __restri
     const int nj = W->n_jobs;
     const int sh = W->tile_sh;
     const int u24 = W->depth_u24;
-    for (int64_t item = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; item < tot;
-         item += (int64_t)gridDim.x * blockDim.x) {
+    const int grp = mod_group(tot), sub = threadIdx.x & (grp - 1);
+    for (int64_t item = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / grp; item < tot;
+         item += (int64_t)gridDim.x * blockDim.x / grp) {
         int j = job_of(nj, item, [&](int q) { return jobs[q].it_mod; });
         const JobDev& J = jobs[j];
         int64_t li = item - J.it_mod;
@@ -473,7 +514,32 @@ __global__ void k_modsetup(const WaveDev* __restrict__ W, const JobDev* __restri
         float tan_i = sqrtf(fmaxf(0.f, 1.f - cc * cc)) / cc;
         s.bias = lp.delta * (0.70710678f * tan_i + 0.03125f);
         if (u24) s.bias += 2.f / lp.qscale;
-        B.ms[J.ms_base + li] = s;
+        // the depth plane of the samples over the light plane, and how far a
+        // sample's depth may lie from the plane's at the centre of its texel:
+        // the slope over half a texel, the rounding of positions and depths
+        // (of this module and of others on the plane, whose bias may differ by
+        // the rounding of cos i under the square root), of the plane's own
+        // coefficients, and a few steps of 24-bit depth.  No plane within a
+        // degree of the sun.
+        const float lu = M.cu * M.pitch, lv = M.cv * M.pitch;
+        const float det = s.tax * s.tby - s.tay * s.tbx;
+        const float dsum = fabsf(s.tax * s.tby) + fabsf(s.tay * s.tbx);
+        if (fabsf(det) > 1e-6f * dsum && fabsf(c) > 0.017452406f) {
+            const float inv_det = 1.f / det;
+            s.pa = (s.da * s.tby - s.db * s.tay) * inv_det;
+            s.pb = (s.db * s.tax - s.da * s.tbx) * inv_det;
+            const float ex = fabsf(lu * s.tax) + fabsf(lv * s.tbx) + 256.f;
+            const float ey = fabsf(lu * s.tay) + fabsf(lv * s.tby) + 256.f;
+            s.hs = 0.52f * (fabsf(s.pa) + fabsf(s.pb)) +
+                   4e-6f * fabsf(dsum * inv_det) * (fabsf(s.pa) * ex + fabsf(s.pb) * ey) +
+                   2e-6f * (fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + lu + lv) + 2e-5f + 1e-3f * lp.delta +
+                   (u24 ? 8.f / lp.qscale : 0.f);
+        } else {
+            s.pa = s.pb = 0.f;
+            s.hs = INFINITY;
+        }
+        s.pad = 0.f;
+        if (sub == 0) B.ms[J.ms_base + li] = s;
         // A triangle shades a sample only where its depth is below the
         // sample's depth minus the bias, so a tile may drop every triangle whose
         // nearest point is not nearer than (max sample depth - bias).
@@ -481,27 +547,33 @@ __global__ void k_modsetup(const WaveDev* __restrict__ W, const JobDev* __restri
         const uint32_t far_key = u24 ? depth_store_key(tr.dmax - s.bias, lp, 1) + 2u : okey(tr.dmax - s.bias);
         const int64_t te0 = J.te_base + (int64_t)ls * J.tiles_x * J.tiles_x;
         for (int ty = tr.ty0; ty <= tr.ty1; ++ty)
-            for (int tx = tr.tx0; tx <= tr.tx1; ++tx) {
+            for (int tx = tr.tx0 + sub; tx <= tr.tx1; tx += grp) {
                 const int64_t te = te0 + (int64_t)ty * J.tiles_x + tx;
                 atomicMax(&B.t_far[te], far_key);
                 atomicAdd(&B.t_rcnt[te], 1u);
                 // the plane group shared by every receiver of the tile
                 const uint32_t pl = (uint32_t)M.plane;
                 const uint32_t old = atomicCAS(&B.t_plane[te], kPlaneNone, pl);
+                // fused path: a module of the tile, for the plane of a tile of one group
+                if (old == kPlaneNone) B.t_roff[te] = (uint32_t)m;
                 if (old != kPlaneNone && old != pl && old != kPlaneMixed) atomicExch(&B.t_plane[te], kPlaneMixed);
             }
     }
 }
 
-// After the scan: list each module as a receiver of the non-empty tiles it touches.
+// After the scan: list each module as a receiver of the non-empty tiles it
+// touches (fused path: only of tiles of several plane groups, the others need
+// no list).
 __global__ void k_recv_fill(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs, Buffers B)
 {
     const int64_t tot = W->tot_mod;
     const int nj = W->n_jobs;
     const int sh = W->tile_sh;
     const int64_t cap = W->recv_cap;
-    for (int64_t item = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; item < tot;
-         item += (int64_t)gridDim.x * blockDim.x) {
+    const int fused = W->fused;
+    const int grp = mod_group(tot), sub = threadIdx.x & (grp - 1);
+    for (int64_t item = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / grp; item < tot;
+         item += (int64_t)gridDim.x * blockDim.x / grp) {
         int j = job_of(nj, item, [&](int q) { return jobs[q].it_mod; });
         const JobDev& J = jobs[j];
         int64_t li = item - J.it_mod;
@@ -511,9 +583,9 @@ __global__ void k_recv_fill(const WaveDev* __restrict__ W, const JobDev* __restr
         const TileRange tr = module_tiles(s, J.mods[m], J.R, sh);
         const int64_t te0 = J.te_base + (int64_t)ls * J.tiles_x * J.tiles_x;
         for (int ty = tr.ty0; ty <= tr.ty1; ++ty)
-            for (int tx = tr.tx0; tx <= tr.tx1; ++tx) {
+            for (int tx = tr.tx0 + sub; tx <= tr.tx1; tx += grp) {
                 const int64_t te = te0 + (int64_t)ty * J.tiles_x + tx;
-                if (B.t_cnt[te] == 0u) continue;
+                if (B.t_cnt[te] == 0u || (fused && B.t_plane[te] != kPlaneMixed)) continue;
                 const uint32_t pos = atomicAdd(&B.t_rcur[te], 1u);
                 if (pos < (uint64_t)cap) B.recv[pos] = (uint32_t)m;
             }
@@ -539,6 +611,29 @@ __device__ __forceinline__ void project_point(const LightParams& lp, float x, fl
     d = -__fmaf_rn(z, lp.sz, __fmaf_rn(y, lp.sy, __fmul_rn(x, lp.sx)));
 }
 
+// Triangle q of a window group's occluder modules (every module of the
+// generator, posed for the step and projected like the scene).  Not inlined:
+// the pose's sines and cosines would sit in every kernel that reads triangles.
+__device__ __noinline__ void occ_tri_texel(const JobDev& J, const LightParams& lp, int ls, int q, TriT& T)
+{
+    float3 o, u, v;
+    const ModuleDev& M = J.occ_mods[q >> 1];
+    posed_module(J, M, J.step0 + ls, o, u, v);
+    const float lu = M.cu * M.pitch, lv = M.cv * M.pitch;
+    // corners c0 = O, c1 = O + lu U, c2 = O + lu U + lv V, c3 = O + lv V;
+    // triangles (c0, c1, c2) and (c0, c2, c3)
+    const float a1 = lu, b1 = (q & 1) ? lv : 0.f;
+    const float a2 = (q & 1) ? 0.f : lu, b2 = lv;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float a = k == 0 ? 0.f : (k == 1 ? a1 : a2), b = k == 0 ? 0.f : (k == 1 ? b1 : b2);
+        const float x = __fmaf_rn(b, v.x, __fmaf_rn(a, u.x, o.x));
+        const float y = __fmaf_rn(b, v.y, __fmaf_rn(a, u.y, o.y));
+        const float z = __fmaf_rn(b, v.z, __fmaf_rn(a, u.z, o.z));
+        project_point(lp, x, y, z, T.x[k], T.y[k], T.d[k]);
+    }
+}
+
 // Triangle `t` of job J (scene triangle, or module triangle after the scene's)
 // at local step ls in texel coordinates.  Module triangles come from the
 // job's own module frames (ModStep), or, for a window group, from every
@@ -547,23 +642,9 @@ __device__ __forceinline__ void tri_texel(const JobDev& J, const Buffers& B, con
                                           int ls, int t, TriT& T)
 {
     if (t >= J.n_tris && J.occ_mods) {
-        const int q = t - J.n_tris;
-        float3 o, u, v;
-        posed_module(J, J.occ_mods[q >> 1], J.step0 + ls, o, u, v);
-        const ModuleDev& M = J.occ_mods[q >> 1];
-        const float lu = M.cu * M.pitch, lv = M.cv * M.pitch;
-        // corners c0 = O, c1 = O + lu U, c2 = O + lu U + lv V, c3 = O + lv V;
-        // triangles (c0, c1, c2) and (c0, c2, c3)
-        const float a1 = lu, b1 = (q & 1) ? lv : 0.f;
-        const float a2 = (q & 1) ? 0.f : lu, b2 = lv;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float a = k == 0 ? 0.f : (k == 1 ? a1 : a2), b = k == 0 ? 0.f : (k == 1 ? b1 : b2);
-            const float x = __fmaf_rn(b, v.x, __fmaf_rn(a, u.x, o.x));
-            const float y = __fmaf_rn(b, v.y, __fmaf_rn(a, u.y, o.y));
-            const float z = __fmaf_rn(b, v.z, __fmaf_rn(a, u.z, o.z));
-            project_point(lp, x, y, z, T.x[k], T.y[k], T.d[k]);
-        }
+        TriT O;
+        occ_tri_texel(J, lp, ls, t - J.n_tris, O);
+        T = O;
         return;
     }
     if (t < J.n_tris) {
@@ -707,7 +788,7 @@ __global__ void __launch_bounds__(256, 4) k_bin(const WaveDev* __restrict__ W, c
         const int R = J.R;
         const int64_t js = J.js_base + ls;
         const LightParams& lp = B.lp[js];
-        if (!lp.valid) continue;
+        if (!lp.valid || J.tiles_x == 0) continue;  // (a map smaller than a tile has none)
         const int64_t te0 = J.te_base + (int64_t)ls * J.tiles_x * J.tiles_x;
         // scene meshlets, then (window groups) occluder-module meshlets, both
         // with boxes, then the job's own module meshlets
@@ -927,6 +1008,7 @@ __global__ void __launch_bounds__(256) k_scatter(const WaveDev* __restrict__ W, 
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;
+constexpr unsigned long long kFirstBins = 48;  // fused path: tiles of more triangles are taken first
 constexpr int kScanTile = kScanThreads * kScanPer;
 
 // Block-wide exclusive scan of three counters; returns the block totals.
@@ -967,12 +1049,12 @@ __device__ __forceinline__ void block_scan3(unsigned long long v[3], unsigned lo
     __syncthreads();
 }
 
-__device__ __forceinline__ void scan_values(const Buffers& B, int64_t i, unsigned long long v[3])
+__device__ __forceinline__ void scan_values(const Buffers& B, int64_t i, int fused, unsigned long long v[3])
 {
     const uint32_t c = B.t_cnt[i];
     v[0] = c;
     v[1] = c ? 1u : 0u;
-    v[2] = c ? B.t_rcnt[i] : 0u;
+    v[2] = c && (!fused || B.t_plane[i] == kPlaneMixed) ? B.t_rcnt[i] : 0u;
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_a(const WaveDev* __restrict__ W, Buffers B)
@@ -986,7 +1068,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_a(const WaveDev* __restri
         for (int q = 0; q < kScanPer; ++q) {
             if (base + q < tot) {
                 unsigned long long x[3];
-                scan_values(B, base + q, x);
+                scan_values(B, base + q, W->fused, x);
                 v[0] += x[0]; v[1] += x[1]; v[2] += x[2];
             }
         }
@@ -1040,7 +1122,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_c(const WaveDev* __restri
         int64_t base = st * kScanTile + (int64_t)threadIdx.x * kScanPer;
 #pragma unroll
         for (int q = 0; q < kScanPer; ++q) {
-            if (base + q < tot) scan_values(B, base + q, x[q]);
+            if (base + q < tot) scan_values(B, base + q, W->fused, x[q]);
             else x[q][0] = x[q][1] = x[q][2] = 0ull;
             v[0] += x[q][0]; v[1] += x[q][1]; v[2] += x[q][2];
         }
@@ -1057,37 +1139,42 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_c(const WaveDev* __restri
                 B.t_off[i] = (uint32_t)min(v[0], 0xFFFFFFFFull);
                 B.t_cur[i] = (uint32_t)min(v[0], 0xFFFFFFFFull);
                 B.t_slot[i] = (uint32_t)min(v[1], 0xFFFFFFFFull);
-                B.t_roff[i] = (uint32_t)min(v[2], 0xFFFFFFFFull);
-                B.t_rcur[i] = (uint32_t)min(v[2], 0xFFFFFFFFull);
-                B.nonempty[v[1]] = (uint32_t)i;
+                if (x[q][2]) {  // (fused path: t_roff of a tile of one plane group keeps its module)
+                    B.t_roff[i] = (uint32_t)min(v[2], 0xFFFFFFFFull);
+                    B.t_rcur[i] = (uint32_t)min(v[2], 0xFFFFFFFFull);
+                }
+                if (!W->fused) B.nonempty[v[1]] = (uint32_t)i;
             }
             v[0] += x[q][0]; v[1] += x[q][1]; v[2] += x[q][2];
+            // fused path: tiles of many triangles from the front of the list,
+            // the others from its end, so that k_tile_warp starts with the
+            // long ones and the short ones fill its tail
+            if (W->fused) {
+                const bool ne = i < tot && x[q][1], first = ne && x[q][0] > kFirstBins;
+                const unsigned int bf = __ballot_sync(0xffffffffu, first), br = __ballot_sync(0xffffffffu, ne && !first);
+                const int lane = threadIdx.x & 31;
+                unsigned int pos = 0;
+                if (lane == 0 && bf) pos = atomicAdd(&B.ctr->n_first, (unsigned int)__popc(bf));
+                if (lane == 1 && br) pos = atomicAdd(&B.ctr->n_rest, (unsigned int)__popc(br));
+                const unsigned int pf = __shfl_sync(0xffffffffu, pos, 0), pr = __shfl_sync(0xffffffffu, pos, 1);
+                const unsigned int below = (1u << lane) - 1u;
+                if (first) B.nonempty[pf + __popc(bf & below)] = (uint32_t)i;
+                else if (ne) B.nonempty[tot - 1 - (int64_t)(pr + __popc(br & below))] = (uint32_t)i;
+            }
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// per-tile work: receivers, the sample-driven depth test, and the tile
-// rasteriser (shared by the fused and the map kernels)
+// per-tile work: receivers and the tile rasteriser (map path)
 // ---------------------------------------------------------------------------
 constexpr int kRecvChunk = 64;  // receivers staged in shared memory at a time (two per lane of one warp)
 constexpr int kTriBatchMax = 128;  // triangles set up in shared memory at a time by the rasteriser (one per thread)
-constexpr int kMaxTri = 256;    // triangles a block-wide tile may keep for the sample-driven test
-// Sub-blocks per tile side in the sample-driven test (4, 8 and 16 texels on
-// 32-, 64- and 128-texel tiles; a 16 x 16 grid on 128-texel tiles tests fewer
-// triangles per sample but costs more in its masks than it saves).
+// Sub-blocks per tile side (4, 8 and 16 texels on 32-, 64- and 128-texel tiles).
 template <int TS>
 struct SubGrid {
     static constexpr int side = 8;
     static constexpr int blocks = side * side;
-};
-// Triangles a heavy-tile block may keep for its sample-driven test: 32-texel
-// tiles are always rasterised (k_raster_test), so their shared memory holds
-// only a token list and more blocks fit an SM.
-template <int TS>
-struct HeavyKept {
-    static constexpr int n = TS == 32 ? 32 : kMaxTri;
-    static constexpr int words = n / 32;
 };
 static_assert(kRecvChunk == 64, "receiver prefix sums take two entries per lane of one warp");
 
@@ -1141,15 +1228,6 @@ struct TriSetup {
 };
 static_assert(sizeof(TriSetup) == 17 * 4, "odd word stride");
 
-// A triangle set up for the sample-driven test (48 bytes, three 16-byte loads):
-// edge functions k = 0..2 in tile-local texel coordinates and depths scaled by
-// the inverse doubled area.
-struct TriS {
-    float4 p;  // A0, B0, C0, A1
-    float4 q;  // B1, C1, A2, B2
-    float4 r;  // C2, e0, e1, e2
-};
-
 // q / d for 0 <= q < 2^24 (one float estimate, one correction).
 __device__ __forceinline__ int fdiv(int q, int d, float inv_d)
 {
@@ -1181,33 +1259,11 @@ struct RecvSm {
     int item_pref;             // (row, cell column) items of the receivers staged before this one
 };
 
-// Threads of a k_raster_test block and its register budget (blocks an SM):
-// 32-texel tiles have small shared tiles, and the plants with many heavy
-// 32-texel tiles keep more of them in flight with 128-thread blocks (fewer
-// threads wait at each of a tile's barriers).
-template <int TS>
-struct HeavyCfg {
-    static constexpr int threads = TS == 32 ? 128 : 256;
-    static constexpr int min_blocks = TS == 32 ? 9 : 4;  // 32: 53 registers, 9 x 24 KB shared
-};
-
 template <int TS>
 struct RasterSm {
     uint32_t tile[TS * TS];  // depth keys of the tile
 };
 
-// Kept triangles of a tile for the sample-driven test, up to NT of them.
-template <int TS, int NT, bool SEEN>
-struct KeptSm {
-    TriS tri[NT];
-    uint32_t box[NT];                       // texel box x0 | y0 << 8 | x1 << 16 | y1 << 24
-    float dmin[NT];                         // nearest vertex depth
-    uint2 smask[NT];                        // strict keep: the sub-blocks (bit sb) it may shade a sample of
-    float dlim[SubGrid<TS>::blocks];        // per sub-block: a triangle shades none of its samples
-                                            // unless its nearest depth is below this
-    uint32_t sbm[SubGrid<TS>::blocks][NT / 32];  // per sub-block: triangles that may shade one of its samples
-    uint32_t seen[SEEN ? TS * TS / 32 : 1]; // work counting: texels whose fragments were counted
-};
 static_assert(SubGrid<32>::blocks == 64 && SubGrid<64>::blocks == 64 && SubGrid<128>::blocks == 64,
               "a triangle's sub-block set is one 64-bit mask");
 
@@ -1219,9 +1275,8 @@ struct SubInfo {
 
 template <int TS>
 struct TileSm {
-    union {
+    struct {
         RasterSm<TS> r;
-        KeptSm<TS, HeavyKept<TS>::n, true> s;
     } u;
     float dlim[SubGrid<TS>::blocks]; // per sub-block depth limit (sub_limits)
     SubInfo si;                      // their summary (sub_summary)
@@ -1231,7 +1286,6 @@ struct TileSm {
     int n_recv;                      // receivers staged
     int total_items;                 // (sample row, cell column) items over the staged receivers
     int any_write;                   // some texel of the tile received a depth
-    int n_tri;                       // triangles kept by the sample-driven set-up
     TriSetup tri[kTriBatchMax];      // a batch of set-up triangles, one per thread
     int row_pref[kTriBatchMax + 1];  // prefix of their rows
 };
@@ -1449,13 +1503,6 @@ __device__ __forceinline__ bool tri_box(const TriT& T, int& x0, int& x1, int& y0
     return x0 <= x1 && y0 <= y1;
 }
 
-// ---- sample-driven depth test ----------------------------------------------
-// A tile with few triangles is not rasterised: each of its samples tests the
-// triangles that may cover its texel directly.  The sample is shaded iff some
-// triangle covers its texel centre at a depth it is behind -- the same
-// decision as a depth test against the tile's stored minimum (the comparison
-// is monotone in the stored depth), with the same arithmetic per triangle.
-
 // Summary of a tile's sub-block depth limits, for tri_sub_mask's fast path:
 // the sub-blocks that any receiver meets (limit above -inf) and the smallest
 // limit among them.  Called by one full warp once the limits are written.
@@ -1530,41 +1577,6 @@ __device__ __forceinline__ uint64_t tri_sub_mask(const Edges& ed, int x0, int x1
     return m;
 }
 
-// Set up binned triangle t of tile (ox, oy) for the sample-driven test: false
-// if it lies behind every staged receiver or covers no texel centre of the
-// tile; with `strict`, also if it may shade no sample of any sub-block
-// (tri_sub_mask with the sub-block depth limits dlim), its sub-blocks in
-// smask.  box and dmin feed sub_masks (loose keep).
-template <int TS, bool PROF>
-__device__ __forceinline__ bool setup_tri_s(const JobDev& J, const Buffers& B, const LightParams& lp, int ls, int t,
-                                            float ox, float oy, const RecvSm* recv, int n_recv, bool cull_ok,
-                                            bool strict, const float* dlim, const SubInfo& si, TriS& ts,
-                                            uint32_t& box, float& dmin, uint64_t& smask, unsigned int& culled)
-{
-    TriT T;
-    tri_texel(J, B, lp, ls, t, T);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) { T.x[k] -= ox; T.y[k] -= oy; }
-    if (!may_shade(recv, n_recv, T, cull_ok)) {
-        if (PROF) ++culled;
-        return false;
-    }
-    Edges ed;
-    int x0, x1, y0, y1;
-    if (!make_edges(T, ed) || !tri_box<TS>(T, x0, x1, y0, y1)) return false;
-    dmin = fminf(T.d[0], fminf(T.d[1], T.d[2]));
-    if (strict) {
-        smask = tri_sub_mask<TS>(ed, x0, x1, y0, y1, dmin, dlim, si);
-        if (smask == 0ull) return false;
-    }
-    const float inv_a = 1.f / ed.area2;
-    ts.p = make_float4(ed.A[0], ed.Bc[0], ed.C[0], ed.A[1]);
-    ts.q = make_float4(ed.Bc[1], ed.C[1], ed.A[2], ed.Bc[2]);
-    ts.r = make_float4(ed.C[2], T.d[0] * inv_a, T.d[1] * inv_a, T.d[2] * inv_a);
-    box = (uint32_t)x0 | ((uint32_t)y0 << 8) | ((uint32_t)x1 << 16) | ((uint32_t)y1 << 24);
-    return true;
-}
-
 // Per sub-block, the depth below which a triangle must reach to shade one of
 // its samples: the largest over the receivers whose box meets the sub-block
 // of (receiver plane over the sub-block - bias), plus twice the plane
@@ -1593,215 +1605,6 @@ __device__ __forceinline__ void sub_limits(const RecvSm* recv, int n_recv, float
             lim = fmaxf(lim, pm - R.s.bias + 2.f * R.cull_tol + q1);
         }
         dlim[sb] = lim;
-    }
-}
-
-// Per sub-block of the tile, the kept triangles that may shade one of its
-// samples: nearest depth below the sub-block's limit, box overlap, then each
-// edge at the sub-block's texel centre farthest inside it (exact: edge_at is
-// monotone in px and py, so a covered texel of the sub-block implies a
-// non-negative value there).  Entries q = q_begin, q_begin + q_stride, ... <
-// 64 * words(n) of sbm are written.
-template <int TS, int WORDS>
-__device__ __forceinline__ void sub_masks(const TriS* tri, const uint32_t* boxes, const float* dmin,
-                                          const float* dlim, uint32_t (*sbm)[WORDS], int n, int q_begin, int q_stride)
-{
-    constexpr int kSubSide = SubGrid<TS>::side, kSubBlocks = SubGrid<TS>::blocks;
-    constexpr int SW = TS / kSubSide;  // sub-block side, texels
-    const int nw = (n + 31) >> 5;
-    for (int q = q_begin; q < kSubBlocks * nw; q += q_stride) {
-        const int sb = q & (kSubBlocks - 1), w = q / kSubBlocks;
-        const int sx = (sb % kSubSide) * SW, sy = (sb / kSubSide) * SW;
-        const float fx0 = (float)sx + 0.5f, fx1 = (float)(sx + SW - 1) + 0.5f;
-        const float fy0 = (float)sy + 0.5f, fy1 = (float)(sy + SW - 1) + 0.5f;
-        const float lim = dlim[sb];
-        uint32_t m = 0u;
-        const int kend = min(32, n - w * 32);
-        for (int k = 0; k < kend; ++k) {
-            const int t = w * 32 + k;
-            if (!(dmin[t] < lim)) continue;
-            const uint32_t bx = boxes[t];
-            const int x0 = bx & 255u, y0 = (bx >> 8) & 255u, x1 = (bx >> 16) & 255u, y1 = bx >> 24;
-            if (x0 > sx + SW - 1 || x1 < sx || y0 > sy + SW - 1 || y1 < sy) continue;
-            const float4 p = tri[t].p, qq = tri[t].q, r = tri[t].r;
-            if (edge_at(p.x, p.y, p.z, p.x > 0.f ? fx1 : fx0, p.y > 0.f ? fy1 : fy0) < 0.f) continue;
-            if (edge_at(p.w, qq.x, qq.y, p.w > 0.f ? fx1 : fx0, qq.x > 0.f ? fy1 : fy0) < 0.f) continue;
-            if (edge_at(qq.z, qq.w, r.x, qq.z > 0.f ? fx1 : fx0, qq.w > 0.f ? fy1 : fy0) < 0.f) continue;
-            m |= 1u << k;
-        }
-        sbm[sb][w] = m;
-    }
-}
-
-// Per sub-block of the tile, the kept triangles that may shade one of its
-// samples (bit k of word w: kept triangle 32 w + k), transposed from the
-// triangles' sub-block masks: for a few triangles each lane gathers its two
-// sub-blocks' bits, else one ballot per sub-block.  Words w =
-// w_begin, w_begin + w_stride, ... of the n kept triangles are written; called
-// by whole warps.
-template <int WORDS>
-__device__ __forceinline__ void build_sbm(const uint2* smask, uint32_t (*sbm)[WORDS], int n, int w_begin,
-                                          int w_stride)
-{
-    const int lane = threadIdx.x & 31;
-    const int nw = (n + 31) >> 5;
-    if (n <= 24) {
-        // few triangles: each lane assembles its two sub-blocks' words
-        if (w_begin != 0) return;
-        uint32_t lo = 0u, hi = 0u;
-        for (int t = 0; t < n; ++t) {
-            const uint2 m = smask[t];
-            lo |= ((m.x >> lane) & 1u) << t;
-            hi |= ((m.y >> lane) & 1u) << t;
-        }
-        sbm[lane][0] = lo;
-        sbm[lane + 32][0] = hi;
-        return;
-    }
-    for (int w = w_begin; w < nw; w += w_stride) {
-        const int t = (w << 5) | lane;
-        const uint2 m = t < n ? smask[t] : make_uint2(0u, 0u);
-        uint32_t lo = 0u, hi = 0u;
-#pragma unroll
-        for (int sb = 0; sb < 32; ++sb) {
-            const uint32_t a = __ballot_sync(0xffffffffu, (m.x >> sb) & 1u);
-            const uint32_t b = __ballot_sync(0xffffffffu, (m.y >> sb) & 1u);
-            if (lane == sb) { lo = a; hi = b; }
-        }
-        sbm[lane][w] = lo;
-        sbm[lane + 32][w] = hi;
-    }
-}
-
-// Does kept triangle T cover texel centre (px, py) at a depth that the
-// sample (depth d, bias) is behind?
-__device__ __forceinline__ bool tri_shades(const TriS& T, float px, float py, float d, float bias,
-                                           const LightParams& lp, int u24, bool& covers)
-{
-    const float4 p = T.p, q = T.q, r = T.r;
-    const float w0 = edge_at(p.x, p.y, p.z, px, py);
-    const float w1 = edge_at(p.w, q.x, q.y, px, py);
-    const float w2 = edge_at(q.z, q.w, r.x, px, py);
-    covers = w0 >= 0.f && w1 >= 0.f && w2 >= 0.f;
-    if (!covers) return false;
-    const float depth = depth_at(w0, w1, w2, r.y, r.z, r.w);
-    if (u24) return behind_key(d, bias, depth_store_key(depth, lp, 1), lp.dnear, lp.qscale, 1);
-    return d > __fadd_rn(depth, bias);  // = behind_key(d, bias, okey(depth), ...): okey is invertible
-}
-
-// Depth test of one sample (tile-local texel lx, ly) against the kept
-// triangles of its sub-block; stops at the first that shades it.  With
-// PROF, also counts the fragments a depth map needs at the texel (the kept
-// triangles covering it) once per texel, using the `seen` bitmap.
-template <int TS, int WORDS, bool PROF>
-__device__ __forceinline__ bool sample_test(const TriS* tri, int n_kept, const uint32_t (*sbm)[WORDS], int nw,
-                                            uint32_t* seen, int lx, int ly, float d, float bias,
-                                            const LightParams& lp, int u24, unsigned int& pairs, unsigned int& frags)
-{
-    constexpr int kSubSide = SubGrid<TS>::side;
-    const int sb = (ly / (TS / kSubSide)) * kSubSide + lx / (TS / kSubSide);
-    const float px = texel_centre(lx), py = texel_centre(ly);
-    const uint32_t* ms = sbm[sb];
-    bool shaded = false;
-    for (int w = 0; w < nw && !shaded; ++w) {
-        uint32_t m = ms[w];
-        while (m) {
-            const int t = (w << 5) | (__ffs(m) - 1);
-            m &= m - 1u;
-            bool cov;
-            if (PROF) ++pairs;
-            if (tri_shades(tri[t], px, py, d, bias, lp, u24, cov)) {
-                shaded = true;
-                break;
-            }
-        }
-    }
-    if (PROF) {
-        // the depth map's fragments at this texel: every kept triangle
-        // covering it (before the sub-block depth limits)
-        const uint32_t bit = 1u << (lx & 31);
-        if (!(atomicOr(&seen[(ly * TS + lx) >> 5], bit) & bit)) {
-            for (int t = 0; t < n_kept; ++t) {
-                bool cov;
-                tri_shades(tri[t], px, py, d, bias, lp, u24, cov);
-                frags += cov ? 1u : 0u;
-            }
-        }
-    }
-    return shaded;
-}
-
-// Sub-blocks sx0..sx1 x sy0..sy1 of a tile as a mask (bit sy * 8 + sx).
-__device__ __forceinline__ uint64_t sub_box(int sx0, int sx1, int sy0, int sy1)
-{
-    const uint64_t cols = (uint64_t)((2u << sx1) - (1u << sx0));
-    const uint64_t rows = (0x0101010101010101ull >> (8 * (7 - (sy1 - sy0)))) << (8 * sy0);
-    return rows * cols;  // bytes of rows are 0 or 1: no carries
-}
-
-// Depth-test the samples of staged receivers recv[0, n_recv) (items prefixed
-// in item_pref, total_items in all) that read tile (tx, ty) against the kept
-// triangles: items it_begin, it_begin + it_stride, ... one per thread.  Each
-// item adds its shaded count to its (step, cell) tally with one atomic.  An
-// item is skipped whole when no sub-block of the texel box of its end
-// samples is in cand_sb (the sub-blocks in which some kept triangle may shade
-// a sample; all ones: no skipping) -- exact, since a sample's texel is
-// monotone in its index along the row (sample_texel), so every sample of the
-// item reads a texel of that box.
-template <int TS, int WORDS, bool PROF>
-__device__ __forceinline__ void test_items(const RecvSm* recv, int n_recv, int total_items, const JobDev& J,
-                                           const LightParams& lp, int u24, int tx, int ty, int it_begin,
-                                           int it_stride, const TriS* tri, int n_kept,
-                                           const uint32_t (*sbm)[WORDS], int nw, uint64_t cand_sb, uint32_t* seen,
-                                           uint32_t* tally, int64_t tally0, unsigned long long* bits_row,
-                                           int want_bits,
-                                           unsigned int& cand, unsigned int& samples, unsigned int& pairs,
-                                           unsigned int& frags)
-{
-    constexpr int SH = TS == 128 ? 7 : (TS == 64 ? 6 : 5);
-    constexpr int SWS = SH - 3;  // log2 of the sub-block side (8 x 8 sub-blocks)
-    static_assert(SubGrid<TS>::side == 8, "sub-block index by shifts");
-    const int n = J.n;
-    const float r_max = (float)(J.R - 1);
-    const float inv_n = 1.f / (float)n;
-    for (int it = it_begin; it < total_items; it += it_stride) {
-        int Jr, cu, cv, jj, Ib, Ie;
-        const RecvSm& R = decode_item(recv, n_recv, it, n, inv_n, Jr, cu, cv, jj, Ib, Ie);
-        if (PROF) cand += (unsigned int)max(0, Ie - Ib + 1);
-        if (Ib > Ie) continue;
-        // the receiver's sample frame and the row's base in registers
-        const ModStep s = R.s;
-        const float p_over_n = R.p_over_n;
-        const SampleRow row = sample_row(s, Jr, p_over_n);
-        if (cand_sb != ~0ull) {
-            float dq;
-            int ax, ay, bx, by;
-            sample_texel(s, row, (float)Ib + 0.5f, p_over_n, r_max, ax, ay, dq);
-            sample_texel(s, row, (float)Ie + 0.5f, p_over_n, r_max, bx, by, dq);
-            const int lx0 = max(min(ax, bx) - (tx << SH), 0), lx1 = min(max(ax, bx) - (tx << SH), TS - 1);
-            const int ly0 = max(min(ay, by) - (ty << SH), 0), ly1 = min(max(ay, by) - (ty << SH), TS - 1);
-            if (lx0 > lx1 || ly0 > ly1) continue;
-            if (!(sub_box(lx0 >> SWS, lx1 >> SWS, ly0 >> SWS, ly1 >> SWS) & cand_sb)) continue;
-        }
-        const int i0 = cu * n;
-        uint32_t bits = 0u;  // bit i: sample i of the item's row (within its cell) is shaded
-        float ih = (float)Ib + 0.5f;
-        for (int I = Ib; I <= Ie; ++I, ih += 1.f) {
-            float d;
-            int ix, iy;
-            sample_texel(s, row, ih, p_over_n, r_max, ix, iy, d);
-            if ((ix >> SH) != tx || (iy >> SH) != ty) continue;
-            if (PROF) ++samples;
-            if (sample_test<TS, WORDS, PROF>(tri, n_kept, sbm, nw, seen, ix & (TS - 1), iy & (TS - 1), d, s.bias,
-                                             lp, u24, pairs, frags))
-                bits |= 1u << (I - i0);
-        }
-        if (bits) {
-            const int gcell = R.cell_base + cv * R.cu + cu;
-            tally_add(tally, tally0 + gcell, (uint32_t)__popc(bits));
-            // sample k = jj * n + i of the cell; flags kept for k < 64
-            if (want_bits && jj * n < 64) atomicOr(&bits_row[gcell], (unsigned long long)bits << (jj * n));
-        }
     }
 }
 
@@ -2156,318 +1959,6 @@ __device__ __forceinline__ void tile_receivers(const Buffers& B, const WaveDev* 
 }
 
 // ---------------------------------------------------------------------------
-// k_tile_warp: fused path -- one warp per non-empty tile: the depth test of
-// every sample that reads the tile, sample by sample against the tile's kept
-// triangles; shaded counts go to (step, cell).  A warp takes a tile with at
-// most kWarpRecv receivers, kWarpBins binned (kWarpTri on 32-texel tiles,
-// whose crowded tiles are rasterised anyway: handing them on before the keep
-// loop saves the warp's set-up of triangles it would drop, measured on the
-// tracker plant) and kWarpTri kept triangles; it lists any other tile for
-// k_raster_test.  A tile is a small work item
-// (hundreds of samples, a few triangles): one warp each keeps many tiles in
-// flight per SM, which hides the chain of dependent loads that starts a tile.
-// ---------------------------------------------------------------------------
-constexpr int kWarpTri = 64;
-constexpr int kWarpWords = kWarpTri / 32;
-constexpr int kWarpRecv = 16;
-constexpr int kWarpBins = 512;
-constexpr int kTileWarps = 4;   // warps per block; 6 blocks per SM (80 registers a thread)
-
-template <int TS, bool PROF>
-struct WarpSm {
-    KeptSm<TS, kWarpTri, PROF> k;
-    RecvSm recv[kWarpRecv];
-};
-
-template <int TS, bool PROF>
-__global__ void __launch_bounds__(kTileWarps * 32, 6) k_tile_warp(const WaveDev* __restrict__ W,
-                                                                  const JobDev* __restrict__ jobs, Buffers B)
-{
-    __shared__ __align__(16) WarpSm<TS, PROF> sm_all[kTileWarps];
-    unsigned int p_samples = 0, p_writes = 0, p_culled = 0, p_cand = 0, p_tiles = 0, p_stiles = 0, p_pairs = 0;
-    unsigned int p_hr = 0, p_hb = 0, p_ht = 0;
-    const int lane = threadIdx.x & 31;
-    WarpSm<TS, PROF>& sm = sm_all[threadIdx.x >> 5];
-    // the bins are incomplete when the pool overflowed: the wave is rerun
-    // with a larger pool, so nothing here may read them
-    const unsigned int n_ne = (B.ctr->overflow & 1u) ? 0u : B.ctr->n_nonempty;
-    const int nj = W->n_jobs;
-    const int want_bits = W->want_bits;
-    const int u24 = W->depth_u24;
-    const uint64_t bin_cap = (uint64_t)W->bin_cap;
-    unsigned int next = 0;
-    if (lane == 0) next = atomicAdd(&B.ctr->raster_next, 1u);
-    next = __shfl_sync(0xffffffffu, next, 0);
-    while (next < n_ne) {
-        const unsigned int item = next;
-        if (lane == 0) next = atomicAdd(&B.ctr->raster_next, 1u);  // claim the following tile now
-        const uint32_t te = B.nonempty[item];
-        int j, ls, tx, ty;
-        decode_tile(jobs, nj, te, j, ls, tx, ty);
-        const JobDev& J = jobs[j];
-        uint64_t r0;
-        int nrecv;
-        tile_receivers(B, W, te, r0, nrecv);
-        const uint64_t off = B.t_off[te];
-        uint64_t cnt = B.t_cnt[te];
-        if (off + cnt > bin_cap) cnt = off < bin_cap ? bin_cap - off : 0;
-        bool heavy = nrecv > kWarpRecv || cnt > (uint64_t)(TS == 32 ? kWarpTri : kWarpBins);
-        if (PROF && lane == 0) {
-            if (nrecv > kWarpRecv) ++p_hr;
-            else if (heavy) ++p_hb;
-        }
-        if (!heavy) {
-            const LightParams& lp = B.lp[J.js_base + ls];
-            if (lane < nrecv) stage_one<TS>(sm.recv[lane], J, B, ls, tx, ty, (int)B.recv[r0 + lane]);
-            if (PROF)
-                for (int q = lane; q < TS * TS / 32; q += 32) sm.k.seen[q] = 0u;
-            __syncwarp();
-            const int c = lane < nrecv ? sm.recv[lane].item_pref : 0;
-            const int inc = warp_incl_scan(c);
-            const int total = __shfl_sync(0xffffffffu, inc, 31);
-            if (lane < nrecv) sm.recv[lane].item_pref = inc - c;
-            sub_limits<TS>(sm.recv, nrecv, sm.k.dlim, u24 ? 1.f / lp.qscale : 0.f, lane, 32);
-            __syncwarp();
-            const float ox = (float)(tx * TS), oy = (float)(ty * TS);
-            // strict keep (only the triangles that may shade a sample of some
-            // sub-block, tri_sub_mask: fewer kept, tighter sub-block masks,
-            // more set-up per triangle) on 32-texel tiles, whose samples are
-            // dense over few texels, and on crowded tiles; otherwise the loose
-            // keep (in front of some receiver's plane, covering a texel centre
-            // of the tile), cheaper for the few large triangles of a 64- or
-            // 128-texel tile (measured on the tracker plant and the facade)
-            const bool strict = TS == 32 || cnt > (uint64_t)kWarpTri;
-            SubInfo si{};
-            if (strict) si = sub_summary(sm.k.dlim);
-            int n = 0;
-            for (uint64_t b0 = 0; b0 < cnt && n <= kWarpTri; b0 += 32) {
-                TriS ts;
-                uint32_t box = 0u;
-                float dmin = 0.f;
-                uint64_t smask = 0ull;
-                const bool keep = b0 + lane < cnt &&
-                                  setup_tri_s<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.recv,
-                                                        nrecv, true, strict, sm.k.dlim, si, ts, box, dmin, smask,
-                                                        p_culled);
-                const unsigned int bal = __ballot_sync(0xffffffffu, keep);
-                const int slot = n + __popc(bal & ((1u << lane) - 1u));
-                if (keep && slot < kWarpTri) {
-                    sm.k.tri[slot] = ts;
-                    sm.k.box[slot] = box;
-                    sm.k.dmin[slot] = dmin;
-                    sm.k.smask[slot] = make_uint2((uint32_t)smask, (uint32_t)(smask >> 32));
-                }
-                n += __popc(bal);
-            }
-            heavy = n > kWarpTri;
-            if (PROF && lane == 0 && heavy) ++p_ht;
-            if (!heavy && n > 0) {
-                __syncwarp();
-                if (strict) build_sbm<kWarpWords>(sm.k.smask, sm.k.sbm, n, 0, 1);
-                else sub_masks<TS, kWarpWords>(sm.k.tri, sm.k.box, sm.k.dmin, sm.k.dlim, sm.k.sbm, n, lane, 32);
-                __syncwarp();
-                const int C = J.n_cells;
-                // sub-blocks in which some kept triangle may shade a sample
-                uint32_t a0 = 0u, a1 = 0u;
-                for (int w = 0; w < ((n + 31) >> 5); ++w) {
-                    a0 |= sm.k.sbm[lane][w];
-                    a1 |= sm.k.sbm[lane + 32][w];
-                }
-                const uint64_t cand_sb = (uint64_t)__ballot_sync(0xffffffffu, a0 != 0u) |
-                                         ((uint64_t)__ballot_sync(0xffffffffu, a1 != 0u) << 32);
-                test_items<TS, kWarpWords, PROF>(sm.recv, nrecv, total, J, lp, u24, tx, ty, lane, 32, sm.k.tri, n,
-                                                 sm.k.sbm, (n + 31) >> 5, cand_sb, sm.k.seen,
-                                                 B.cs_cnt, J.cs_base + (int64_t)ls * C,
-                                                 B.cs_bits + J.cs_base + (int64_t)ls * C, want_bits, p_cand,
-                                                 p_samples, p_pairs, p_writes);
-            }
-            if (PROF && lane == 0 && !heavy) { ++p_tiles; ++p_stiles; }
-        }
-        if (heavy && lane == 0) {
-            const unsigned int pos = atomicAdd(&B.ctr->n_heavy, 1u);
-            if (pos < (uint64_t)W->tot_te) B.heavy[pos] = te;
-        }
-        __syncwarp();  // the warp's shared memory may be reused
-        next = __shfl_sync(0xffffffffu, next, 0);
-    }
-    if (PROF) {
-        flush_profile(B, p_samples, 0u, p_writes, p_culled);
-        flush_profile2(B, p_cand, p_tiles, 0u, p_stiles, p_pairs);
-#pragma unroll
-        for (int off = 16; off; off >>= 1) {
-            p_hr += __shfl_xor_sync(0xffffffffu, p_hr, off);
-            p_hb += __shfl_xor_sync(0xffffffffu, p_hb, off);
-            p_ht += __shfl_xor_sync(0xffffffffu, p_ht, off);
-        }
-        if (lane == 0) {
-            atomicAdd(&B.ctr->prof_heavy_why[0], (unsigned long long)p_hr);
-            atomicAdd(&B.ctr->prof_heavy_why[1], (unsigned long long)p_hb);
-            atomicAdd(&B.ctr->prof_heavy_why[2], (unsigned long long)p_ht);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// k_raster_test: fused path, the tiles k_tile_warp listed (more receivers,
-// binned or kept triangles than a warp takes) -- one CTA per tile.  On 64-
-// and 128-texel tiles the binned triangles are first set up by the whole
-// block, keeping those that may shade a sample of some sub-block
-// (tri_sub_mask); with at most kMaxTri kept, every sample is tested against
-// the kept triangles of its sub-block (few large triangles over sparse
-// samples: most samples stop at their first occluder).  Otherwise, and always
-// on 32-texel tiles, the tile is rasterised in shared memory (tile_raster:
-// texel-centre coverage, atomicMin of order-preserving depth keys, only at
-// the texels samples read and only where a triangle may shade) and the
-// samples read it (many small triangles -- lattice members, grazing terrain
-// -- each drawn once instead of tested by every sample near it; measured
-// faster on the tracker plant for every kept count).  Both give the same
-// decisions.
-// ---------------------------------------------------------------------------
-
-// Set up the tile's binned triangles that may shade a sample of a staged
-// receiver (strict keep), for the whole block; the sub-block depth limits
-// must be ready (tile_limits).  Returns how many were kept, or -1 if more than
-// kMaxTri were.
-template <int TS, bool PROF>
-__device__ int setup_sample_tris(TileSm<TS>& sm, const JobDev& J, const Buffers& B, const WaveDev* W,
-                                 const LightParams& lp, int ls, int tx, int ty, int64_t te, bool cull_ok,
-                                 unsigned int& culled)
-{
-    const int tid = threadIdx.x, lane = tid & 31;
-    const float ox = (float)(tx * TS), oy = (float)(ty * TS);
-    const uint64_t off = B.t_off[te];
-    uint64_t cnt = B.t_cnt[te];
-    const uint64_t cap = (uint64_t)W->bin_cap;
-    if (off + cnt > cap) cnt = off < cap ? cap - off : 0;
-    if (PROF)
-        for (int q = tid; q < TS * TS / 32; q += blockDim.x) sm.u.s.seen[q] = 0u;
-    if (tid == 0) sm.n_tri = 0;
-    __syncthreads();
-    const SubInfo si = sm.si;
-    for (uint64_t b0 = 0; b0 < cnt; b0 += blockDim.x) {
-        TriS ts;
-        uint32_t box = 0u;
-        float dmin = 0.f;
-        uint64_t smask = 0ull;
-        const bool keep = b0 + tid < cnt &&
-                          setup_tri_s<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + tid], ox, oy, sm.recv,
-                                                sm.n_recv, cull_ok, true, sm.dlim, si, ts, box, dmin, smask, culled);
-        const unsigned int bal = __ballot_sync(0xffffffffu, keep);
-        int base = 0;
-        if (lane == 0 && bal) base = atomicAdd(&sm.n_tri, __popc(bal));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (keep) {
-            const int slot = base + __popc(bal & ((1u << lane) - 1u));
-            if (slot < HeavyKept<TS>::n) {
-                sm.u.s.tri[slot] = ts;
-                sm.u.s.smask[slot] = make_uint2((uint32_t)smask, (uint32_t)(smask >> 32));
-            }
-        }
-    }
-    __syncthreads();
-    const int n = sm.n_tri;
-    return n > HeavyKept<TS>::n ? -1 : n;
-}
-
-template <int TS, bool PROF>
-__global__ void __launch_bounds__(HeavyCfg<TS>::threads, HeavyCfg<TS>::min_blocks)
-    k_raster_test(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs, Buffers B)
-{
-    extern __shared__ __align__(16) unsigned char tile_smem[];  // sizeof(TileSm<TS>), set at launch
-    TileSm<TS>& sm = *reinterpret_cast<TileSm<TS>*>(tile_smem);
-    unsigned int p_samples = 0, p_visits = 0, p_writes = 0, p_culled = 0, p_cand = 0, p_dense = 0, p_tiles = 0;
-    unsigned int p_stiles = 0, p_pairs = 0;
-    __shared__ unsigned int s_item[2];
-    // incomplete bins (pool overflow, the wave is rerun): nothing to read
-    const unsigned int n_ne = (B.ctr->overflow & 1u) ? 0u : min(B.ctr->n_heavy, (unsigned int)W->tot_te);
-    const int nj = W->n_jobs;
-    const int u24 = W->depth_u24;
-    const int want_bits = W->want_bits;
-    const int tid = threadIdx.x;
-    if (tid == 0) s_item[0] = atomicAdd(&B.ctr->heavy_next, 1u);
-    __syncthreads();
-    for (int par = 0;; par ^= 1) {
-        // the next tile is claimed while this one runs; the barriers inside
-        // the tile publish it
-        const unsigned int item = s_item[par];
-        if (item >= n_ne) break;
-        if (tid == 0) s_item[par ^ 1] = atomicAdd(&B.ctr->heavy_next, 1u);
-        const uint32_t te = B.heavy[item];
-        int j, ls, tx, ty;
-        decode_tile(jobs, nj, te, j, ls, tx, ty);
-        const JobDev& J = jobs[j];
-        uint64_t r0;
-        int nrecv;
-        tile_receivers(B, W, te, r0, nrecv);
-        stage_receivers<TS>(sm, J, B, ls, tx, ty, r0, min(nrecv, kRecvChunk));
-        if (PROF && tid == 0) ++p_tiles;
-        const LightParams& lp = B.lp[J.js_base + ls];
-        const int C = J.n_cells;
-        const int64_t tally0 = J.cs_base + (int64_t)ls * C;
-        unsigned long long* bits_row = B.cs_bits + J.cs_base + (int64_t)ls * C;
-        const bool cull_ok = nrecv <= kRecvChunk;
-        tile_limits<TS>(sm, lp, u24, cull_ok);
-        // 32-texel tiles are always rasterised (dense samples over few
-        // texels: each kept triangle drawn once beats every sample testing
-        // it); larger tiles take the sample-driven test when at most kMaxTri
-        // triangles are kept (few large triangles over sparse samples)
-        const int nt = TS == 32 ? -1
-                                : setup_sample_tris<TS, PROF>(sm, J, B, W, lp, ls, tx, ty, te, cull_ok, p_culled);
-        const bool sample_driven = nt >= 0;
-        if (sample_driven) {
-            // sample-driven test (no triangle kept: every sample of the tile is lit)
-            if (PROF && tid == 0) ++p_stiles;
-            if (nt > 0) build_sbm<HeavyKept<TS>::words>(sm.u.s.smask, sm.u.s.sbm, nt, tid >> 5, blockDim.x >> 5);
-            __syncthreads();
-            for (int c0 = 0; nt > 0 && c0 < nrecv; c0 += kRecvChunk) {
-                if (c0 > 0) {
-                    __syncthreads();
-                    stage_receivers<TS>(sm, J, B, ls, tx, ty, r0 + c0, min(kRecvChunk, nrecv - c0));
-                }
-                test_items<TS, HeavyKept<TS>::words, PROF>(sm.recv, sm.n_recv, sm.total_items, J, lp, u24, tx, ty, tid,
-                                                blockDim.x, sm.u.s.tri, nt, sm.u.s.sbm, (nt + 31) >> 5, ~0ull,
-                                                sm.u.s.seen, B.cs_cnt, tally0, bits_row, want_bits, p_cand, p_samples,
-                                                p_pairs, p_writes);
-            }
-        } else if (tile_raster<TS, PROF>(sm, J, B, W, ls, tx, ty, te, r0, nrecv, true, p_visits, p_writes, p_culled,
-                                         p_cand, p_dense) != 0) {
-            for (int c0 = 0; c0 < nrecv; c0 += kRecvChunk) {
-                if (c0 > 0) stage_receivers<TS>(sm, J, B, ls, tx, ty, r0 + c0, min(kRecvChunk, nrecv - c0));
-                uint32_t cnt = 0;
-                unsigned long long bits = 0ull;
-                for_tile_samples<TS, PROF>(
-                    sm.recv, sm.n_recv, sm.total_items, J, tx, ty, tid, blockDim.x, p_cand,
-                    [&](const RecvSm& R, int k, int ix, int iy, float d) {
-                        if (PROF) ++p_samples;
-                        const uint32_t key = sm.u.r.tile[(iy & (TS - 1)) * TS + (ix & (TS - 1))];
-                        if (key == kEmpty) return;
-                        if (behind_key(d, R.s.bias, key, lp.dnear, lp.qscale, u24)) {
-                            ++cnt;
-                            if (k < 64) bits |= 1ull << k;
-                        }
-                    },
-                    [&](const RecvSm& R, int cu, int cv) {
-                        if (cnt) {
-                            const int gcell = R.cell_base + cv * R.cu + cu;
-                            tally_add(B.cs_cnt, tally0 + gcell, cnt);
-                            if (want_bits) atomicOr(&bits_row[gcell], bits);
-                        }
-                        cnt = 0;
-                        bits = 0ull;
-                    });
-                __syncthreads();
-            }
-        }
-        __syncthreads();  // the tile's shared memory may be reused
-    }
-    if (PROF) {
-        flush_profile(B, p_samples, p_visits, p_writes, p_culled);
-        flush_profile2(B, p_cand, p_tiles, p_dense, p_stiles, p_pairs);
-        flush_heavy(B, p_samples, p_writes, p_tiles);
-    }
-}
-
-// ---------------------------------------------------------------------------
 // k_raster_map: map path -- rasterise the tile and store it in HBM for the
 // gather kernel (coalesced 16-byte stores)
 // ---------------------------------------------------------------------------
@@ -2507,6 +1998,911 @@ __global__ void __launch_bounds__(256) k_raster_map(const WaveDev* __restrict__ 
         __syncthreads();
     }
     if (PROF) flush_profile(B, 0u, p_visits, p_writes, p_culled);
+}
+
+// ---------------------------------------------------------------------------
+// fused path: coverage of a tile's texels, and the samples that look it up
+//
+// A sample is shaded iff some triangle covers its texel's centre at a depth
+// that the sample, less its bias, is behind.  The samples of the modules of
+// one plane (a tracker's table, a facade) lie on that plane, so at a texel a
+// triangle is in front of all of them, behind all of them, or in a thin band
+// about the plane (the plane's slope over the texel and rounding) where each
+// sample must compare depths.  A tile therefore keeps one bit per texel and
+// plane: covered by something in front of the plane.  Triangles wholly in
+// front of a plane set whole row spans, those wholly behind are dropped, and
+// only those that cross the plane's band in the tile compare depths, texel by
+// texel; texels in the band are "open", and the few samples that read them
+// test the triangles there one by one (or the tile's nearest depth).  The
+// decisions are those of a depth map, sample by sample.
+//
+// The kernels of this path are bound by instruction issue and fetch (a tile
+// runs a few thousand instructions of straight-line code, and the warps of an
+// SM are all at different places in it), so the code is kept small: one copy
+// of each loop, none unrolled that is not short and hot.
+// ---------------------------------------------------------------------------
+
+// Planes of a tile with bits of their own; further ones share the last.
+template <int TS>
+struct Levels {
+    static constexpr int n = TS == 32 ? 12 : (TS == 64 ? 8 : 4);
+};
+
+// Of these, the ones a warp of k_tile_warp keeps (k_raster_test keeps all): the
+// less shared memory a warp takes, the more of them an SM holds.
+template <int TS>
+struct WarpLevels {
+    static constexpr int n = TS == 32 ? 12 : (TS == 64 ? 8 : 1);
+};
+
+template <int TS>
+struct TileSh {  // log2 of the tile side
+    static constexpr int v = TS == 128 ? 7 : (TS == 64 ? 6 : 5);
+};
+
+// A plane of the tile's receivers: depth d = pa x + pb y + pc at tile-local
+// texel coordinates.  A triangle's depth at a texel centre less the plane's is
+// below -front: it shades every sample of the plane that reads the texel; not
+// below back: none.  front = inf, back = inf where no such bound is known (the
+// sun within a degree of the plane, planes that share a level): every texel
+// that a triangle covers is open.
+struct Level {
+    float pa, pb, pc;
+    float front, back;
+    float cull;  // a triangle nowhere nearer than the plane by more shades no sample of it; -1: no such bound
+    int plane;  // plane group, or -1: any group without a level of its own
+};
+
+// What tile entry t_cnt holds once the tile kernels are done: kTileLit, a
+// tile that shades every sample of every receiver, or 1 + the 16-byte offset
+// of the tile's record in the pool B.cov:
+//   word 0      levels | kRecOpen | kRecDepth | kRecHeavy | open triangles << 16
+//   words 1-12  plane group of each level
+//   words 13-24 box of each level's covered and open texels, x0 | x1 << 8 | y0
+//               << 16 | y1 << 24 (kBoxNone: none)
+//   word 28 ... TS * TS / 32 words of coverage bits per level (bit x & 31 of
+//               word y * TS / 32 + x / 32)
+// and, with kRecOpen, as many words of open texels, then the open triangles
+// (TriS, 12 words each) or, with kRecDepth, TS * TS depth keys.
+constexpr uint32_t kTileLit = 0u;
+constexpr uint32_t kTileFull = 0xFFFFFFFFu, kTileFullHeavy = 0xFFFFFFFEu;  // (heavy: k_raster_test's, for the counters)
+constexpr uint32_t kRecLevels = 0xFFu, kRecOpen = 1u << 8, kRecDepth = 1u << 9, kRecHeavy = 1u << 10;
+constexpr int kRecHead = 28, kRecBox = 13;
+constexpr uint32_t kBoxNone = 0x000000FFu;
+static_assert(Levels<32>::n <= 12 && Levels<64>::n <= 12 && Levels<128>::n <= 12, "record header");
+
+// A triangle set up for the sample-driven test (48 bytes, three 16-byte loads):
+// edge functions k = 0..2 in tile-local texel coordinates and depths scaled by
+// the inverse doubled area.
+struct TriS {
+    float4 p;  // A0, B0, C0, A1
+    float4 q;  // B1, C1, A2, B2
+    float4 r;  // C2, e0, e1, e2
+};
+
+// Does triangle T cover texel centre (px, py) at a depth that the sample
+// (depth d, bias) is behind?
+__device__ __forceinline__ bool tri_shades(const TriS& T, float px, float py, float d, float bias,
+                                           const LightParams& lp, int u24)
+{
+    const float4 p = T.p, q = T.q, r = T.r;
+    const float w0 = edge_at(p.x, p.y, p.z, px, py);
+    const float w1 = edge_at(p.w, q.x, q.y, px, py);
+    const float w2 = edge_at(q.z, q.w, r.x, px, py);
+    if (!(w0 >= 0.f && w1 >= 0.f && w2 >= 0.f)) return false;
+    const float depth = depth_at(w0, w1, w2, r.y, r.z, r.w);
+    if (u24) return behind_key(d, bias, depth_store_key(depth, lp, 1), lp.dnear, lp.qscale, 1);
+    return d > __fadd_rn(depth, bias);  // = behind_key(d, bias, okey(depth), ...): okey is invertible
+}
+
+// A triangle set up for drawing: edge functions, depths scaled by the inverse
+// doubled area, its texel box, the levels it is in front of and those it is
+// to be compared with texel by texel (bit l of front, deep).  21 words: lanes
+// reading different triangles' fields hit different banks.
+struct TriDraw {
+    float A[3], Bc[3], C[3];
+    float inv[3];        // -1 / A, about (infinite for A = 0)
+    float e[3];
+    short x0, x1;
+    int y0;
+    float err;           // bound on the rounding of its depths
+    uint32_t front, deep;
+    int rows;
+};
+static_assert(sizeof(TriDraw) == 21 * 4, "odd word stride");
+
+// Triangles being drawn by a warp, one per lane, and the inclusive prefix of
+// their rows.
+struct DrawSm {
+    TriDraw tri[32];
+    int pref[32];
+    uint32_t open;  // triangles that left a texel open
+};
+
+// Level of module m (ModStep s) in tile (tx, ty).
+template <int TS>
+__device__ __forceinline__ void fill_level(Level& L, const ModStep& s, int plane, int tx, int ty, float cull)
+{
+    L.pa = s.pa;
+    L.pb = s.pb;
+    L.pc = s.d0 - s.pa * (s.tx0 - (float)(tx * TS)) - s.pb * (s.ty0 - (float)(ty * TS));
+    L.front = s.hs + s.bias;
+    L.back = s.hs - s.bias;
+    // (less than half of the bias that is no slope: what lies in the plane or
+    // behind it, which at a low sun rounding alone may bring past the bias)
+    L.cull = s.cosi > 0.017452406f && s.hs < FLT_MAX ? cull : -1.f;
+    L.plane = plane;
+}
+
+// Put nl levels in order, front to back; true if each is in front of the next
+// all over the tile (planes that do not cross in it, such as parallel tables):
+// what is in front of one level is then in front of all after it.
+template <int TS>
+__device__ __forceinline__ bool order_levels(Level* lv, int nl)
+{
+    const int lane = threadIdx.x & 31;
+    const Level L = lv[min(lane, nl - 1)];
+    // levels without a plane last, in their order: the shared level stays the last
+    const float key = L.front < FLT_MAX ? L.pc + (L.pa + L.pb) * (0.5f * TS) - L.front : INFINITY;
+    int rank = 0;
+#pragma unroll 1
+    for (int q = 0; q < nl; ++q) {
+        const float o = __shfl_sync(0xffffffffu, key, q);
+        rank += o < key || (o == key && q < lane) ? 1 : 0;
+    }
+    __syncwarp();
+    if (lane < nl) lv[rank] = L;
+    __syncwarp();
+    bool ok = true;
+    if (lane < nl) {
+        const Level& a = lv[max(lane - 1, 0)];
+        const Level& b = lv[lane];
+        const float d = (b.pc - b.front) - (a.pc - a.front), x = (b.pa - a.pa) * TS, y = (b.pb - a.pb) * TS;
+        ok = b.front < FLT_MAX && d + fminf(x, 0.f) + fminf(y, 0.f) >= 0.f;
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+
+// The levels of tile te, for one full warp; returns their number, and whether
+// they are nested (order_levels).  A tile of one plane group takes the plane
+// from any of its modules (t_roff), others go through the receiver list.
+template <int TS>
+__device__ __forceinline__ int build_levels(Level* lv, const JobDev& J, const Buffers& B, const WaveDev* W, uint32_t te,
+                                            int ls, int tx, int ty, uint32_t plane, bool& nested)
+{
+    nested = false;
+    const int lane = threadIdx.x & 31;
+    const ModStep* ms = B.ms + J.ms_base + (int64_t)ls * J.n_mods;
+    const uint32_t r0 = B.t_roff[te];
+    const float cull = B.t_rcnt[te] <= (uint32_t)kRecvChunk ? B.lp[J.js_base + ls].delta * (1.f / 64.f) : -1.f;
+    if (plane != kPlaneMixed) {
+        if (lane == 0) fill_level<TS>(lv[0], ms[r0], (int)plane, tx, ty, cull);
+        __syncwarp();
+        return 1;
+    }
+    uint32_t r1 = r0 + B.t_rcnt[te];
+    if (r1 > (uint64_t)W->recv_cap) r1 = (uint32_t)W->recv_cap;
+    int nl = 0;
+#pragma unroll 1
+    for (uint32_t r = r0; r < r1; r += 32) {
+        const bool have = r + lane < r1;
+        const int m = have ? (int)B.recv[r + lane] : 0;
+        const int pl = have ? J.mods[m].plane : -1;
+        bool known = !have;
+        for (int q = 0; q < nl; ++q) known = known || lv[q].plane == pl;
+        unsigned int todo = __ballot_sync(0xffffffffu, !known);
+#pragma unroll 1
+        while (todo) {
+            const int lead = __ffs((int)todo) - 1;
+            const int p = __shfl_sync(0xffffffffu, pl, lead);
+            todo &= ~__ballot_sync(0xffffffffu, have && pl == p);
+            if (lane == lead) {
+                if (nl < Levels<TS>::n) {
+                    fill_level<TS>(lv[nl], ms[m], pl, tx, ty, cull);
+                } else {
+                    Level& L = lv[Levels<TS>::n - 1];
+                    L.pa = L.pb = L.pc = 0.f;
+                    L.front = L.back = INFINITY;
+                    L.cull = -1.f;
+                    L.plane = -1;
+                }
+            }
+            if (nl < Levels<TS>::n) ++nl;
+            __syncwarp();
+        }
+    }
+    if (nl > 1) nested = order_levels<TS>(lv, nl);
+    return nl;
+}
+
+// A binned triangle over the tile: its texel-space vertices (tile-local,
+// counter-clockwise), edges and texel box, and what it is to the tile's
+// levels.
+struct TriWork {
+    TriT T;
+    Edges ed;
+    int x0, x1, y0, y1;
+    float err;             // bound on the rounding of its depths
+    uint32_t front, deep;  // bit l: in front of level l; to be compared with it texel by texel
+    bool whole;            // covers every texel centre of the tile
+};
+
+// Set up binned triangle t of tile (ox, oy); front = deep = 0 if it covers no
+// texel centre of the tile or is behind every level, or lies in or behind the
+// planes of all.
+//
+// The triangle's depth less a plane's is linear, so over the tile it lies
+// between its values at the vertices, up to what rounding makes of the depth
+// at a texel (depth_at): the mean of the vertex depths d_k weighted by the
+// edge functions w_k >= 0 as computed, over the doubled area as computed, is
+// off by at most |d| (|sum w_k / area - 1| + 6 u), u = 2^-24.  Each w_k is off
+// its exact value by at most 5 u (|A_k| (|px| + |x_a|) + |B_k| (|py| + |y_a|))
+// (the rounding of A, B, C and of the two multiply-adds; x_a, y_a the vertex C
+// was taken at, |px|, |py| <= TS) and the area by 3 u of the same sum S over
+// the three edges: |sum w_k / area - 1| <= 8 u S / area = 4.8e-7 S / area.
+// Twice that is allowed for, and 1e-5 of the plane's terms at the vertices.
+template <int TS, bool PROF>
+__device__ __forceinline__ void classify_tri(const JobDev& J, const Buffers& B, const LightParams& lp, int ls, int t,
+                                             float ox, float oy, const Level* lv, int nl, TriWork& w,
+                                             unsigned int& culled)
+{
+    tri_texel(J, B, lp, ls, t, w.T);
+    TriT& T = w.T;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { T.x[k] -= ox; T.y[k] -= oy; }
+    if (!make_edges(T, w.ed) || !tri_box<TS>(T, w.x0, w.x1, w.y0, w.y1)) return;
+    const Edges& e = w.ed;
+    const float xm = fmaxf(fabsf(T.x[0]), fmaxf(fabsf(T.x[1]), fabsf(T.x[2]))) + (float)TS;
+    const float ym = fmaxf(fabsf(T.y[0]), fmaxf(fabsf(T.y[1]), fabsf(T.y[2]))) + (float)TS;
+    const float S = (fabsf(e.A[0]) + fabsf(e.A[1]) + fabsf(e.A[2])) * xm +
+                    (fabsf(e.Bc[0]) + fabsf(e.Bc[1]) + fabsf(e.Bc[2])) * ym;
+    const float dabs = fmaxf(fabsf(T.d[0]), fmaxf(fabsf(T.d[1]), fabsf(T.d[2])));
+    const float err = dabs * (1e-6f * __fdividef(S, e.area2) + 1e-6f);
+    w.err = err;
+    bool keep = false;
+#pragma unroll 1
+    for (int l = 0; l < nl; ++l) {
+        const float pa = lv[l].pa, pb = lv[l].pb, pc = lv[l].pc;
+        float lo = FLT_MAX, hi = -FLT_MAX;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float g = T.d[k] - (pa * T.x[k] + pb * T.y[k] + pc);
+            lo = fminf(lo, g);
+            hi = fmaxf(hi, g);
+        }
+        const float tol = err + 1e-5f * (fabsf(pa) * xm + fabsf(pb) * ym);
+        keep = keep || lv[l].cull < 0.f || !(lo >= -lv[l].cull);
+        if (hi + tol < -lv[l].front) w.front |= 1u << l;
+        else if (!(lo - tol >= lv[l].back)) w.deep |= 1u << l;
+    }
+    if (!keep) w.deep = 0u;  // (front none)
+    if (PROF && !(w.front | w.deep)) ++culled;
+    // each edge at the texel centre farthest outside it (edge_at is monotone
+    // in px and py)
+    if (w.x0 == 0 && w.y0 == 0 && w.x1 == TS - 1 && w.y1 == TS - 1) {
+        w.whole = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            w.whole = w.whole && edge_at(e.A[k], e.Bc[k], e.C[k], e.A[k] > 0.f ? 0.5f : TS - 0.5f,
+                                         e.Bc[k] > 0.f ? 0.5f : TS - 0.5f) >= 0.f;
+    }
+}
+
+// Narrow the texel range [lo, hi] (whole numbers, or empty: lo = hi + 1) of a
+// row to the texels whose centre px has fma(A, px, t) >= 0 -- edge_at on that
+// row, which is monotone in px, so the texels form an interval that ends at
+// one end of the range (the high one for A >= 0).  Its other end is found from
+// the edge's root t inv, inv = -1/A about.  The sign of fma is that of A px + t exactly, and
+// within the range (at most 128 texels) the root's estimate is off by far less
+// than one texel, so one step either way corrects it.  A = 0 (or so small that
+// the root overflows): the estimate is infinite, beyond the range on the side
+// where the sign of t puts the interval's end; t = 0 then makes it NaN, which
+// the clamp takes to the low end (A >= 0: every texel; A < 0: none).
+__device__ __forceinline__ void row_edge(float A, float inv, float t, float& lo, float& hi)
+{
+    const float s = A >= 0.f ? 1.f : -1.f;
+    const float begin = A >= 0.f ? lo : hi, end = (A >= 0.f ? hi : lo) + s;
+    const float r = __fmaf_rn(t, inv, -0.5f);
+    float i = fminf(fmaxf(A >= 0.f ? ceilf(r) : floorf(r), fminf(begin, end)), fmaxf(begin, end));
+    if (i != begin && __fmaf_rn(A, i - s + 0.5f, t) >= 0.f) i -= s;
+    if (i != end && __fmaf_rn(A, i + 0.5f, t) < 0.f) i += s;
+    if (A >= 0.f) lo = i;
+    else hi = i;
+}
+
+// Narrow the texels [lo, hi] to those where a value that is linear along them,
+// from ga at lo to gb at hi, is below T: with margin < 0 to fewer (each of them
+// is), with margin > 0 to more (no other is), by that part of a texel, which is
+// far above what the root's estimate is off by.  False if none is.  A NaN (an
+// infinite bound) leaves none and all.
+__device__ __forceinline__ bool below(float ga, float gb, float T, float margin, float& lo, float& hi)
+{
+    const bool in_a = margin > 0.f ? !(ga >= T) : ga < T, in_b = margin > 0.f ? !(gb >= T) : gb < T;
+    if (in_a != in_b) {
+        const float x = __fmaf_rn(__fdividef(T - ga, gb - ga), hi - lo, lo);
+        if (margin > 0.f) {
+            if (in_a) hi = fminf(hi, ceilf(x + margin));
+            else lo = fmaxf(lo, floorf(x - margin));
+        } else {
+            if (in_a) hi = fmaxf(lo - 1.f, floorf(x + margin));
+            else lo = fminf(hi + 1.f, ceilf(x - margin));
+        }
+    }
+    return (in_a || in_b) && lo <= hi;
+}
+
+// A triangle's rows are one lane each.  On 64- and 128-texel tiles a triangle
+// has rows enough for the warp, so its rows are drawn together: its set-up is
+// read by all lanes at once, and a warp that has the tile to itself
+// (k_tile_warp) updates a row's words with one vector load and store in place
+// of atomics.  On 32-texel tiles most have five to ten rows and several
+// triangles share the warp.  (128 texels, the facade year: 4.7 -> 3.9 ms for
+// k_tile_warp; 64 texels, 45 suns over 13 modules: 68 -> 53 us.)
+//
+// Draw the warp's triangles (w, one per lane; `full`: the levels covered
+// everywhere, neither drawn nor compared any more): row spans into the coverage bits of the levels they are in
+// front of (cov, TS * TS / 32 words each; nested levels: of the first of them
+// only, finish_words adds the bits to the levels after it), and for the levels
+// they cross, each texel compared with the plane: in front, a coverage bit; in
+// the band, open.  `open` (level-free): the open texels' bits; with TILE, their nearest depth in
+// `tile` too.  D.open receives the triangles that left a texel open.
+template <int TS, bool TILE, bool PROF>
+__device__ __forceinline__ void draw_tris(DrawSm& D, const TriWork& w, uint32_t full, bool nested, const Level* lv,
+                                          uint32_t* cov,
+                                          uint32_t* open, uint32_t* tile, const LightParams& lp, int u24,
+                                          unsigned int& visits, unsigned int& writes)
+{
+    constexpr int WPR = TS / 32, NW = TS * WPR;
+    constexpr bool kRowsOfOne = TS >= 64, kOwnRow = kRowsOfOne && !TILE;
+    const int lane = threadIdx.x & 31;
+    uint32_t front = w.front & ~full, deep = w.deep & ~full;
+    if (nested) {
+        const uint32_t low = w.front & (0u - w.front);
+        front &= low;
+        deep &= low - 1u;  // low = 0: all
+    }
+    int rows = 0;
+    if (front | deep) {
+        TriDraw& S = D.tri[lane];
+        const float inv_a = 1.f / w.ed.area2;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            S.A[k] = w.ed.A[k]; S.Bc[k] = w.ed.Bc[k]; S.C[k] = w.ed.C[k];
+            S.inv[k] = __fdividef(-1.f, __fadd_rn(w.ed.A[k], 0.f));  // A = -0 is 0
+            S.e[k] = w.T.d[k] * inv_a;
+        }
+        S.x0 = (short)w.x0;
+        S.x1 = (short)w.x1;
+        S.y0 = w.y0;
+        S.err = w.err;
+        S.rows = rows = w.y1 - w.y0 + 1;
+        S.front = front;
+        S.deep = deep;
+    }
+    if (lane == 0) D.open = 0u;
+    auto draw_row = [&](const TriDraw& S, int t, int iy) {
+        const float py = (float)iy + 0.5f;
+        float a = (float)S.x0, b = (float)S.x1;
+        float tk[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            tk[k] = __fmaf_rn(S.Bc[k], py, S.C[k]);
+            row_edge(S.A[k], S.inv[k], tk[k], a, b);
+        }
+        const int lo = (int)a, hi = (int)b;
+        if (lo > hi) return;
+        if (PROF) visits += (unsigned int)(hi - lo + 1);
+#pragma unroll 1
+        for (uint32_t m = S.front; m; m &= m - 1u) {
+            uint32_t* row = cov + (__ffs((int)m) - 1) * NW + iy * WPR;
+            if constexpr (kOwnRow && TS == 128) {
+                uint4 v = *reinterpret_cast<uint4*>(row);
+                v.x |= span_word(lo, hi, 0); v.y |= span_word(lo, hi, 1);
+                v.z |= span_word(lo, hi, 2); v.w |= span_word(lo, hi, 3);
+                *reinterpret_cast<uint4*>(row) = v;
+            } else if constexpr (kOwnRow && TS == 64) {
+                uint2 v = *reinterpret_cast<uint2*>(row);
+                v.x |= span_word(lo, hi, 0); v.y |= span_word(lo, hi, 1);
+                *reinterpret_cast<uint2*>(row) = v;
+            } else {
+#pragma unroll 1
+                for (int q = lo >> 5; q <= (hi >> 5); ++q) atomicOr(&row[q], span_word(lo, hi, q));
+            }
+        }
+        uint32_t m = S.deep;
+        if (m == 0u) return;
+        const float A0 = S.A[0], A1 = S.A[1], A2 = S.A[2], e0 = S.e[0], e1 = S.e[1], e2 = S.e[2];
+        auto depth_px = [&](float px) {
+            return depth_at(__fmaf_rn(A0, px, tk[0]), __fmaf_rn(A1, px, tk[1]), __fmaf_rn(A2, px, tk[2]), e0, e1, e2);
+        };
+        const float pl = a + 0.5f, ph = b + 0.5f, dl = depth_px(pl), dh = depth_px(ph), err2 = 2.f * S.err;
+#pragma unroll 1
+        for (; m; m &= m - 1u) {
+            const int l = __ffs((int)m) - 1;
+            const float pa = lv[l].pa, base = __fmaf_rn(lv[l].pb, py, lv[l].pc);
+            const float fr = -lv[l].front, bk = lv[l].back;
+            // the gap is linear along the row, up to the depths' rounding: its
+            // ends tell which texels are in front and which are behind, but
+            // for those about the roots
+            const float ga = dl - __fmaf_rn(pa, pl, base), gb = dh - __fmaf_rn(pa, ph, base);
+            float fa = a, fb = b, ca = a, cb = b;
+            if (!below(ga, gb, fr - err2, -0.02f, fa, fb)) fb = fa - 1.f;
+            if (!below(ga, gb, bk + err2, 0.02f, ca, cb)) continue;
+            const int f0 = (int)fa, f1 = (int)fb, c0 = (int)ca, c1 = (int)cb;
+#pragma unroll 1
+            for (int q = c0 >> 5; q <= (c1 >> 5); ++q) {
+                const int word = iy * WPR + q;
+                uint32_t c = f0 <= f1 && q >= (f0 >> 5) && q <= (f1 >> 5) ? span_word(f0, f1, q) : 0u, o = 0u;
+                uint32_t r = span_word(c0, c1, q) & ~c & ~cov[l * NW + word];
+#pragma unroll 1
+                for (; r; r &= r - 1u) {
+                    const int x = __ffs((int)r) - 1;
+                    const float px = (float)(32 * q + x) + 0.5f;
+                    const float depth = depth_px(px), gap = depth - __fmaf_rn(pa, px, base);
+                    if (PROF) ++writes;
+                    if (gap < fr) {
+                        c |= 1u << x;
+                    } else if (!(gap >= bk)) {
+                        o |= 1u << x;
+                        if (TILE) atomicMin(&tile[iy * TS + 32 * q + x], depth_store_key(depth, lp, u24));
+                    }
+                }
+                if (c) atomicOr(&cov[l * NW + word], c);
+                if (o) {
+                    atomicOr(&open[word], o);
+                    atomicOr(&D.open, 1u << t);
+                }
+            }
+        }
+    };
+    if constexpr (kRowsOfOne) {
+        unsigned int todo = __ballot_sync(0xffffffffu, rows > 0);
+        __syncwarp();
+#pragma unroll 1
+        for (; todo; todo &= todo - 1u) {
+            const int t = __ffs((int)todo) - 1;
+            const TriDraw& S = D.tri[t];
+            const int end = S.y0 + S.rows;
+#pragma unroll 1
+            for (int iy = S.y0 + lane; iy < end; iy += 32) draw_row(S, t, iy);
+            __syncwarp();  // the next triangle's rows are other lanes'
+        }
+    } else {
+        const int inc = warp_incl_scan(rows);
+        D.pref[lane] = inc;
+        __syncwarp();
+        const int total = __shfl_sync(0xffffffffu, inc, 31);
+#pragma unroll 1
+        for (int u = lane; u < total; u += 32) {
+            int t = 0;  // the row's triangle: the first with pref > u
+#pragma unroll
+            for (int step = 16; step; step >>= 1)
+                if (D.pref[t + step - 1] <= u) t += step;
+            const TriDraw& S = D.tri[t];
+            draw_row(S, t, S.y0 + u - (t ? D.pref[t - 1] : 0));
+        }
+        __syncwarp();
+    }
+}
+
+// Levels that are covered everywhere given that those of f are.
+__device__ __forceinline__ uint32_t full_after(uint32_t f, bool nested, uint32_t all)
+{
+    return nested && f ? all & ~((f & (0u - f)) - 1u) : f;
+}
+
+// Coverage word q of every level in turn, with the levels' nesting and the
+// full levels applied: f(l, word).
+template <int TS, typename F>
+__device__ __forceinline__ void for_levels(const uint32_t* cov, int nl, bool nested, uint32_t full, int q, F f)
+{
+    uint32_t c = 0u;
+#pragma unroll 1
+    for (int l = 0; l < nl; ++l) {
+        const uint32_t v = cov[l * (TS * TS / 32) + q];
+        c = (full >> l) & 1u ? 0xFFFFFFFFu : (nested ? c | v : v);
+        f(l, c);
+    }
+}
+
+// The levels whose coverage bits are all set, for one full warp.
+template <int TS>
+__device__ __forceinline__ uint32_t full_levels(const uint32_t* cov, int nl, bool nested, uint32_t full)
+{
+    uint32_t ok = (1u << nl) - 1u;
+#pragma unroll 1
+    for (int q = threadIdx.x & 31; q < TS * TS / 32; q += 32)
+        for_levels<TS>(cov, nl, nested, full, q, [&](int l, uint32_t c) {
+            if (c != 0xFFFFFFFFu) ok &= ~(1u << l);
+        });
+    return __reduce_and_sync(0xffffffffu, ok);
+}
+
+// Write the levels' nesting and the full levels into the coverage words q =
+// q_begin, q_begin + q_stride, ...: some = a bit is set, hole = a bit is not.
+template <int TS>
+__device__ __forceinline__ void finish_words(uint32_t* cov, int nl, bool nested, uint32_t full, int q_begin, int q_stride,
+                                             uint32_t& some, uint32_t& hole)
+{
+#pragma unroll 1
+    for (int q = q_begin; q < TS * TS / 32; q += q_stride)
+        for_levels<TS>(cov, nl, nested, full, q, [&](int l, uint32_t c) {
+            cov[l * (TS * TS / 32) + q] = c;
+            some |= c;
+            hole |= ~c;
+        });
+}
+
+// Bins of a tile, clamped to the bin pool.
+__device__ __forceinline__ void tile_bins(const Buffers& B, const WaveDev* W, uint32_t te, uint64_t& off, uint32_t& cnt)
+{
+    off = B.t_off[te];
+    cnt = B.t_cnt[te];
+    const uint64_t cap = (uint64_t)W->bin_cap;
+    if (off + cnt > cap) cnt = off < cap ? (uint32_t)(cap - off) : 0u;
+}
+
+// Words of a tile's record, and its place in the pool: the 16-byte offset
+// plus one, or 0 when the pool is full (the host grows it and reruns the
+// wave).  Called by one thread.
+__device__ __forceinline__ uint32_t alloc_record(const Buffers& B, const WaveDev* W, uint32_t words)
+{
+    const unsigned long long quads = (words + 3u) / 4u;
+    const unsigned long long pos = atomicAdd(&B.ctr->cov_next, quads);
+    return pos + quads <= (unsigned long long)W->cov_cap ? (uint32_t)pos + 1u : 0u;
+}
+
+// Box of the texels set in cov or open (TS * TS / 32 words each), packed as in
+// the record's header; by one full warp.
+template <int TS>
+__device__ __forceinline__ uint32_t texel_box(const uint32_t* cov, const uint32_t* open)
+{
+    constexpr int WPR = TS / 32, NW = TS * WPR;
+    int x0 = 255, x1 = -1, y0 = 255, y1 = -1;
+#pragma unroll 1
+    for (int q = threadIdx.x & 31; q < NW; q += 32) {
+        const uint32_t c = cov[q] | open[q];
+        if (c) {
+            const int y = q / WPR, xb = (q % WPR) * 32;
+            y0 = min(y0, y); y1 = max(y1, y);
+            x0 = min(x0, xb + __ffs((int)c) - 1); x1 = max(x1, xb + 31 - __clz((int)c));
+        }
+    }
+    x0 = __reduce_min_sync(0xffffffffu, x0); x1 = __reduce_max_sync(0xffffffffu, x1);
+    y0 = __reduce_min_sync(0xffffffffu, y0); y1 = __reduce_max_sync(0xffffffffu, y1);
+    return x1 < 0 ? kBoxNone : (uint32_t)x0 | ((uint32_t)x1 << 8) | ((uint32_t)y0 << 16) | ((uint32_t)y1 << 24);
+}
+
+// ---------------------------------------------------------------------------
+// k_tile_warp: fused path -- one warp per non-empty tile: the tile's coverage
+// bits.  A tile with more than warp_bins() binned triangles or more than
+// kWarpOpen that leave texels open, and a 64-texel tile with more than
+// kWarpRecv receivers or more than kWarpKept triangles in front of or across a
+// level, is listed for k_raster_test.  A tile is a small
+// work item: one warp each keeps many tiles in flight per SM, which hides the
+// chain of dependent loads that starts a tile.
+//
+// What bounds it: instruction issue (53-70 % of the slots over full waves, the
+// rest waits for the triangles' vertices).  A depth per texel and a test per
+// sample cost one step per covered texel and one per sample; a bit per texel
+// costs one step per row of a triangle, and a plane's samples read it as
+// words.  The code is kept small (loops not unrolled, one copy of each): at
+// twice the size the warps waited for instructions up to nine cycles each.
+// With k_cells, against depth tiles and a test per sample: 2 520 modules on
+// trackers over terrain, 33 suns: 3.2 -> 1.8 ms all told; a facade of 200
+// modules, 50 000 triangles, n = 8, a year of hours: 17.5 -> 13.4 ms.
+// ---------------------------------------------------------------------------
+constexpr int kWarpOpen = 32;
+constexpr int kWarpKept = 80;
+constexpr int kWarpRecv = 16;
+constexpr int kTileWarps = 4;  // warps per block
+constexpr int kTileBlocks = 8; // blocks per SM (64 registers a thread)
+
+template <int TS>
+__device__ constexpr uint32_t warp_bins() { return TS == 32 ? 256u : (TS == 64 ? 512u : 96u); }
+
+template <int TS>
+struct __align__(16) WarpSm {
+    TriS tri[kWarpOpen];
+    DrawSm d;
+    Level lv[Levels<TS>::n];
+    __align__(16) uint32_t cov[WarpLevels<TS>::n * TS * TS / 32];  // draw_tris takes a row at once
+    uint32_t open[TS * TS / 32];
+};
+static_assert(offsetof(WarpSm<64>, cov) % 16 == 0 && sizeof(WarpSm<64>) % 16 == 0 &&
+              offsetof(WarpSm<128>, cov) % 16 == 0 && sizeof(WarpSm<128>) % 16 == 0, "rows are read as vectors");
+
+template <int TS, bool PROF>
+__global__ void __launch_bounds__(kTileWarps * 32, kTileBlocks) k_tile_warp(const WaveDev* __restrict__ W,
+                                                                  const JobDev* __restrict__ jobs, Buffers B)
+{
+    extern __shared__ __align__(16) unsigned char tile_smem[];  // kTileWarps WarpSm, set at launch
+    constexpr int NW = TS * TS / 32;
+    unsigned int p_visits = 0, p_writes = 0, p_culled = 0, p_tiles = 0, p_stiles = 0, p_hr = 0, p_hb = 0, p_ht = 0;
+    const int lane = threadIdx.x & 31;
+    WarpSm<TS>& sm = reinterpret_cast<WarpSm<TS>*>(tile_smem)[threadIdx.x >> 5];
+    // the bins are incomplete when the pool overflowed: the wave is rerun
+    // with a larger pool, so nothing here may read them
+    const unsigned int n_ne = (B.ctr->overflow & 1u) ? 0u : B.ctr->n_nonempty;
+    // tiles of many triangles come first, from the front of the list, the
+    // others from its end (k_scan_c)
+    const unsigned int n_first = B.ctr->n_first, last = (unsigned int)(W->tot_te - 1);
+    const int nj = W->n_jobs;
+    const int u24 = W->depth_u24;
+    // with a tile or less for each resident warp the largest tile is the
+    // kernel's time: 32 triangles of up to 128 rows are enough for a warp
+    // (77 facade modules, 72 suns: both tile kernels 353 us with 96, 240 with 32)
+    const uint32_t most = TS == 128 && n_ne <= gridDim.x * (unsigned int)kTileWarps ? 32u : warp_bins<TS>();
+    unsigned int next = 0;
+    if (lane == 0) next = atomicAdd(&B.ctr->raster_next, 1u);
+    next = __shfl_sync(0xffffffffu, next, 0);
+    while (next < n_ne) {
+        const unsigned int item = next;
+        if (lane == 0) next = atomicAdd(&B.ctr->raster_next, 1u);  // claim the following tile now
+        const uint32_t te = B.nonempty[item < n_first ? item : last - (item - n_first)];
+        uint64_t off;
+        uint32_t cnt;
+        tile_bins(B, W, te, off, cnt);
+        const uint32_t nrecv = B.t_rcnt[te], plane = B.t_plane[te];
+        int j, ls, tx, ty;
+        decode_tile(jobs, nj, te, j, ls, tx, ty);
+        const JobDev& J = jobs[j];
+        const bool crowd = TS == 64 && nrecv > (uint32_t)kWarpRecv;
+        bool heavy = crowd || cnt > most;
+        if (PROF && lane == 0) {
+            if (crowd) ++p_hr;
+            else if (heavy) ++p_hb;
+        }
+        if (!heavy) {
+            const LightParams& lp = B.lp[J.js_base + ls];
+            bool nested;
+            const int nl = build_levels<TS>(sm.lv, J, B, W, te, ls, tx, ty, plane, nested);
+            heavy = nl > WarpLevels<TS>::n;
+#pragma unroll 4
+            for (int q = lane; q < (heavy ? 0 : nl * NW); q += 32) sm.cov[q] = 0u;
+#pragma unroll 4
+            for (int q = lane; q < NW; q += 32) sm.open[q] = 0u;
+            __syncwarp();
+            const uint32_t all = (1u << nl) - 1u;
+            const float ox = (float)(tx * TS), oy = (float)(ty * TS);
+            uint32_t full = 0u;    // levels covered everywhere
+            int n = 0, kept = 0;   // triangles that left a texel open; in front of or across a level
+#pragma unroll 1
+            for (uint32_t b0 = 0; b0 < cnt && !heavy && full != all; b0 += 32) {
+                TriWork w;
+                w.front = w.deep = 0u;
+                w.whole = false;
+                if (b0 + lane < cnt)
+                    classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, w, p_culled);
+                full = full_after(full | __reduce_or_sync(0xffffffffu, w.whole ? w.front : 0u), nested, all);
+                const unsigned int use = __ballot_sync(0xffffffffu, (w.front | w.deep) != 0u);
+                kept += __popc(use);
+                if (use == 0u || full == all) continue;
+                draw_tris<TS, false, PROF>(sm.d, w, full, nested, sm.lv, sm.cov, sm.open, nullptr, lp, u24, p_visits,
+                                           p_writes);
+                const uint32_t op = sm.d.open;
+                const int slot = n + __popc(op & ((1u << lane) - 1u));
+                if (((op >> lane) & 1u) && slot < kWarpOpen) {
+                    const TriDraw& S = sm.d.tri[lane];
+                    sm.tri[slot].p = make_float4(S.A[0], S.Bc[0], S.C[0], S.A[1]);
+                    sm.tri[slot].q = make_float4(S.Bc[1], S.C[1], S.A[2], S.Bc[2]);
+                    sm.tri[slot].r = make_float4(S.C[2], S.e[0], S.e[1], S.e[2]);
+                }
+                n += __popc(op);
+                heavy = n > kWarpOpen || (TS == 64 && kept > kWarpKept);
+                __syncwarp();  // the set-up may be replaced
+                if (b0 + 32 < cnt) full = full_levels<TS>(sm.cov, nl, nested, full);
+            }
+            if (full == all) heavy = false;
+            if (PROF && lane == 0) {
+                if (heavy) ++p_ht;
+                else {
+                    ++p_tiles;
+                    if (kept == 0) ++p_stiles;
+                }
+            }
+            if (!heavy) {
+                uint32_t state = kTileFull;
+                if (full != all) {
+                    // does any texel matter, is any not covered?
+                    uint32_t some = 0u, hole = 0u;
+                    finish_words<TS>(sm.cov, nl, nested, full, lane, 32, some, hole);
+                    __syncwarp();
+                    if (!__any_sync(0xffffffffu, hole != 0u)) {
+                        state = kTileFull;
+                    } else if (n == 0 && !__any_sync(0xffffffffu, some != 0u)) {
+                        state = kTileLit;
+                    } else {
+                        const uint32_t words = (uint32_t)(kRecHead + nl * NW + (n ? NW + 12 * n : 0));
+                        if (lane == 0) state = alloc_record(B, W, words);
+                        state = __shfl_sync(0xffffffffu, state, 0);
+                        if (state) {
+                            uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
+                            if (lane == 0) rec[0] = (uint32_t)nl | (n ? kRecOpen | ((uint32_t)n << 16) : 0u);
+                            else if (lane <= nl) rec[lane] = (uint32_t)sm.lv[lane - 1].plane;
+#pragma unroll 1
+                            for (int l = 0; l < nl; ++l) {
+                                const uint32_t box = texel_box<TS>(sm.cov + l * NW, sm.open);
+                                if (lane == 0) rec[kRecBox + l] = box;
+                            }
+                            uint32_t* dst = rec + kRecHead;
+                            for (int q = lane; q < nl * NW; q += 32) dst[q] = sm.cov[q];
+                            if (n) {
+                                dst += nl * NW;
+                                for (int q = lane; q < NW; q += 32) dst[q] = sm.open[q];
+                                dst += NW;
+                                const uint32_t* src = reinterpret_cast<const uint32_t*>(sm.tri);
+                                for (int q = lane; q < 12 * n; q += 32) dst[q] = src[q];
+                            }
+                        }
+                    }
+                }
+                if (lane == 0) B.t_cnt[te] = state;
+            }
+        }
+        if (heavy && lane == 0) {
+            const unsigned int pos = atomicAdd(&B.ctr->n_heavy, 1u);
+            if (pos < (uint64_t)W->tot_te) B.heavy[pos] = te;
+        }
+        __syncwarp();  // the warp's shared memory may be reused
+        next = __shfl_sync(0xffffffffu, next, 0);
+    }
+    if (PROF) {
+        flush_profile(B, 0u, p_visits, p_visits + p_writes, p_culled);
+        flush_profile2(B, 0u, p_tiles, 0u, p_stiles, 0u);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) {
+            p_hr += __shfl_xor_sync(0xffffffffu, p_hr, off);
+            p_hb += __shfl_xor_sync(0xffffffffu, p_hb, off);
+            p_ht += __shfl_xor_sync(0xffffffffu, p_ht, off);
+        }
+        if (lane == 0) {
+            atomicAdd(&B.ctr->prof_heavy_why[0], (unsigned long long)p_hr);
+            atomicAdd(&B.ctr->prof_heavy_why[1], (unsigned long long)p_hb);
+            atomicAdd(&B.ctr->prof_heavy_why[2], (unsigned long long)p_ht);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_raster_test: fused path, the tiles k_tile_warp listed -- one block per
+// tile, its warps taking up to 32 triangles at a time by themselves (as many
+// each: with 32 for some and none for others the facade year's share of this
+// kernel was 0.96 ms, now 0.63); texels left open keep their nearest depth in
+// a shared tile that goes to the record.  Bound by the longest tile: there are
+// fewer than blocks in most waves.
+// ---------------------------------------------------------------------------
+template <int TS>
+struct HeavyCfg {
+    static constexpr int threads = TS == 32 ? 128 : 256;
+    static constexpr int min_blocks = TS == 32 ? 8 : (TS == 64 ? 4 : 3);
+};
+
+template <int TS>
+struct __align__(16) HeavySm {
+    uint32_t tile[TS * TS];  // nearest depth keys of open texels
+    uint32_t cov[Levels<TS>::n * TS * TS / 32];
+    uint32_t open[TS * TS / 32];
+    DrawSm d[HeavyCfg<TS>::threads / 32];
+    Level lv[Levels<TS>::n];
+    int nl;
+    int nested;
+    uint32_t full, state;
+    unsigned int item[2];
+};
+
+template <int TS, bool PROF>
+__global__ void __launch_bounds__(HeavyCfg<TS>::threads, HeavyCfg<TS>::min_blocks)
+    k_raster_test(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs, Buffers B)
+{
+    constexpr int NW = TS * TS / 32, kWarps = HeavyCfg<TS>::threads / 32;
+    extern __shared__ __align__(16) unsigned char tile_smem[];  // HeavySm, set at launch
+    HeavySm<TS>& sm = *reinterpret_cast<HeavySm<TS>*>(tile_smem);
+    unsigned int p_visits = 0, p_writes = 0, p_culled = 0, p_tiles = 0;
+    // incomplete bins (pool overflow, the wave is rerun): nothing to read
+    const unsigned int n_ne = (B.ctr->overflow & 1u) ? 0u : min(B.ctr->n_heavy, (unsigned int)W->tot_te);
+    const int nj = W->n_jobs;
+    const int u24 = W->depth_u24;
+    const int tid = threadIdx.x, bd = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) sm.item[0] = atomicAdd(&B.ctr->heavy_next, 1u);
+    __syncthreads();
+    for (int par = 0;; par ^= 1) {
+        // the next tile is claimed while this one runs; the barriers inside
+        // the tile publish it
+        const unsigned int item = sm.item[par];
+        if (item >= n_ne) break;
+        if (tid == 0) sm.item[par ^ 1] = atomicAdd(&B.ctr->heavy_next, 1u);
+        const uint32_t te = B.heavy[item];
+        uint64_t off;
+        uint32_t cnt;
+        tile_bins(B, W, te, off, cnt);
+        int j, ls, tx, ty;
+        decode_tile(jobs, nj, te, j, ls, tx, ty);
+        const JobDev& J = jobs[j];
+        const LightParams& lp = B.lp[J.js_base + ls];
+        if (warp == 0) {
+            bool nested;
+            const int nl = build_levels<TS>(sm.lv, J, B, W, te, ls, tx, ty, B.t_plane[te], nested);
+            if (lane == 0) {
+                sm.nl = nl;
+                sm.nested = nested;
+                sm.full = 0u;
+            }
+        }
+        uint4* t4 = reinterpret_cast<uint4*>(sm.tile);
+        for (int q = tid; q < TS * TS / 4; q += bd) t4[q] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+        for (int q = tid; q < Levels<TS>::n * NW; q += bd) sm.cov[q] = 0u;
+        for (int q = tid; q < NW; q += bd) sm.open[q] = 0u;
+        if (PROF && tid == 0) ++p_tiles;
+        __syncthreads();
+        const int nl = sm.nl;
+        const bool nested = sm.nested != 0;
+        const uint32_t all = (1u << nl) - 1u;
+        const float ox = (float)(tx * TS), oy = (float)(ty * TS);
+        uint32_t full = 0u;
+        // up to 32 triangles a warp and turn, the same number for each
+        const uint32_t turns = (cnt + 32u * kWarps - 1u) / (32u * kWarps);
+        const uint32_t share = (cnt + kWarps * turns - 1u) / (kWarps * turns);
+#pragma unroll 1
+        for (uint32_t b0 = share * warp; b0 < cnt; b0 += share * kWarps) {
+            full |= *(volatile uint32_t*)&sm.full;
+            full = __reduce_or_sync(0xffffffffu, full);
+            if (full == all) break;  // every sample of the tile is shaded
+            TriWork w;
+            w.front = w.deep = 0u;
+            w.whole = false;
+            if ((uint32_t)lane < share && b0 + lane < cnt)
+                classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, w, p_culled);
+            const uint32_t f = full_after(__reduce_or_sync(0xffffffffu, w.whole ? w.front : 0u), nested, all);
+            if (f & ~full) {
+                full |= f;
+                if (lane == 0) atomicOr(&sm.full, f);
+            }
+            if (full == all || !__any_sync(0xffffffffu, (w.front | w.deep) != 0u)) continue;
+            draw_tris<TS, true, PROF>(sm.d[warp], w, full, nested, sm.lv, sm.cov, sm.open, sm.tile, lp, u24, p_visits,
+                                      p_writes);
+            if (b0 + share * kWarps < cnt) full = full_levels<TS>(sm.cov, nl, nested, full);
+        }
+        __syncthreads();
+        full = sm.full;
+        uint32_t some = 0u, hole = 0u, op = 0u;
+        finish_words<TS>(sm.cov, nl, nested, full, tid, bd, some, hole);
+        for (int q = tid; q < NW; q += bd) op |= sm.open[q];
+        const bool any_hole = __syncthreads_or(hole != 0u), any_open = __syncthreads_or(op != 0u),
+                   any_some = __syncthreads_or(some != 0u);
+        uint32_t state = !any_hole ? kTileFullHeavy : kTileLit;
+        if (any_hole && (any_some || any_open)) {
+            const uint32_t words = (uint32_t)(kRecHead + nl * NW + (any_open ? NW + TS * TS : 0));
+            if (tid == 0) sm.state = alloc_record(B, W, words);
+            __syncthreads();
+            state = sm.state;
+            if (state) {
+                uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
+                if (tid == 0) rec[0] = (uint32_t)nl | kRecHeavy | (any_open ? kRecOpen | kRecDepth : 0u);
+                else if (tid <= nl) rec[tid] = (uint32_t)sm.lv[tid - 1].plane;
+#pragma unroll 1
+                for (int l = warp; l < nl; l += kWarps) {
+                    const uint32_t box = texel_box<TS>(sm.cov + l * NW, sm.open);
+                    if (lane == 0) rec[kRecBox + l] = box;
+                }
+                uint32_t* dst = rec + kRecHead;
+                for (int q = tid; q < nl * NW; q += bd) dst[q] = sm.cov[q];
+                if (any_open) {
+                    dst += nl * NW;
+                    for (int q = tid; q < NW; q += bd) dst[q] = sm.open[q];
+                    dst += NW;
+                    for (int q = tid; q < TS * TS; q += bd) dst[q] = sm.tile[q];
+                }
+            }
+        }
+        if (tid == 0) B.t_cnt[te] = state;
+        __syncthreads();  // the tile's shared memory may be reused
+    }
+    if (PROF) {
+        flush_profile(B, 0u, p_visits, p_visits + p_writes, p_culled);
+        flush_profile2(B, 0u, p_tiles, 0u, 0u, 0u);
+        flush_heavy(B, 0u, p_visits + p_writes, p_tiles);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2580,248 +2976,667 @@ __device__ __forceinline__ void zero_step_module(const JobDev& J, const ModuleDe
     }
 }
 
-// Fused path: the tallies were accumulated by the tile kernels.  The PV model
-// of one (step, module) item by one warp: lanes over its cells into substring
-// minima in shared memory, then over the candidate currents of the MPP.
-// `imin` holds kMaxSub entries.
-__device__ void pv_module_warp(const JobDev* jobs, int nj, int64_t item, const Buffers& B, uint32_t* imin)
+// ---------------------------------------------------------------------------
+// k_pv, k_cells: fused path -- the PV model per (step, module) (Section 2, step
+// 4), with the shaded samples per cell from the tiles' coverage
+//
+// k_pv, one (step, module) per lane: a module over lit tiles only (most of
+// them) carries one current in every cell, so its maximum power point needs no
+// cell; the others, and all when the diffuse term or an output is per cell,
+// are listed.  k_cells takes the list one module a warp (the modules of a
+// shaded table are neighbours: left to the warp that found them, 32 in a row
+// kept one warp busy while others had none), or one a block when there are
+// fewer modules than half the warps, a lane per cell: the texels of
+// the cell's extreme samples box those of all (a sample's texel is monotone in
+// its indices), and where nothing in that box is covered, or all of it, the
+// cell is lit or shaded whole; the samples of the remaining cells are shared
+// out over the lanes.  Nothing is accumulated across tiles, so there are no
+// tallies to clear and no atomics in device memory.  Bound by instruction
+// issue: a third of the year of 2 520 tracker modules' time goes to the samples
+// of mixed cells.
+// ---------------------------------------------------------------------------
+constexpr int kPvTiles = 8;    // k_pv: a module over more tiles is looked at by the whole warp
+constexpr int kPvFastSub = 8;  // up to so many substrings a module's voltages are summed in order
+constexpr int kCellWarps = 8, kCellBlocks = 4;  // warps a block, blocks an SM
+
+// Level of plane `plane` in a tile's record (header word h), and its coverage
+// bits.
+__device__ __forceinline__ int level_of(const uint32_t* rec, uint32_t h, int plane)
 {
-    const int lane = threadIdx.x & 31;
-    const int j = job_of(nj, item, [&](int q) { return jobs[q].it_mod; });
-    const JobDev& J = jobs[j];
-    const int64_t li = item - J.it_mod;
-    const int ls = (int)(li / J.n_mods), m = (int)(li % J.n_mods);
-    const int64_t msi = J.ms_base + li;
-    const LightParams& lp = B.lp[J.js_base + ls];
-    const ModuleDev& M = J.mods[m];
-    const int ncell = M.cu * M.cv, C = J.n_cells;
-    const int64_t row = (int64_t)(J.out_row0 + ls);
-    const int64_t cbase = J.cs_base + (int64_t)ls * C + M.cell_base;
-    if (!lp.valid) {
-        if (lane == 0) { B.ms_p[msi] = 0.f; B.ms_pu[msi] = 0.f; B.ms_beam[msi] = 0.f; }
-        for (int c = lane; c < ncell; c += 32) {
-            tally_set(B.cs_cnt, cbase + c, 0u);
-            if (J.out_counts) J.out_counts[row * J.out_cstride + M.cell_base + c] = 0;
-            if (J.out_bits) J.out_bits[row * J.out_cstride + M.cell_base + c] = 0ull;
-        }
-        return;
-    }
-    const ModStep& s = B.ms[msi];
-    const float beam = lp.dni * fmaxf(0.f, s.cosi);
-    const float diff = lp.dhi * (1.f + s.nz) * 0.5f;
-    const float inv_nn = 1.f / J.nn;
-    const int* csub = J.lay_sub + J.lay_off[M.layout];
-    const int ns = M.n_sub;
-    for (int k = lane; k < ns; k += 32) imin[k] = 0x7F800000u;  // +inf
-    __syncwarp();
-    const float* fd = diffuse_row(J, ls);
-    for (int c = lane; c < ncell; c += 32) {
-        const uint32_t cnt = tally_get(B.cs_cnt, cbase + c);
-        if (J.out_counts) J.out_counts[row * J.out_cstride + M.cell_base + c] = (uint8_t)cnt;
-        if (J.out_bits) J.out_bits[row * J.out_cstride + M.cell_base + c] = B.cs_bits[cbase + c];
-        const float gd = fd ? diff * (1.f - fd[M.cell_base + c]) : diff;
-        const float G = beam * (1.f - cnt * inv_nn) + gd;
-        const float I = J.i_ref * G * 1e-3f;
-        atomicMin(&imin[csub[c]], __float_as_uint(I));  // I >= 0: uint order = float order
-    }
-    __syncwarp();
-    if (J.n_str) {  // substring currents for the series-string model (k_string)
-        float* ss = B.ss_i + J.ss_base + (int64_t)ls * J.n_sub_tot + J.sub_base[m];
-        for (int k = lane; k < ns; k += 32) ss[k] = __uint_as_float(imin[k]);
-        if (lane == 0) B.ms_iu[msi] = J.i_ref * (beam + diff) * 1e-3f;
-    }
-    const int* nk = J.lay_nk + J.lay_nk_off[M.layout];
-    float best = 0.f, vsum = 0.f;
-    for (int k = lane; k < ns; k += 32) {
-        const float ik = __uint_as_float(imin[k]);
-        float volt = 0.f;
-        for (int q = 0; q < ns; ++q) volt += __uint_as_float(imin[q]) >= ik ? nk[q] * J.v_cell : -J.v_diode;
-        best = fmaxf(best, ik * volt);
-        vsum += nk[k] * J.v_cell;
-    }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
-        vsum += __shfl_xor_sync(0xffffffffu, vsum, off);
-    }
-    if (lane == 0) {
-        B.ms_p[msi] = best;
-        B.ms_pu[msi] = J.i_ref * (beam + diff) * 1e-3f * vsum;
-        B.ms_beam[msi] = beam;
-    }
-    __syncwarp();
+    const int nl = (int)(h & kRecLevels);
+    int l = 0;
+#pragma unroll 1
+    while (l < nl - 1 && (int)rec[1 + l] != plane) ++l;  // the last level takes every other plane
+    return l;
+}
+__device__ __forceinline__ const uint32_t* level_words(const uint32_t* rec, uint32_t h, int plane, int words)
+{
+    return rec + kRecHead + level_of(rec, h, plane) * words;
 }
 
-// A warp takes bw consecutive (step, module) items, one per lane (bw = 32, or
-// the smallest power of two that still covers the wave in one pass of the
-// grid, so that small waves spread over all warps).  Each lane decodes its
-// item (job, step, module, irradiance, cell layout); the warp then walks the
-// items' cells one module at a time (lanes over its cells, the module's fields
-// taken from its lane) into per-module substring minima in shared memory, and
-// each lane evaluates its own module's MPP.  The arithmetic is that of
-// pv_module_warp, operation for operation (a module's voltage sum is exact in
-// either order), which the warp falls back to when one of its modules has
-// more than kPvFastSub substrings.
-constexpr int kPvWarps = kPvThreads / 32;
-constexpr int kPvFastSub = 8;
-constexpr int kPvUnroll = 4;
-static_assert(32 * kPvFastSub >= kMaxSub, "the per-module path reuses the warp's minima");
+// The words of a row of TS / 32 coverage words, together.
+template <int TS>
+struct RowWords {
+    uint32_t v[TS / 32];
+};
+template <int TS>
+__device__ __forceinline__ RowWords<TS> load_row(const uint32_t* p)
+{
+    RowWords<TS> r;
+    if constexpr (TS == 128) {
+        const uint4 v = *reinterpret_cast<const uint4*>(p);
+        r.v[0] = v.x; r.v[1] = v.y; r.v[2] = v.z; r.v[3] = v.w;
+    } else if constexpr (TS == 64) {
+        const uint2 v = *reinterpret_cast<const uint2*>(p);
+        r.v[0] = v.x; r.v[1] = v.y;
+    } else {
+        r.v[0] = *p;
+    }
+    return r;
+}
+
+// Is the sample at texel (ix, iy), depth d, bias, of a receiver of plane
+// `plane` shaded?  tc: the states of the step's tiles.
+template <int TS, bool PROF>
+__device__ __forceinline__ bool sample_shaded(const Buffers& B, const uint32_t* tc, int tiles_x, int ix, int iy, float d,
+                                              float bias, int plane, const LightParams& lp, int u24,
+                                              unsigned int& samples, unsigned int& h_samples, unsigned int& pairs)
+{
+    constexpr int SH = TileSh<TS>::v, WPR = TS / 32, NW = TS * WPR;
+    const uint32_t state = tc[(iy >> SH) * tiles_x + (ix >> SH)];
+    if (state == kTileLit) return false;
+    if (PROF) ++samples;
+    if (state >= kTileFullHeavy) {
+        if (PROF && state == kTileFullHeavy) ++h_samples;
+        return true;
+    }
+    const uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
+    const uint32_t h = rec[0];
+    if (PROF && (h & kRecHeavy)) ++h_samples;
+    const int lx = ix & (TS - 1), ly = iy & (TS - 1), word = ly * WPR + (lx >> 5);
+    if ((level_words(rec, h, plane, NW)[word] >> (lx & 31)) & 1u) return true;
+    if (!(h & kRecOpen)) return false;
+    const uint32_t* open = rec + kRecHead + (int)(h & kRecLevels) * NW;
+    if (!((open[word] >> (lx & 31)) & 1u)) return false;
+    if (h & kRecDepth) {
+        const uint32_t key = open[NW + ly * TS + lx];
+        return behind_key(d, bias, key, lp.dnear, lp.qscale, u24);
+    }
+    const TriS* tri = reinterpret_cast<const TriS*>(open + NW);
+    const float px = texel_centre(lx), py = texel_centre(ly);
+#pragma unroll 1
+    for (int t = 0; t < (int)(h >> 16); ++t) {
+        if (PROF) ++pairs;
+        if (tri_shades(tri[t], px, py, d, bias, lp, u24)) return true;
+    }
+    return false;
+}
+
+// Samples are looked for per tile by mapping the tile back onto the module
+// (stage_one's box, row_range), one sample more each side.  Where that map
+// magnifies the rounding of positions to more than that -- 2: the sun all but
+// in the module's plane, anywhere; 1: an axis of texels all but constant along
+// the module's rows, at the tile's border -- some samples are not found, and
+// count as lit: sample_found asks for them one by one.
+__device__ __forceinline__ int find_risk(const ModStep& s, float lu, float lv, float inv_p, int R)
+{
+    const float ext = fabsf(lu * s.tax) + fabsf(lv * s.tbx) + fabsf(lu * s.tay) + fabsf(lv * s.tby) + 256.f;
+    const float e = 5e-7f * ((float)R + ext) * inv_p;
+    const float p0 = fabsf(s.tax * s.tby), p1 = fabsf(s.tay * s.tbx), det = fabsf(s.tax * s.tby - s.tay * s.tbx);
+    if (det > 1e-6f * (p0 + p1) &&
+        e * fmaxf(fabsf(s.tbx) + fabsf(s.tby), fabsf(s.tax) + fabsf(s.tay)) > 0.5f * det)
+        return 2;
+    return (fabsf(s.tax) > 1e-6f && e > 0.5f * fabsf(s.tax)) || (fabsf(s.tay) > 1e-6f && e > 0.5f * fabsf(s.tay));
+}
+
+// Is sample (I, Jr) of the module of touch-list entry e among those that tile
+// (tx, ty) finds?
+template <int TS>
+__device__ __noinline__ bool sample_found(const JobDev* jobs, const Buffers& B, unsigned int e, int tx, int ty, int I,
+                                          int Jr)
+{
+    const uint4 entry = B.touch[e];
+    RecvSm R;
+    stage_one<TS>(R, jobs[entry.x & 0x7FFFFFFFu], B, (int)entry.y, tx, ty, (int)entry.z);
+    if (R.item_pref == 0 || I < R.I0 || I > R.I1 || Jr < R.J0 || (Jr - R.J0) * R.ncol >= R.item_pref) return false;
+    int Ib = R.I0, Ie = R.I1;
+    row_range(R, Jr, Ib, Ie);
+    return I >= Ib && I <= Ie;
+}
+
+// Cells of a module some of whose samples are shaded, and some not: coverage
+// and open bits of their texel box (bit 8 r + c: row r, column c of the box),
+// first sample indices and first texel.  A box larger than 8 x 8 (big) has no
+// bits: in cov its tile's coverage words (address), in open.x the distance of
+// the open words to them (0: none); or none of these (0), when it meets
+// several tiles and its samples look their tiles up one by one.
+struct CellQueue {
+    uint2 cov[32], open[32];
+    uint32_t ij[32], xy[32];
+    uint32_t big;  // bit k: entry k is big
+    int risk;            // the module's find_risk
+    unsigned int entry;  // and its place in the list
+};
+
+// floor of one coordinate of the sample at (a, b) along the module axes, as
+// sample_texel has it.
+__device__ __forceinline__ int axis_texel(float a, float b, float ta, float tb, float t0, float r_max)
+{
+    return texel_floor(__fmaf_rn(a, ta, __fmaf_rn(b, tb, t0)), r_max);
+}
+
+// Shaded samples of cell c of a module (have: c is one), a lane per cell, for
+// one full warp and one module; `bits` receives the flags of samples k = j * n
+// + i < 64.  tc: the states of the step's tiles.
+template <int TS, bool PROF>
+__device__ __forceinline__ int cell_shaded(const Buffers& B, const JobDev& J, const ModStep& s, int cu, int plane,
+                                           float p_over_n, const LightParams& lp, int u24, const uint32_t* tc, int c,
+                                           bool have, const JobDev* jobs, CellQueue& Q, unsigned long long& bits, unsigned int& cand,
+                                           unsigned int& samples, unsigned int& h_samples, unsigned int& pairs)
+{
+    constexpr int SH = TileSh<TS>::v, WPR = TS / 32, NW = TS * WPR;
+    const int lane = threadIdx.x & 31;
+    const int n = J.n, nn = J.nn, tiles_x = J.tiles_x;
+    const float r_max = (float)(J.R - 1);
+    bool full = false, mixed = false, big = false;
+    int I0 = 0, J0 = 0, x0 = 0, y0 = 0, xe = -1, ye = -1;
+    if (have) {
+        const int cv = fdiv(c, cu, __frcp_rn((float)cu));
+        I0 = (c - cv * cu) * n;
+        J0 = cv * n;
+        // along each module axis the end samples reach the least and the
+        // largest texel of either coordinate
+        const float a0 = __fmul_rn((float)I0 + 0.5f, p_over_n), a1 = __fmul_rn((float)(I0 + n - 1) + 0.5f, p_over_n);
+        const float b0 = __fmul_rn((float)J0 + 0.5f, p_over_n), b1 = __fmul_rn((float)(J0 + n - 1) + 0.5f, p_over_n);
+        x0 = axis_texel(s.tax > 0.f ? a0 : a1, s.tbx > 0.f ? b0 : b1, s.tax, s.tbx, s.tx0, r_max);
+        y0 = axis_texel(s.tay > 0.f ? a0 : a1, s.tby > 0.f ? b0 : b1, s.tay, s.tby, s.ty0, r_max);
+        const int x1 = axis_texel(s.tax > 0.f ? a1 : a0, s.tbx > 0.f ? b1 : b0, s.tax, s.tbx, s.tx0, r_max);
+        const int y1 = axis_texel(s.tay > 0.f ? a1 : a0, s.tby > 0.f ? b1 : b0, s.tay, s.tby, s.ty0, r_max);
+        xe = x1;
+        ye = y1;
+        big = x1 - x0 > 7 || y1 - y0 > 7;
+    }
+    uint32_t clo = 0u, chi = 0u, olo = 0u, ohi = 0u;  // rows 0-3 and 4-7 of the box's bits
+    bool some = false, hole = false;
+    const uint32_t* word = nullptr;  // big, one tile: its coverage words
+    int odist = 0;
+    if (have) {
+        const int txa = x0 >> SH, txb = xe >> SH, tya = y0 >> SH, tyb = ye >> SH;
+#pragma unroll 1
+        for (int ty = tya; ty <= tyb; ++ty)
+#pragma unroll 1
+            for (int tx = txa; tx <= txb; ++tx) {
+                const uint32_t state = tc[ty * tiles_x + tx];
+                if (state == kTileLit) {
+                    hole = true;
+                    continue;
+                }
+                const int lx0 = max(x0 - (tx << SH), 0), lx1 = min(xe - (tx << SH), TS - 1);
+                const int ly0 = max(y0 - (ty << SH), 0), ly1 = min(ye - (ty << SH), TS - 1);
+                const bool all = state >= kTileFullHeavy;
+                const uint32_t* w = nullptr;  // the level's coverage
+                int o = 0;                    // its distance to the open bits, 0: none
+                if (!all) {
+                    const uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
+                    const uint32_t h = rec[0];
+                    w = level_words(rec, h, plane, NW);
+                    if (h & kRecOpen) o = (int)(rec + kRecHead + (int)(h & kRecLevels) * NW - w);
+                }
+                if (!big) {
+                    const int q = lx0 >> 5, col = (tx << SH) + lx0 - x0, row = (ty << SH) + ly0 - y0;
+                    const uint32_t m = (2u << (lx1 - lx0)) - 1u;
+#pragma unroll 1
+                    for (int r = 0; r <= ly1 - ly0; ++r) {
+                        const int sh = 8 * ((row + r) & 3) + col;
+                        uint32_t v = 0xFFFFFFFFu;
+                        if (!all) {
+                            const uint32_t* wr = w + (ly0 + r) * WPR + q;
+                            const bool two = WPR > 1 && q + 1 < WPR;
+                            v = WPR > 1 ? __funnelshift_r(wr[0], two ? wr[1] : 0u, lx0 & 31) : wr[0] >> lx0;
+                            if (o) {
+                                const uint32_t p =
+                                    WPR > 1 ? __funnelshift_r(wr[o], two ? wr[o + 1] : 0u, lx0 & 31) : wr[o] >> lx0;
+                                if (row + r < 4) olo |= (p & m) << sh;
+                                else ohi |= (p & m) << sh;
+                            }
+                        }
+                        if (row + r < 4) clo |= (v & m) << sh;
+                        else chi |= (v & m) << sh;
+                        hole = hole || (~v & m) != 0u;
+                    }
+                } else if (all) {
+                    some = true;
+                } else {
+                    RowWords<TS> m;
+                    uint32_t sm = 0u, hl = 0u;
+#pragma unroll
+                    for (int k = 0; k < WPR; ++k) m.v[k] = span_word(lx0, lx1, k);
+#pragma unroll 4
+                    for (int ly = ly0; ly <= ly1; ++ly) {
+                        const RowWords<TS> v = load_row<TS>(w + ly * WPR);
+#pragma unroll
+                        for (int k = 0; k < WPR; ++k) {
+                            sm |= v.v[k] & m.v[k];
+                            hl |= ~v.v[k] & m.v[k];
+                        }
+                    }
+                    if (o && sm == 0u) {
+#pragma unroll 1
+                        for (int ly = ly0; ly <= ly1; ++ly) {
+                            const RowWords<TS> v = load_row<TS>(w + o + ly * WPR);
+#pragma unroll
+                            for (int k = 0; k < WPR; ++k) sm |= v.v[k] & m.v[k];
+                        }
+                    }
+                    some = some || sm != 0u;
+                    hole = hole || hl != 0u;
+                    if (txa == txb && tya == tyb) {
+                        word = w;
+                        odist = o;
+                    }
+                }
+            }
+        some = some || (clo | chi | olo | ohi) != 0u;
+        // (a box at a tile's border: texel coordinates 0 or TS - 1)
+        const int risk = Q.risk;
+        if (risk && !hole && (risk == 2 || x0 >> SH != (x0 - 1) >> SH || xe >> SH != (xe + 1) >> SH ||
+                              y0 >> SH != (y0 - 1) >> SH || ye >> SH != (ye + 1) >> SH || txa != txb || tya != tyb)) {
+            hole = some = big = true;
+            word = nullptr;
+        }
+        full = !hole;
+        mixed = some && hole;
+        if (PROF) {
+            cand += (unsigned int)nn;
+            if (full) samples += (unsigned int)nn;
+        }
+    }
+    int cnt = full ? nn : 0;
+    bits = full ? (nn >= 64 ? ~0ull : (1ull << nn) - 1ull) : 0ull;
+    const unsigned int mx = __ballot_sync(0xffffffffu, mixed);
+    if (mx == 0u) return cnt;
+    // the samples of the mixed cells, nn each, over the lanes
+    const int rank = __popc(mx & ((1u << lane) - 1u));
+    if (lane == 0) Q.big = 0u;
+    __syncwarp();
+    if (mixed) {
+        if (big) {
+            const unsigned long long p = (unsigned long long)(uintptr_t)word;
+            clo = (uint32_t)p;
+            chi = (uint32_t)(p >> 32);
+            olo = (uint32_t)odist;
+        }
+        Q.cov[rank] = make_uint2(clo, chi);
+        Q.open[rank] = make_uint2(olo, ohi);
+        Q.ij[rank] = (uint32_t)I0 | ((uint32_t)J0 << 16);
+        Q.xy[rank] = (uint32_t)x0 | ((uint32_t)y0 << 16);
+        if (big) atomicOr(&Q.big, 1u << rank);
+    }
+    __syncwarp();
+    const int total = __popc(mx) * nn;
+    const uint32_t bigs = Q.big;
+    const float inv_n = __frcp_rn((float)n);
+    // sample base + lane: entry r, sample kk of its cell
+    const int step_r = 32 / nn, step_k = 32 - step_r * nn;
+    int r = lane / nn, kk = lane - r * nn;
+#pragma unroll 1
+    for (int base = 0; base < total; base += 32) {
+        bool hit = false;
+        if (base + lane < total) {
+            const int jj = fdiv(kk, n, inv_n), ii = kk - jj * n;
+            const uint32_t e = Q.ij[r], xy = Q.xy[r];
+            float d;
+            int ix, iy;
+            sample_texel(s, sample_row(s, (int)(e >> 16) + jj, p_over_n), (float)((int)(e & 0xFFFFu) + ii) + 0.5f,
+                         p_over_n, r_max, ix, iy, d);
+            const uint2 cv = Q.cov[r], op = Q.open[r];
+            bool look;
+            if (!((bigs >> r) & 1u)) {
+                const int bit = 8 * (iy - (int)(xy >> 16)) + ix - (int)(xy & 0xFFFFu);
+                hit = (((bit < 32 ? cv.x : cv.y) >> (bit & 31)) & 1u) != 0u;
+                look = !hit && (((bit < 32 ? op.x : op.y) >> (bit & 31)) & 1u) != 0u;
+            } else {
+                const uint32_t* w = reinterpret_cast<const uint32_t*>((uintptr_t)(((unsigned long long)cv.y << 32) | cv.x));
+                look = w == nullptr;
+                if (w) {
+                    const int k2 = (iy & (TS - 1)) * WPR + ((ix & (TS - 1)) >> 5);
+                    hit = ((w[k2] >> (ix & 31)) & 1u) != 0u;
+                    look = !hit && op.x && ((w[(int)op.x + k2] >> (ix & 31)) & 1u) != 0u;
+                }
+            }
+            if (PROF && !look) ++samples;
+            if (look)
+                hit = sample_shaded<TS, PROF>(B, tc, tiles_x, ix, iy, d, s.bias, plane, lp, u24, samples, h_samples,
+                                              pairs);
+            const int risk = Q.risk;
+            if (risk && hit && (risk == 2 || ((ix + 1) & (TS - 1)) < 2 || ((iy + 1) & (TS - 1)) < 2))
+                hit = sample_found<TS>(jobs, B, Q.entry, ix >> SH, iy >> SH, (int)(e & 0xFFFFu) + ii, (int)(e >> 16) + jj);
+        }
+        r += step_r;
+        kk += step_k;
+        if (kk >= nn) {
+            kk -= nn;
+            ++r;
+        }
+        const uint32_t ball = __ballot_sync(0xffffffffu, hit);
+        if (mixed) {
+            // this cell's samples among the 32: lanes [a, b)
+            const int a = max(rank * nn - base, 0), b = min((rank + 1) * nn - base, 32);
+            if (a < b) {
+                const uint32_t part = (ball >> a) & (b - a >= 32 ? 0xFFFFFFFFu : (1u << (b - a)) - 1u);
+                cnt += __popc(part);
+                const int sh = base + a - rank * nn;  // the first of them, within the cell
+                if (sh < 64) bits |= (unsigned long long)part << sh;
+            }
+        }
+    }
+    __syncwarp();  // the queue may be replaced
+    return cnt;
+}
+
+// The cells of a module some sample of which may read a texel of the box
+// [x0, x1] x [y0, y1]: first column | columns << 8 | first row << 16 | rows <<
+// 24 (the box's corners, two texels wider, mapped back onto the module; every
+// cell if the module is seen edge-on).  False if there are none.
+__device__ __forceinline__ bool cell_box(const ModStep& s, const ModuleDev& M, int x0, int x1, int y0, int y1,
+                                         uint32_t& cells)
+{
+    int ca = 0, cols = M.cu, ra = 0, rows = M.cv;
+    if (s.hs < FLT_MAX) {  // the module has a plane
+        const float inv = 1.f / ((s.tax * s.tby - s.tay * s.tbx) * M.pitch);
+        const float px0 = (float)(x0 - 2) - s.tx0, px1 = (float)(x1 + 3) - s.tx0;
+        const float py0 = (float)(y0 - 2) - s.ty0, py1 = (float)(y1 + 3) - s.ty0;
+        const float axl = s.tby * inv, axr = -s.tbx * inv, bxl = -s.tay * inv, bxr = s.tax * inv;
+        const float amin = fminf(axl * px0, axl * px1) + fminf(axr * py0, axr * py1);
+        const float amax = fmaxf(axl * px0, axl * px1) + fmaxf(axr * py0, axr * py1);
+        const float bmin = fminf(bxl * px0, bxl * px1) + fminf(bxr * py0, bxr * py1);
+        const float bmax = fmaxf(bxl * px0, bxl * px1) + fmaxf(bxr * py0, bxr * py1);
+        ca = (int)fminf(fmaxf(floorf(amin), 0.f), (float)M.cu);
+        ra = (int)fminf(fmaxf(floorf(bmin), 0.f), (float)M.cv);
+        cols = (int)fminf(fmaxf(ceilf(amax), 0.f), (float)M.cu) - ca;
+        rows = (int)fminf(fmaxf(ceilf(bmax), 0.f), (float)M.cv) - ra;
+    }
+    cells = (uint32_t)ca | ((uint32_t)cols << 8) | ((uint32_t)ra << 16) | ((uint32_t)rows << 24);
+    return cols > 0 && rows > 0;
+}
+
+// Add the covered and open texels of tile t of module m's range to a box.
+__device__ __forceinline__ void add_tile_box(const Buffers& B, const JobDev& J, int ls, int m, const TileRange& tr, int t,
+                                             int sh, int& x0, int& x1, int& y0, int& y1)
+{
+    const int wx = tr.tx1 - tr.tx0 + 1;
+    const int ty = tr.ty0 + t / wx, tx = tr.tx0 + t % wx;
+    const uint32_t state = B.t_cnt[J.te_base + (int64_t)ls * J.tiles_x * J.tiles_x + (int64_t)ty * J.tiles_x + tx];
+    if (state == kTileLit) return;
+    const int side = (1 << sh) - 1;
+    uint32_t box = (uint32_t)side << 8 | (uint32_t)side << 24;
+    if (state < kTileFullHeavy) {
+        const uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
+        box = rec[kRecBox + level_of(rec, rec[0], J.mods[m].plane)];
+    }
+    if (box == kBoxNone) return;
+    x0 = min(x0, (tx << sh) + (int)(box & 255u));
+    x1 = max(x1, (tx << sh) + (int)((box >> 8) & 255u));
+    y0 = min(y0, (ty << sh) + (int)((box >> 16) & 255u));
+    y1 = max(y1, (ty << sh) + (int)(box >> 24));
+}
 
 __global__ void __launch_bounds__(kPvThreads) k_pv(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs,
                                                    Buffers B)
 {
-    __shared__ uint32_t s_imin[kPvWarps][32 * kPvFastSub];
     const int64_t tot = W->tot_mod;
-    const int nj = W->n_jobs;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    uint32_t* imin = s_imin[wib];
-    const int64_t n_warps = (int64_t)gridDim.x * kPvWarps;
+    const int nj = W->n_jobs, sh = W->tile_sh;
+    // incomplete bins (pool overflow, the wave is rerun): the tiles have no state
+    const bool tiles_ok = !(B.ctr->overflow & 1u);
+    const int lane = threadIdx.x & 31;
+    // a warp takes bw items: 32, or fewer so that a small wave spreads over
+    // all warps
+    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int bw = 32;
     while (bw > 1 && n_warps * (bw >> 1) >= tot) bw >>= 1;
-    for (int64_t base = ((int64_t)blockIdx.x * kPvWarps + wib) * bw; base < tot; base += n_warps * bw) {
-        const int64_t item = base + lane;
-        const bool have = lane < bw && item < tot;
-        int j = 0, ls = 0, m = 0, ncell = 0, ns = 0, cell0 = 0;
-        int64_t msi = 0, cbase = 0;
-        const int* csub = nullptr;
+    for (int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * bw; base < tot; base += n_warps * bw) {
+        const int64_t item = lane < bw ? base + lane : tot;
+        bool list = false, touched = false;
+        int j = 0, ls = 0, m = 0;
+        uint32_t cells = 0u;  // the cells that a covered or open texel may reach (cell_box)
         bool lit = false;
         float beam = 0.f, diff = 0.f;
-        if (have) {
+        TileRange tr{};
+        int nt = 0;
+        if (item < tot) {
             j = job_of(nj, item, [&](int q) { return jobs[q].it_mod; });
             const JobDev& J = jobs[j];
             const int64_t li = item - J.it_mod;
             ls = (int)(li / J.n_mods);
             m = (int)(li - (int64_t)ls * J.n_mods);
-            msi = J.ms_base + li;
+            const int64_t msi = J.ms_base + li;
             const LightParams& lp = B.lp[J.js_base + ls];
             const ModuleDev& M = J.mods[m];
-            ncell = M.cu * M.cv;
-            ns = M.n_sub;
-            cell0 = M.cell_base;
-            cbase = J.cs_base + (int64_t)ls * J.n_cells + cell0;
-            csub = J.lay_sub + J.lay_off[M.layout];
             lit = lp.valid != 0;
+            list = lit && (J.fdiff || M.n_sub > kPvFastSub);
             if (lit) {
-                const ModStep& s = B.ms[msi];
+                const ModStep s = B.ms[msi];
                 beam = lp.dni * fmaxf(0.f, s.cosi);
                 diff = lp.dhi * (1.f + s.nz) * 0.5f;
+                tr = module_tiles(s, M, J.R, sh);
+                nt = tiles_ok ? (tr.tx1 - tr.tx0 + 1) * (tr.ty1 - tr.ty0 + 1) : 0;
             }
         }
-        if (__reduce_max_sync(0xffffffffu, ns) > kPvFastSub) {
-            for (int q = 0; q < bw && base + q < tot; ++q) pv_module_warp(jobs, nj, base + q, B, imin);
-            continue;
+        // box of the texels covered or open in the module's tiles: by its lane,
+        // or by the warp for a module over many tiles
+        int x0 = INT_MAX, x1 = -1, y0 = INT_MAX, y1 = -1;
+        for (int t = 0; t < (nt <= kPvTiles ? nt : 0); ++t)
+            add_tile_box(B, jobs[j], ls, m, tr, t, sh, x0, x1, y0, y1);
+#pragma unroll 1
+        for (unsigned int many = __ballot_sync(0xffffffffu, nt > kPvTiles); many; many &= many - 1u) {
+            const int q = __ffs((int)many) - 1;
+            const int jq = __shfl_sync(0xffffffffu, j, q), lq = __shfl_sync(0xffffffffu, ls, q);
+            const int mq = __shfl_sync(0xffffffffu, m, q), nq = __shfl_sync(0xffffffffu, nt, q);
+            TileRange tq;
+            tq.tx0 = __shfl_sync(0xffffffffu, tr.tx0, q); tq.tx1 = __shfl_sync(0xffffffffu, tr.tx1, q);
+            tq.ty0 = __shfl_sync(0xffffffffu, tr.ty0, q);
+            int a0 = INT_MAX, a1 = -1, b0 = INT_MAX, b1 = -1;
+            for (int t = lane; t < nq; t += 32) add_tile_box(B, jobs[jq], lq, mq, tq, t, sh, a0, a1, b0, b1);
+            a0 = __reduce_min_sync(0xffffffffu, a0); a1 = __reduce_max_sync(0xffffffffu, a1);
+            b0 = __reduce_min_sync(0xffffffffu, b0); b1 = __reduce_max_sync(0xffffffffu, b1);
+            if (lane == q) { x0 = a0; x1 = a1; y0 = b0; y1 = b1; }
         }
-        uint32_t* im = imin + lane * kPvFastSub;
-        for (int k = 0; k < kPvFastSub; ++k) im[k] = 0x7F800000u;  // +inf
-        if (bw == 32) {
-            // a full batch: each lane walks its own module's cells (their
-            // tallies are one byte each, consecutive per module: the warp's
-            // lanes share the few cache lines of their modules), the
-            // substring minima in its slice of shared memory
-            if (have) {
-                const JobDev& J = jobs[j];
-                const int64_t row = (int64_t)(J.out_row0 + ls);
-                if (!lit) {
-                    for (int c = 0; c < ncell; ++c) {
-                        tally_set(B.cs_cnt, cbase + c, 0u);
-                        if (J.out_counts) J.out_counts[row * J.out_cstride + cell0 + c] = 0;
-                        if (J.out_bits) J.out_bits[row * J.out_cstride + cell0 + c] = 0ull;
-                    }
-                } else {
-                    const float* fd = diffuse_row(J, ls);
-                    const float inv_nn = 1.f / J.nn;
-                    for (int c = 0; c < ncell; ++c) {
-                        const uint32_t cnt = tally_get(B.cs_cnt, cbase + c);
-                        if (J.out_counts) J.out_counts[row * J.out_cstride + cell0 + c] = (uint8_t)cnt;
-                        if (J.out_bits) J.out_bits[row * J.out_cstride + cell0 + c] = B.cs_bits[cbase + c];
-                        const float gd = fd ? diff * (1.f - fd[cell0 + c]) : diff;
-                        const float G = beam * (1.f - cnt * inv_nn) + gd;
-                        const uint32_t I = __float_as_uint(J.i_ref * G * 1e-3f);  // I >= 0: uint order = float order
-                        const int k = csub[c];
-                        if (I < im[k]) im[k] = I;
-                    }
-                }
-            }
-        } else {
-            // a short batch (a wave too small to fill the grid): the lanes
-            // take the cells of one item after another, loads of 32 cells at
-            // a time issued together before the minima are taken
-            __syncwarp();
-            for (unsigned int act = __ballot_sync(0xffffffffu, have); act; act &= act - 1u) {
-                const int q = __ffs(act) - 1;
-                const JobDev& J = jobs[__shfl_sync(0xffffffffu, j, q)];
-                const int nc = __shfl_sync(0xffffffffu, ncell, q);
-                const int c0 = __shfl_sync(0xffffffffu, cell0, q);
-                const int64_t cb = __shfl_sync(0xffffffffu, cbase, q);
-                const int* cs = reinterpret_cast<const int*>(
-                    __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(csub), q));
-                const int lsq = __shfl_sync(0xffffffffu, ls, q);
-                const int64_t row = (int64_t)(J.out_row0 + lsq);
-                const float* fd = diffuse_row(J, lsq);
-                const bool litq = __shfl_sync(0xffffffffu, (int)lit, q) != 0;
-                const float bq = __shfl_sync(0xffffffffu, beam, q), dq = __shfl_sync(0xffffffffu, diff, q);
-                const float inv_nn = 1.f / J.nn;
-                uint32_t* iq = imin + q * kPvFastSub;
-                if (!litq) {
-                    for (int c = lane; c < nc; c += 32) {
-                        tally_set(B.cs_cnt, cb + c, 0u);
-                        if (J.out_counts) J.out_counts[row * J.out_cstride + c0 + c] = 0;
-                        if (J.out_bits) J.out_bits[row * J.out_cstride + c0 + c] = 0ull;
-                    }
-                    continue;
-                }
-                for (int cr = lane; cr < nc; cr += 32 * kPvUnroll) {
-                    uint32_t cnt[kPvUnroll];
-                    int sub[kPvUnroll];
-#pragma unroll
-                    for (int u = 0; u < kPvUnroll; ++u) {
-                        const int c = cr + 32 * u;
-                        cnt[u] = c < nc ? tally_get(B.cs_cnt, cb + c) : 0u;
-                        sub[u] = c < nc ? cs[c] : 0;
-                    }
-#pragma unroll
-                    for (int u = 0; u < kPvUnroll; ++u) {
-                        const int c = cr + 32 * u;
-                        if (c >= nc) continue;
-                        if (J.out_counts) J.out_counts[row * J.out_cstride + c0 + c] = (uint8_t)cnt[u];
-                        if (J.out_bits) J.out_bits[row * J.out_cstride + c0 + c] = B.cs_bits[cb + c];
-                        const float gd = fd ? dq * (1.f - fd[c0 + c]) : dq;
-                        const float G = bq * (1.f - cnt[u] * inv_nn) + gd;
-                        const float I = J.i_ref * G * 1e-3f;
-                        atomicMin(&iq[sub[u]], __float_as_uint(I));  // I >= 0: uint order = float order
-                    }
-                }
-            }
-        }
-        __syncwarp();
-        if (have) {
+        if (item < tot) {
             const JobDev& J = jobs[j];
-            if (!lit) {
-                B.ms_p[msi] = 0.f;
-                B.ms_pu[msi] = 0.f;
-                B.ms_beam[msi] = 0.f;
-            } else {
-                const ModuleDev& M = J.mods[m];
-                if (J.n_str) {  // substring currents for the series-string model (k_string)
-                    float* ss = B.ss_i + J.ss_base + (int64_t)ls * J.n_sub_tot + J.sub_base[m];
-                    for (int k = 0; k < ns; ++k) ss[k] = __uint_as_float(im[k]);
-                    B.ms_iu[msi] = J.i_ref * (beam + diff) * 1e-3f;
-                }
-                const int* nk = J.lay_nk + J.lay_nk_off[M.layout];
+            const ModuleDev& M = J.mods[m];
+            const int64_t msi = J.ms_base + (int64_t)ls * J.n_mods + m;
+            if (x1 >= 0) touched = cell_box(B.ms[msi], M, x0, x1, y0, y1, cells);
+            const int ns = M.n_sub;
+            list = list || touched;
+            if (!list) {
+                // every substring carries the module's one current, and the
+                // voltage at it is the sum over all of them (k_cells' terms,
+                // rounded as there)
                 float best = 0.f, vsum = 0.f;
-                for (int k = 0; k < ns; ++k) {
-                    const float ik = __uint_as_float(im[k]);
+                if (lit) {
+                    const float I = J.i_ref * (beam * 1.f + diff) * 1e-3f;
+                    const int* nk = J.lay_nk + J.lay_nk_off[M.layout];
                     float volt = 0.f;
-                    for (int q = 0; q < ns; ++q) volt += __uint_as_float(im[q]) >= ik ? nk[q] * J.v_cell : -J.v_diode;
-                    best = fmaxf(best, ik * volt);
-                    vsum += nk[k] * J.v_cell;
+#pragma unroll 1
+                    for (int k = 0; k < ns; ++k) {
+                        volt = __fadd_rn(volt, __fmul_rn((float)nk[k], J.v_cell));
+                        vsum += nk[k] * J.v_cell;
+                    }
+                    best = fmaxf(0.f, I * volt);
+                    if (J.n_str) {  // substring currents for the series-string model (k_string)
+                        float* ss = B.ss_i + J.ss_base + (int64_t)ls * J.n_sub_tot + J.sub_base[m];
+                        for (int k = 0; k < ns; ++k) ss[k] = I;
+                        B.ms_iu[msi] = J.i_ref * (beam + diff) * 1e-3f;
+                    }
+                    vsum = J.i_ref * (beam + diff) * 1e-3f * vsum;
                 }
                 B.ms_p[msi] = best;
-                B.ms_pu[msi] = J.i_ref * (beam + diff) * 1e-3f * vsum;
+                B.ms_pu[msi] = vsum;
                 B.ms_beam[msi] = beam;
             }
         }
-        __syncwarp();  // the warp's minima may be reset
+        const unsigned int bal = __ballot_sync(0xffffffffu, list);
+        unsigned int pos = 0;
+        if (lane == 0 && bal) pos = atomicAdd(&B.ctr->n_touch, (unsigned int)__popc(bal));
+        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (list) B.touch[pos] = make_uint4((uint32_t)j | (touched ? 1u << 31 : 0u), (uint32_t)ls, (uint32_t)m, cells);
+    }
+}
+
+template <int TS, bool PROF>
+__global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_cells(const WaveDev* __restrict__ W,
+                                                              const JobDev* __restrict__ jobs, Buffers B)
+{
+    __shared__ CellQueue s_queue[kCellWarps];
+    __shared__ uint32_t s_imin[kCellWarps][kMaxSub];
+    unsigned int p_cand = 0, p_samples = 0, p_hsamples = 0, p_pairs = 0;
+    const unsigned int n_touch = B.ctr->n_touch;
+    const int u24 = W->depth_u24;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // few modules: the block's warps share one module's cells
+    const bool shared = n_touch <= gridDim.x * (kCellWarps / 2);
+    uint32_t* imin = s_imin[shared ? 0 : wib];
+    CellQueue& Q = s_queue[wib];
+    const unsigned int e0 = shared ? blockIdx.x : blockIdx.x * kCellWarps + wib;
+    const unsigned int e_stride = shared ? gridDim.x : gridDim.x * kCellWarps;
+#pragma unroll 1
+    for (unsigned int e = e0; e < n_touch; e += e_stride) {
+        const uint4 entry = B.touch[e];
+        const bool touched = (entry.x >> 31) != 0u;
+        const JobDev& J = jobs[entry.x & 0x7FFFFFFFu];
+        const int ls = (int)entry.y, m = (int)entry.z;
+        const int64_t msi = J.ms_base + (int64_t)ls * J.n_mods + m;
+        const LightParams& lp = B.lp[J.js_base + ls];
+        const ModuleDev& M = J.mods[m];
+        const ModStep& s = B.ms[msi];
+        const bool lit = lp.valid != 0;
+        const int c0 = M.cell_base, ns = M.n_sub, cu = M.cu, plane = M.plane;
+        const float p_over_n = __fdiv_rn(M.pitch, (float)J.n);
+        if (lane == 0) {
+            Q.risk = find_risk(s, cu * M.pitch, M.cv * M.pitch, 1.f / p_over_n, J.R);
+            Q.entry = e;
+        }
+        __syncwarp();
+        const float beam = lit ? lp.dni * fmaxf(0.f, s.cosi) : 0.f;
+        const float diff = lit ? lp.dhi * (1.f + s.nz) * 0.5f : 0.f;
+        const uint32_t* tc = B.t_cnt + J.te_base + (int64_t)ls * J.tiles_x * J.tiles_x;
+        const int64_t cbase = J.cs_base + (int64_t)ls * J.n_cells + c0;
+        const int64_t row = (int64_t)(J.out_row0 + ls) * J.out_cstride + c0;
+        const float* fd = diffuse_row(J, ls);
+        const int* csub = J.lay_sub + J.lay_off[M.layout];
+        const float inv_nn = 1.f / J.nn;
+        const bool few = ns <= kPvFastSub;
+        // without a diffuse term per cell only the cells that a covered or open
+        // texel reaches are looked at: the others carry the unshaded current,
+        // which no cell exceeds, so every substring's minimum starts from it
+        const bool every = fd != nullptr;
+        uint32_t mine = 0x7F800000u;  // +inf; few substrings: lane k keeps substring k's minimum
+        if (!every && lit) mine = __float_as_uint(J.i_ref * (beam * 1.f + diff) * 1e-3f);
+        const int* nk = J.lay_nk + J.lay_nk_off[M.layout];
+        const int nk_l = few && lane < ns ? nk[lane] : 0;
+        if (shared) {
+            if (wib == 0)
+                for (int k = lane; k < ns; k += 32) imin[k] = mine;
+            __syncthreads();
+        } else if (!few) {
+            for (int k = lane; k < ns; k += 32) imin[k] = mine;
+            __syncwarp();
+        }
+        int ca = 0, cols = cu, ra = 0, rows = M.cv;
+        if (!every) {
+            ca = (int)(entry.w & 255u);
+            cols = (int)((entry.w >> 8) & 255u);
+            ra = (int)((entry.w >> 16) & 255u);
+            rows = touched ? (int)(entry.w >> 24) : 0;
+        }
+        const int count = cols * rows;
+        const float inv_cols = __frcp_rn((float)max(cols, 1));
+        // cells at a time, one per lane
+        const int per = shared ? min((count + kCellWarps - 1) / kCellWarps, 32) : 32;
+#pragma unroll 1
+        for (int cr = shared ? wib * per : 0; cr < count; cr += shared ? kCellWarps * per : 32) {
+            const bool have = lane < per && cr + lane < count;
+            const int rr = fdiv(cr + lane, max(cols, 1), inv_cols);
+            const int c = (ra + rr) * cu + ca + cr + lane - rr * cols;
+            unsigned long long bits = 0ull;
+            int cnt = 0;
+            if (touched)
+                cnt = cell_shaded<TS, PROF>(B, J, s, cu, plane, p_over_n, lp, u24, tc, c, have, jobs, Q, bits, p_cand,
+                                            p_samples, p_hsamples, p_pairs);
+            uint32_t cur = 0x7F800000u;
+            int sub = -1;
+            if (have) {
+                if (J.kahan_cell) tally_set(B.cs_cnt, cbase + c, (uint32_t)cnt);
+                if (J.out_counts) J.out_counts[row + c] = (uint8_t)cnt;
+                if (J.out_bits) J.out_bits[row + c] = bits;
+                const float gd = fd ? diff * (1.f - fd[c0 + c]) : diff;
+                const float G = beam * (1.f - (uint32_t)cnt * inv_nn) + gd;
+                cur = __float_as_uint(J.i_ref * G * 1e-3f);  // I >= 0: uint order = float order
+                sub = csub[c];
+            }
+            if (!lit) continue;
+            if (few) {
+#pragma unroll 1
+                for (int k = 0; k < ns; ++k) {
+                    const uint32_t v = __reduce_min_sync(0xffffffffu, sub == k ? cur : 0x7F800000u);
+                    if (lane == k) mine = min(mine, v);
+                }
+            } else if (have) {
+                atomicMin(&imin[sub], cur);
+            }
+        }
+        if (shared) {
+            if (few && lane < ns) atomicMin(&imin[lane], mine);
+            __syncthreads();
+            if (few && lane < ns) mine = imin[lane];
+        } else {
+            __syncwarp();
+        }
+        float best = 0.f, vsum = 0.f;
+        if (lit && (!shared || wib == 0)) {
+            float* ss = J.n_str ? B.ss_i + J.ss_base + (int64_t)ls * J.n_sub_tot + J.sub_base[m] : nullptr;
+            if (few) {
+                // lane k < ns takes candidate current k
+                const float ik = __uint_as_float(mine);
+                float volt = 0.f;
+#pragma unroll 1
+                for (int q = 0; q < ns; ++q) {
+                    const float vq = __fmul_rn((float)__shfl_sync(0xffffffffu, nk_l, q), J.v_cell);
+                    volt += __uint_as_float(__shfl_sync(0xffffffffu, mine, q)) >= ik ? vq : -J.v_diode;
+                    vsum += nk[q] * J.v_cell;
+                }
+                if (lane < ns) best = fmaxf(0.f, ik * volt);
+                if (ss && lane < ns) ss[lane] = ik;
+            } else {
+                for (int k = lane; k < ns; k += 32) {
+                    const float ik = __uint_as_float(imin[k]);
+                    float volt = 0.f;
+#pragma unroll 1
+                    for (int q = 0; q < ns; ++q)
+                        volt += __uint_as_float(imin[q]) >= ik ? nk[q] * J.v_cell : -J.v_diode;
+                    best = fmaxf(best, ik * volt);
+                    vsum += nk[k] * J.v_cell;
+                    if (ss) ss[k] = ik;
+                }
+#pragma unroll
+                for (int off = 16; off; off >>= 1) vsum += __shfl_xor_sync(0xffffffffu, vsum, off);
+            }
+            best = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best)));  // best >= 0
+            if (ss && lane == 0) B.ms_iu[msi] = J.i_ref * (beam + diff) * 1e-3f;
+            vsum = J.i_ref * (beam + diff) * 1e-3f * vsum;
+        }
+        if (lane == 0 && (!shared || wib == 0)) {
+            B.ms_p[msi] = best;
+            B.ms_pu[msi] = vsum;
+            B.ms_beam[msi] = beam;
+        }
+        if (shared) __syncthreads();  // the minima may be reset
+        else __syncwarp();
+    }
+    if (PROF) {
+        flush_profile(B, p_samples, 0u, 0u, 0u);
+        flush_profile2(B, p_cand, 0u, 0u, 0u, p_pairs);
+        flush_heavy(B, p_hsamples, 0u, 0u);
     }
 }
 
@@ -2879,7 +3694,7 @@ __global__ void __launch_bounds__(kPvThreads) k_sample(const WaveDev* __restrict
                 sample_texel(s, sample_row(s, cv_ * n + jj, p_over_n), (float)I + 0.5f, p_over_n,
                              (float)(R - 1), ix, iy, d);
                 const int64_t te = te0 + (int64_t)(iy >> sh) * J.tiles_x + (ix >> sh);
-                if (B.t_cnt[te] != 0u) {
+                if (J.tiles_x > 0 && B.t_cnt[te] != 0u) {
                     const uint32_t slot = B.t_slot[te];
                     if (slot < map_cap) {
                         const uint32_t key = B.map[((size_t)slot << (2 * sh)) + ((iy & tmask) << sh) + (ix & tmask)];
@@ -3154,6 +3969,11 @@ __global__ void __launch_bounds__(256) k_epilogue(const WaveDev* __restrict__ W,
     const int64_t tot = W->tot_epi;
     const int nj = W->n_jobs;
     const int lane = threadIdx.x & 31;
+    if (W->fused && blockIdx.x == 0 && threadIdx.x == 0) {  // the tiles' records are all allocated by now
+        Counters* c = B.ctr;
+        if (c->cov_next > c->need_cov) c->need_cov = c->cov_next;
+        if (c->cov_next > (unsigned long long)W->cov_cap) c->overflow |= 16u;
+    }
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t item = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; item < tot; item += n_warps) {
         const int j = job_of(nj, item, [&](int q) { return jobs[q].it_epi; });
@@ -3375,10 +4195,14 @@ constexpr int tile_blocks() { return TS == 128 ? 2 : 4; }
 template <int TS, bool PROF>
 static cudaError_t allow_tile_smem()
 {
-    const int bytes = (int)sizeof(TileSm<TS>);
-    cudaError_t e = cudaFuncSetAttribute(k_raster_test<TS, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(k_raster_test<TS, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(HeavySm<TS>));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_raster_map<TS, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        e = cudaFuncSetAttribute(k_raster_map<TS, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(TileSm<TS>));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tile_warp<TS, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kTileWarps * sizeof(WarpSm<TS>)));
     return e;
 }
 
@@ -3398,15 +4222,22 @@ template <int TS, bool PROF>
 static void launch_tile_kernels(const WaveDev* W, const JobDev* d_jobs, const Buffers& b, const LaunchCfg& cfg)
 {
     const int sm = cfg.sm_count;
-    const size_t tsm = sizeof(TileSm<TS>);
     if (cfg.fused) {
-        k_tile_warp<TS, PROF><<<sm * 6, kTileWarps * 32, 0, cfg.stream>>>(W, d_jobs, b);
+        k_tile_warp<TS, PROF><<<sm * kTileBlocks, kTileWarps * 32, kTileWarps * sizeof(WarpSm<TS>), cfg.stream>>>(
+            W, d_jobs, b);
         if (cfg.ev) cudaEventRecord(cfg.ev[3], cfg.stream);
-        k_raster_test<TS, PROF><<<sm * (TS == 32 ? HeavyCfg<TS>::min_blocks : tile_blocks<TS>()), HeavyCfg<TS>::threads,
-                                   tsm, cfg.stream>>>(W, d_jobs, b);
+        k_raster_test<TS, PROF><<<sm * HeavyCfg<TS>::min_blocks, HeavyCfg<TS>::threads, sizeof(HeavySm<TS>),
+                                  cfg.stream>>>(W, d_jobs, b);
+        if (cfg.ev) cudaEventRecord(cfg.ev[4], cfg.stream);
+        k_pv<<<sm * 16, kPvThreads, 0, cfg.stream>>>(W, d_jobs, b);
+        k_cells<TS, PROF><<<sm * kCellBlocks, kCellWarps * 32, 0, cfg.stream>>>(W, d_jobs, b);
     } else {
-        k_raster_map<TS, PROF><<<sm * tile_blocks<TS>(), 256, tsm, cfg.stream>>>(W, d_jobs, b);
-        if (cfg.ev) cudaEventRecord(cfg.ev[3], cfg.stream);
+        k_raster_map<TS, PROF><<<sm * tile_blocks<TS>(), 256, sizeof(TileSm<TS>), cfg.stream>>>(W, d_jobs, b);
+        if (cfg.ev) {
+            cudaEventRecord(cfg.ev[3], cfg.stream);
+            cudaEventRecord(cfg.ev[4], cfg.stream);
+        }
+        k_sample<<<sm * 16, kPvThreads, 0, cfg.stream>>>(W, d_jobs, b);
     }
 }
 
@@ -3418,7 +4249,7 @@ cudaError_t launch_wave(const WaveDev* d_wave, const JobDev* d_jobs, const Buffe
     const int sm = cfg.sm_count;
     (void)tot_te_host;
     if (cfg.ev) cudaEventRecord(cfg.ev[0], st);
-    k_clear<<<sm * 8, 256, 0, st>>>(W, b);
+    k_clear<<<sm * 8, 256, 0, st>>>(W, d_jobs, b);
     k_window<<<sm * 8, kWinPerItem, 0, st>>>(W, d_jobs, b);
     k_light<<<sm, 128, 0, st>>>(W, d_jobs, b);
     k_modsetup<<<sm * 8, 256, 0, st>>>(W, d_jobs, b);
@@ -3441,9 +4272,6 @@ cudaError_t launch_wave(const WaveDev* d_wave, const JobDev* d_jobs, const Buffe
         if (cfg.profile) launch_tile_kernels<128, true>(W, d_jobs, b, cfg);
         else launch_tile_kernels<128, false>(W, d_jobs, b, cfg);
     }
-    if (cfg.ev) cudaEventRecord(cfg.ev[4], st);
-    if (cfg.fused) k_pv<<<sm * 32, kPvThreads, 0, st>>>(W, d_jobs, b);
-    else k_sample<<<sm * 16, kPvThreads, 0, st>>>(W, d_jobs, b);
     if (cfg.extras & 1) k_string<<<sm * 4, 256, 0, st>>>(W, d_jobs, b);
     if (cfg.extras & 4) k_array<<<sm * 4, kArrayWarps * 32, 0, st>>>(W, d_jobs, b);
     if (cfg.extras & 2) {

@@ -47,16 +47,19 @@ struct LightParams {
     int32_t pad;
 };
 
-// One module at one step in texel space (48 bytes): a point a*U + b*V of the
+// One module at one step in texel space (64 bytes): a point a*U + b*V of the
 // module (a, b in metres) maps to texel coordinates
 // (tx0 + a*tax + b*tbx, ty0 + a*tay + b*tby) and depth d0 + a*da + b*db.
-struct ModStep {
+struct __align__(16) ModStep {
     float tx0, ty0, d0;
     float tax, tay, da;
     float tbx, tby, db;
     float cosi;   // cosine of incidence on the front face
     float bias;   // depth bias, metres
     float nz;     // z of the front normal (cos of the tilt)
+    float pa, pb; // depth of its plane per texel in x and y
+    float hs;     // bound on |a sample's depth - the plane's at its texel's centre| (inf: no plane)
+    float pad;
 };
 
 struct JobDev {
@@ -161,8 +164,7 @@ struct WaveDev {
     int32_t n_jobs;
     int32_t tile_sh;    // log2 of the tile side
     int32_t depth_u24;
-    int32_t fused;      // 1: depth tests inside the tile CTA; 0: map in HBM + gather kernel
-    int32_t want_bits;  // per-sample flags requested by some job of the wave
+    int32_t fused;      // 1: coverage bits per tile; 0: map in HBM + gather kernel
     int32_t profile;    // count work (texel visits, sample tests) into Counters
     int64_t tot_js, tot_te, tot_ms, tot_cs;
     int64_t tot_win, tot_mod, tot_tri, tot_epi;  // tot_tri: (group of 32 meshlets, step) warp items
@@ -170,16 +172,19 @@ struct WaveDev {
     int64_t tot_heat;                            // heat-map bins over the jobs
     int64_t tot_sa;                              // (step, array) entries
     int64_t bin_cap, map_cap_tiles, big_cap, recv_cap;
+    int64_t cov_cap;  // 16-byte units of the tile record pool
 };
 
 struct Counters {
     unsigned int n_big;
     unsigned int n_nonempty;
     unsigned int raster_next;
-    unsigned int overflow;  // bit 0 bins, bit 1 map tiles, bit 2 big list, bit 3 receivers
+    unsigned int overflow;  // bit 0 bins, bit 1 map tiles, bit 2 big list, bit 3 receivers, bit 4 tile records
     unsigned int n_heavy;     // tiles k_tile_warp hands to k_raster_test
     unsigned long long n_pairs;  // (tile, triangle) pairs appended by the binning kernels
     unsigned int heavy_next;  // k_raster_test's work counter
+    unsigned int n_touch;     // modules listed for k_cells
+    unsigned int n_first, n_rest;  // fused path: tiles listed from the front and from the end of nonempty
     unsigned long long tot_bins;
     unsigned long long tot_recv;
     unsigned long long need_recv;
@@ -188,21 +193,24 @@ struct Counters {
     unsigned long long need_bins;    // max over waves of the bins a wave needed
     unsigned long long need_tiles;   // max over waves of the map tiles a wave needed
     unsigned long long need_big;
+    unsigned long long cov_next;     // 16-byte units of tile records allocated
+    unsigned long long need_cov;     // max over waves
     // work counters, filled when WaveDev::profile is set
-    unsigned long long prof_samples;   // sample depth tests in rasterised tiles
-    unsigned long long prof_visits;    // texel coverage tests
-    unsigned long long prof_writes;    // covered texels (depth atomicMin)
-    unsigned long long prof_culled;    // (triangle, tile) pairs skipped by the receiver-plane test
-    unsigned long long prof_cand;      // receiver samples enumerated (marking and testing passes)
+    // (fused path / map path)
+    unsigned long long prof_samples;   // samples decided in tiles that are not lit / depth tests in rasterised tiles
+    unsigned long long prof_visits;    // texels drawn as coverage / texel coverage tests
+    unsigned long long prof_writes;    // those and the texels compared with a plane / covered texels (atomicMin)
+    unsigned long long prof_culled;    // (triangle, tile) pairs behind every receiver plane
+    unsigned long long prof_cand;      // samples of the cells looked at / samples enumerated (marking and testing)
     unsigned long long prof_tiles;     // tiles rasterised
     unsigned long long prof_dense;     // of which rasterised densely
     unsigned long long prof_tris;      // (triangle, tile) pairs set up
-    unsigned long long prof_stiles;    // tiles tested sample by sample (not rasterised)
-    unsigned long long prof_pairs;     // (sample, triangle) coverage tests of the sample-driven test
+    unsigned long long prof_stiles;    // tiles in which nothing was drawn
+    unsigned long long prof_pairs;     // (sample, open triangle) depth tests
     unsigned long long prof_h_samples;  // of prof_samples, prof_writes and prof_tiles: the share of the
     unsigned long long prof_h_writes;   //   kernel that takes the heavy tiles (one block per tile)
     unsigned long long prof_h_tiles;
-    unsigned long long prof_heavy_why[3];  // heavy because of: receivers, binned triangles, kept triangles
+    unsigned long long prof_heavy_why[3];  // heavy because of: receivers, binned triangles, kept or open triangles
 };
 
 // Scratch and pools, sized by the host for the largest wave.
@@ -222,25 +230,26 @@ struct Buffers {
     float* js_p;             // [tot_js]  the generator's P_mpp per step (heat map)
     float* js_pu;            // [tot_js]
     int32_t* js_bin;         // [tot_js]  sky bin of the step's sun, -1 below the horizon
-    uint32_t* cs_cnt;        // [(tot_cs + 3) / 4]  shaded samples per (step, cell): one byte each (a count
-                             //  is at most n^2 <= 225), four to a word for the tile kernels' atomics
-    unsigned long long* cs_bits;  // [tot_cs] shaded flags per (step, cell), fused path with flags requested
+    uint32_t* cs_cnt;        // [(tot_cs + 3) / 4]  shaded samples per (step, cell), one byte each (a count is
+                             //  at most n^2 <= 225), when the per-cell beam loss is wanted
     uint32_t* t_far;         // [tot_te]  far-plane key of the tile (0 = no sample)
-    uint32_t* t_cnt;         // [tot_te]  triangles binned
+    uint32_t* t_cnt;         // [tot_te]  triangles binned; fused path, after the tile kernels: the tile's state
     uint32_t* t_off;         // [tot_te]
     uint32_t* t_cur;         // [tot_te]
     uint32_t* t_slot;        // [tot_te]  index among the wave's non-empty tiles (= map slot)
     uint32_t* t_rcnt;        // [tot_te]  receiver modules touching the tile
     uint32_t* t_plane;       // [tot_te]  plane group of every receiver of the tile, or kPlaneMixed
-    uint32_t* t_roff;        // [tot_te]
+    uint32_t* t_roff;        // [tot_te]  first receiver in recv (fused path, one plane group: one of its modules)
     uint32_t* t_rcur;        // [tot_te]
     uint32_t* nonempty;      // [tot_te]
     uint32_t* heavy;         // [tot_te]  tiles listed for the CTA-per-tile kernel (fused path)
     uint32_t* bins;          // [bin_cap]   triangle ids
     uint2* pairs;            // [bin_cap]   (tile entry, triangle) pairs in binning order
     uint32_t* recv;          // [recv_cap]  receiver module ids
+    uint4* touch;            // [tot_ms]  modules listed for k_cells: job, step, module, 1 if a tile of it is not lit
     uint32_t* map;           // [map_cap_tiles << (2 * tile_sh)]  (map path)
     uint2* big;              // [big_cap]  (triangle, js)
+    uint32_t* cov;           // [cov_cap * 4]  tile records: coverage bits per plane (fused path)
     unsigned long long* block_sums;  // scan partials, 3 per scan tile
     Counters* ctr;
 };
@@ -249,7 +258,7 @@ struct Buffers {
 struct LaunchCfg {
     int sm_count;
     int tile;     // 32, 64 or 128
-    int fused;    // 1: k_raster_test + k_pv; 0: k_raster_map + k_sample
+    int fused;    // 1: k_tile_warp, k_raster_test, k_pv, k_cells; 0: k_raster_map, k_sample
     int profile;  // counting kernels
     cudaStream_t stream;
     cudaEvent_t* ev;  // NULL, or kStages + 1 events recorded at the stage boundaries of the wave
@@ -257,7 +266,7 @@ struct LaunchCfg {
 };
 
 constexpr int kStages = 6;  // setup, bin, tile (warp per tile / map raster), heavy tiles, pv/sample, epilogue
-constexpr int kLaunchesPerWave = 15;     // kernels launch_wave starts (fused path), plus 1 with
+constexpr int kLaunchesPerWave = 16;     // kernels launch_wave starts (fused path), plus 1 with
 constexpr int kLaunchesPerWaveMap = 14;  // strings, 2 with the sky map, 1 with arrays; (map path)
 constexpr int kMaxArraySub = 512;        // bypass substrings an array of parallel strings may hold
 
