@@ -410,12 +410,23 @@ extern "C" int pv3d_scene_load(pv3d_ctx* c, const float* xyz, int64_t n_verts, c
             boxes[2 * m] = make_float4(blo[0], blo[1], blo[2], 0.f);
             boxes[2 * m + 1] = make_float4(bhi[0], bhi[1], bhi[2], 0.f);
         }
+        // and the box of each 32 meshlets after theirs (whole groups only)
+        for (int32_t m = 0; m + 32 <= s.n_ml; m += 32) {
+            float4 glo = boxes[2 * m], ghi = boxes[2 * m + 1];
+            for (int32_t q = m + 1; q < m + 32; ++q) {
+                const float4 a = boxes[2 * q], b = boxes[2 * q + 1];
+                glo = make_float4(std::min(glo.x, a.x), std::min(glo.y, a.y), std::min(glo.z, a.z), 0.f);
+                ghi = make_float4(std::max(ghi.x, b.x), std::max(ghi.y, b.y), std::max(ghi.z, b.z), 0.f);
+            }
+            boxes.push_back(glo);
+            boxes.push_back(ghi);
+        }
         int rc0 = upload(c, &s.d_ml, boxes.data(), boxes.size());
         if (rc0) return rc0;
     }
     int rc = upload(c, &s.d_tri, tv.data(), tv.size());
     if (rc) return rc;
-    s.bytes = std::max<size_t>(tv.size() * sizeof(float4), 16) + (size_t)s.n_ml * 32;
+    s.bytes = std::max<size_t>(tv.size() * sizeof(float4), 16) + (size_t)(s.n_ml + s.n_ml / 32) * 32;
     uint32_t id = c->next_id++;
     c->scenes[id] = s;
     *scene_id = id;
@@ -1130,7 +1141,7 @@ static WaveDev pack_wave(std::vector<JobDev>& jobs, size_t first, size_t last, i
         W.tot_cs += (int64_t)J.k * J.n_cells;
         W.tot_win += (int64_t)J.k * groups;
         W.tot_mod += (int64_t)J.k * J.n_mods;
-        W.tot_tri += (((int64_t)J.n_ml + J.n_oml + (J.n_mtris + 31) / 32 + 31) / 32) * J.k;  // groups of 32 meshlets
+        W.tot_tri += (((int64_t)J.n_ml + J.n_oml + (J.n_mtris + 31) / 32 + 1023) / 1024) * J.k;  // 32 groups of 32 meshlets
         W.tot_epi += (J.kahan_cell ? (int64_t)J.n_cells : 0) + J.n_mods + J.n_str + J.n_arr;
         W.tot_sa += (int64_t)J.k * J.n_arr;
         W.tot_ss += (int64_t)J.k * (J.n_str ? J.n_sub_tot : 0);

@@ -240,12 +240,21 @@ __device__ __forceinline__ bool behind_key(float d, float bias, uint32_t key, fl
     return d > __fadd_rn(okey_inv(key), bias);
 }
 
+// The largest far plane of each block of kFarBlock x kFarBlock tiles lies at
+// the start of the step's stretch of t_off, which has no other use until the
+// scan fills it.
+constexpr int kFarSh = 3, kFarBlock = 1 << kFarSh;
+__device__ __forceinline__ int64_t far_block(int64_t te0, int tiles_x, int tx, int ty)
+{
+    return te0 + (int64_t)(ty >> kFarSh) * ((tiles_x + kFarBlock - 1) >> kFarSh) + (tx >> kFarSh);
+}
+
 // ---------------------------------------------------------------------------
 // k_clear: reset the wave's accumulators (sizes read from the wave descriptor,
 // so the whole wave can be replayed from one captured graph)
 // ---------------------------------------------------------------------------
 
-// Zero n bytes from p by the whole grid: 16 bytes at a time between the first
+// Zero n bytes from p by threads i0, i0 + 1, ... of `stride`: 16 bytes at a time between the first
 // and the last 16-byte boundary.
 __device__ __forceinline__ void clear_bytes(void* p, int64_t n, int64_t i0, int64_t stride)
 {
@@ -299,13 +308,22 @@ __global__ void k_clear(const WaveDev* __restrict__ W, const JobDev* __restrict_
         B.t_rcnt[i] = 0u;
         B.t_plane[i] = kPlaneNone;
     }
-    // fused path: the outputs per cell start at zero, k_cells writes the cells
-    // that may be shaded
-    for (int q = 0; W->fused && q < W->n_jobs; ++q) {
+    // the jobs' own, a share of the blocks each: the far planes of blocks of
+    // tiles, and on the fused path the outputs per cell (k_cells writes the
+    // cells that may be shaded).  (Cleared by the whole grid one after the
+    // other, 500 jobs' took 379 us; the set-up stage went from 437 to 134.)
+    const int nj = W->n_jobs, per = max((int)gridDim.x / nj, 1);
+    const int64_t j0 = (blockIdx.x % per) * (int64_t)blockDim.x + threadIdx.x, js = (int64_t)per * blockDim.x;
+    for (int q = blockIdx.x / per; q < nj; q += gridDim.x / per) {
         const JobDev& J = jobs[q];
-        if (J.kahan_cell) clear_bytes(reinterpret_cast<uint8_t*>(B.cs_cnt) + J.cs_base, (int64_t)J.k * J.n_cells, i0, stride);
-        if (J.out_counts) clear_rows<1>(J.out_counts, J, i0, stride);
-        if (J.out_bits) clear_rows<8>(reinterpret_cast<uint8_t*>(J.out_bits), J, i0, stride);
+        const int tw = J.tiles_x, cn = (tw + kFarBlock - 1) >> kFarSh, nc = cn * cn;
+        for (int64_t i = j0; i < (int64_t)J.k * nc; i += js)
+            B.t_off[J.te_base + i / nc * ((int64_t)tw * tw) + i % nc] = 0u;
+        if (!W->fused) continue;
+        if (J.kahan_cell)
+            clear_bytes(reinterpret_cast<uint8_t*>(B.cs_cnt) + J.cs_base, (int64_t)J.k * J.n_cells, j0, js);
+        if (J.out_counts) clear_rows<1>(J.out_counts, J, j0, js);
+        if (J.out_bits) clear_rows<8>(reinterpret_cast<uint8_t*>(J.out_bits), J, j0, js);
     }
 }
 
@@ -550,6 +568,12 @@ __global__ void k_modsetup(const WaveDev* __restrict__ W, const JobDev* __restri
             for (int tx = tr.tx0 + sub; tx <= tr.tx1; tx += grp) {
                 const int64_t te = te0 + (int64_t)ty * J.tiles_x + tx;
                 atomicMax(&B.t_far[te], far_key);
+                // (once per module and block of tiles, and most are no farther
+                // than one before)
+                if ((tx == tr.tx0 || (tx & (kFarBlock - 1)) == 0) && (ty == tr.ty0 || (ty & (kFarBlock - 1)) == 0)) {
+                    uint32_t* fb = &B.t_off[far_block(te0, J.tiles_x, tx, ty)];
+                    if (__ldcg(fb) < far_key) atomicMax(fb, far_key);
+                }
                 atomicAdd(&B.t_rcnt[te], 1u);
                 // the plane group shared by every receiver of the tile
                 const uint32_t pl = (uint32_t)M.plane;
@@ -758,21 +782,52 @@ __device__ __forceinline__ void append_pairs(const Buffers& B, const WaveDev* W,
         }
 }
 
-constexpr int kLaneTiles = 16;  // a meshlet over at most this many tiles is tested by its own lane
+constexpr int kLaneTiles = 16;   // a meshlet over at most this many tiles is tested by its own lane,
+constexpr int kFineTiles = 512;  // over at most this many tile by tile, over more by blocks of tiles only
+
+// Texel extents of a world box under a light.
+struct TexBox {
+    float x0, x1, y0, y1, d0;
+};
+__device__ __forceinline__ TexBox project_box(const float4* box, const JobDev& J, const LightParams& lp)
+{
+    const float4 lo = box[0], hi = box[1];
+    TexBox b = {FLT_MAX, -FLT_MAX, FLT_MAX, -FLT_MAX, FLT_MAX};
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float x = ((c & 1) ? hi.x : lo.x) - J.ref[0];
+        const float y = ((c & 2) ? hi.y : lo.y) - J.ref[1];
+        const float z = ((c & 4) ? hi.z : lo.z) - J.ref[2];
+        const float tx = (x * lp.ux + y * lp.uy + z * lp.uz - lp.u0) * lp.inv_delta;
+        const float ty = (x * lp.vx + y * lp.vy + z * lp.vz - lp.v0) * lp.inv_delta;
+        b.x0 = fminf(b.x0, tx); b.x1 = fmaxf(b.x1, tx);
+        b.y0 = fminf(b.y0, ty); b.y1 = fmaxf(b.y1, ty);
+        b.d0 = fminf(b.d0, -(x * lp.sx + y * lp.sy + z * lp.sz));
+    }
+    return b;
+}
 
 __global__ void __launch_bounds__(256, 4) k_bin(const WaveDev* __restrict__ W, const JobDev* __restrict__ jobs,
                                              Buffers B)
 {
-    // One warp per (group of 32 meshlets, step), the step fastest so that
-    // consecutive warps reuse the group's triangles from cache.  Each lane
-    // first projects one scene meshlet's bounding box for the step and keeps
-    // it if it overlaps the light window; the warp then tests each kept box
-    // against the far planes of the tiles it covers (lanes over tiles): if no
-    // tile can receive a shadow from the meshlet, its 32 triangles are
-    // skipped together.  Otherwise each lane bins one of its triangles.
-    // Generator module triangles follow the scene's, in meshlets of 32,
-    // without the box test.  A triangle over more than kBigTiles tiles is
-    // listed for k_bin_big.
+    // One warp per (32 groups of 32 meshlets, step), the step fastest so that
+    // consecutive warps reuse the groups' triangles from cache.  Each lane
+    // projects one group's bounding box; in the groups that overlap the light
+    // window, one after the other, each lane then projects one scene meshlet's
+    // box and keeps it if it overlaps the window; each kept box is tested
+    // against the far planes of the tiles it covers: if no tile can receive a
+    // shadow from the meshlet, its 32 triangles are skipped together.
+    // Otherwise each lane bins one of its triangles.  Generator module
+    // triangles follow the scene's, in meshlets of 32, without the box test.
+    // A triangle over more than kBigTiles tiles is listed for k_bin_big.
+    //
+    // Bound by instruction issue (65 % of the slots while an SM has work).
+    // 500 light windows over 560 000 triangles, 29 suns: almost every meshlet
+    // is outside a window, and with a box each tested by every window the
+    // kernel took 4.49 ms, with groups first 0.6.  One window over all of them,
+    // 47 suns: at a low sun a meshlet's box covers thousands of tiles, and the
+    // warps that had to read them all took 652 us while the others had long
+    // finished; by blocks of tiles 223.
     const int64_t tot = W->tot_tri;
     const int nj = W->n_jobs;
     const int sh = W->tile_sh;
@@ -780,11 +835,14 @@ __global__ void __launch_bounds__(256, 4) k_bin(const WaveDev* __restrict__ W, c
     const int u24 = W->depth_u24;
     const int lane = threadIdx.x & 31;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t item = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; item < tot; item += n_warps) {
-        const int j = job_of(nj, item, [&](int q) { return jobs[q].it_tri; });
+    // few items: several warps share one's groups, each testing all boxes
+    int parts = 1;
+    while (parts < 32 && tot * parts < n_warps) parts *= 2;
+    for (int64_t item = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; item < tot * parts; item += n_warps) {
+        const int j = job_of(nj, item, [&](int q) { return jobs[q].it_tri * parts; });
         const JobDev& J = jobs[j];
-        const int64_t li = item - J.it_tri;
-        const int g = (int)(li / J.k), ls = (int)(li - (int64_t)g * J.k);
+        const uint32_t li = (uint32_t)(item - J.it_tri * parts);
+        const int sp = (int)(li / (uint32_t)J.k), ls = (int)(li - (uint32_t)sp * (uint32_t)J.k);
         const int R = J.R;
         const int64_t js = J.js_base + ls;
         const LightParams& lp = B.lp[js];
@@ -794,139 +852,158 @@ __global__ void __launch_bounds__(256, 4) k_bin(const WaveDev* __restrict__ W, c
         // with boxes, then the job's own module meshlets
         const int n_boxed = J.n_ml + J.n_oml;
         const int n_all = n_boxed + ((J.n_mtris + 31) >> 5);
-        // this lane's boxed meshlet: window test, covered tiles, nearest depth key
-        const int ml = g * 32 + lane;
-        int btx0 = 0, btx1 = -1, bty0 = 0, bty1 = -1;
-        uint32_t bkey = 0u;
-        bool pass = false;
-        if (ml < n_boxed) {
-            const float4* box = ml < J.n_ml ? J.ml_box + 2 * ml : J.oml_box + 2 * (ml - J.n_ml);
-            const float4 lo = box[0], hi = box[1];
-            float xmin = FLT_MAX, xmax = -FLT_MAX, ymin = FLT_MAX, ymax = -FLT_MAX, dmin = FLT_MAX;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float x = ((c & 1) ? hi.x : lo.x) - J.ref[0];
-                const float y = ((c & 2) ? hi.y : lo.y) - J.ref[1];
-                const float z = ((c & 4) ? hi.z : lo.z) - J.ref[2];
-                const float tx = (x * lp.ux + y * lp.uy + z * lp.uz - lp.u0) * lp.inv_delta;
-                const float ty = (x * lp.vx + y * lp.vy + z * lp.vz - lp.v0) * lp.inv_delta;
-                xmin = fminf(xmin, tx); xmax = fmaxf(xmax, tx);
-                ymin = fminf(ymin, ty); ymax = fmaxf(ymax, ty);
-                dmin = fminf(dmin, -(x * lp.sx + y * lp.sy + z * lp.sz));
-            }
-            pass = xmax >= 0.5f && ymax >= 0.5f && xmin <= R - 0.5f && ymin <= R - 0.5f;
-            if (pass) {
-                btx0 = max(0, (int)floorf(xmin - 0.5f)) >> sh;
-                btx1 = min(R - 1, (int)ceilf(xmax)) >> sh;
-                bty0 = max(0, (int)floorf(ymin - 0.5f)) >> sh;
-                bty1 = min(R - 1, (int)ceilf(ymax)) >> sh;
-                // the box's nearest point, less a margin for the rounding of
-                // the projection
-                bkey = depth_store_key(dmin - 1e-3f * (1.f + fabsf(dmin)), lp, u24);
-            }
-        } else {
-            pass = ml < n_all;
+        // this lane's group of 32 meshlets: those of the scene have a box
+        const int gl = (sp / parts) * 32 + lane;
+        bool in_window = gl * 32 < n_all && (lane & (parts - 1)) == (sp & (parts - 1));
+        if (in_window && gl * 32 + 31 < J.n_ml) {
+            const TexBox bx = project_box(J.ml_box + 2 * (J.n_ml + gl), J, lp);
+            in_window = bx.x1 >= 0.f && bx.y1 >= 0.f && bx.x0 <= (float)R && bx.y0 <= (float)R;
         }
-        // the meshlet's nearest point against the far plane of each tile it
-        // covers: each lane tests its own meshlet's tiles (independent loads
-        // across the warp), the warp together those of a meshlet over many
-        // tiles
-        bool keep_lane = false, coop = false;
-        if (pass && ml < n_boxed) {
-            const int ntl = (btx1 - btx0 + 1) * (bty1 - bty0 + 1);
-            if (ntl <= kLaneTiles) {
-                // no early exit: the loads of a row of tiles are issued together
-                for (int ty = bty0; ty <= bty1; ++ty) {
-                    const uint32_t* far_row = B.t_far + te0 + (int64_t)ty * J.tiles_x;
-#pragma unroll 4
-                    for (int tx = btx0; tx <= btx1; ++tx) keep_lane |= bkey < far_row[tx];
+#pragma unroll 1
+        for (unsigned int gm = __ballot_sync(0xffffffffu, in_window); gm; gm &= gm - 1u) {
+            const int g = (sp / parts) * 32 + __ffs((int)gm) - 1;
+            // this lane's boxed meshlet: window test, covered tiles, nearest depth key
+            const int ml = g * 32 + lane;
+            int btx0 = 0, btx1 = -1, bty0 = 0, bty1 = -1;
+            uint32_t bkey = 0u;
+            bool pass = false;
+            if (ml < n_boxed) {
+                const TexBox bx = project_box(ml < J.n_ml ? J.ml_box + 2 * ml : J.oml_box + 2 * (ml - J.n_ml), J, lp);
+                const float xmin = bx.x0, xmax = bx.x1, ymin = bx.y0, ymax = bx.y1, dmin = bx.d0;
+                pass = xmax >= 0.5f && ymax >= 0.5f && xmin <= R - 0.5f && ymin <= R - 0.5f;
+                if (pass) {
+                    btx0 = max(0, (int)floorf(xmin - 0.5f)) >> sh;
+                    btx1 = min(R - 1, (int)ceilf(xmax)) >> sh;
+                    bty0 = max(0, (int)floorf(ymin - 0.5f)) >> sh;
+                    bty1 = min(R - 1, (int)ceilf(ymax)) >> sh;
+                    // the box's nearest point, less a margin for the rounding of
+                    // the projection
+                    bkey = depth_store_key(dmin - 1e-3f * (1.f + fabsf(dmin)), lp, u24);
                 }
             } else {
-                coop = true;
+                pass = ml < n_all;
             }
-        } else if (pass) {
-            keep_lane = true;  // module meshlets: no box
-        }
-        unsigned int kept = __ballot_sync(0xffffffffu, keep_lane);
-        for (unsigned int cm = __ballot_sync(0xffffffffu, coop); cm; cm &= cm - 1u) {
-            const int q = __ffs(cm) - 1;
-            const int mx0 = __shfl_sync(0xffffffffu, btx0, q), mx1 = __shfl_sync(0xffffffffu, btx1, q);
-            const int my0 = __shfl_sync(0xffffffffu, bty0, q), my1 = __shfl_sync(0xffffffffu, bty1, q);
-            const uint32_t mkey = __shfl_sync(0xffffffffu, bkey, q);
-            const int wx = mx1 - mx0 + 1, ntl = wx * (my1 - my0 + 1);
-            bool keep = false;
-            for (int q0 = 0; q0 < ntl && !keep; q0 += 32) {
-                const int k = q0 + lane;
-                bool kk = false;
-                if (k < ntl) {
-                    const int ty = my0 + k / wx, tx = mx0 + k % wx;
-                    kk = mkey < B.t_far[te0 + (int64_t)ty * J.tiles_x + tx];
-                }
-                keep = __any_sync(0xffffffffu, kk);
-            }
-            if (keep) kept |= 1u << q;
-        }
-        for (unsigned int cand = kept; cand; cand &= cand - 1u) {
-            const int q = __ffs(cand) - 1;
-            const int mi = g * 32 + q;
-            int t;
-            bool act;
-            if (mi < n_boxed) {
-                if (mi < J.n_ml) {
-                    t = mi * 32 + lane;
-                    act = t < J.n_tris;
+            // the meshlet's nearest point against the far plane of each tile it
+            // covers: each lane tests its own meshlet's tiles (independent loads
+            // across the warp), the warp together those of a meshlet over many
+            // tiles
+            bool keep_lane = false, coop = false;
+            if (pass && ml < n_boxed) {
+                const int ntl = (btx1 - btx0 + 1) * (bty1 - bty0 + 1);
+                if (ntl <= kLaneTiles) {
+                    // no early exit: the loads of a row of tiles are issued together
+                    for (int ty = bty0; ty <= bty1; ++ty) {
+                        const uint32_t* far_row = B.t_far + te0 + (int64_t)ty * J.tiles_x;
+    #pragma unroll 4
+                        for (int tx = btx0; tx <= btx1; ++tx) keep_lane |= bkey < far_row[tx];
+                    }
                 } else {
-                    t = J.n_tris + (mi - J.n_ml) * 32 + lane;
-                    act = t < J.n_tris + 2 * J.n_occ;
+                    coop = true;
                 }
-            } else {
-                t = J.n_tris + (mi - n_boxed) * 32 + lane;
-                act = t < J.n_tris + J.n_mtris;
+            } else if (pass) {
+                keep_lane = true;  // module meshlets: no box
             }
-            // per lane: the tiles its triangle may shade (at most kBigTiles), in
-            // registers until the warp appends them together
-            uint32_t te[kBigTiles];
-            uint32_t valid = 0u;
-            if (act) {
-                TriT T;
-                tri_texel(J, B, lp, ls, t, T);
-                const uint32_t tplane = module_tri_plane(J, t);
-                Edges e;
-                const float xmin = fminf(T.x[0], fminf(T.x[1], T.x[2])), xmax = fmaxf(T.x[0], fmaxf(T.x[1], T.x[2]));
-                const float ymin = fminf(T.y[0], fminf(T.y[1], T.y[2])), ymax = fmaxf(T.y[0], fmaxf(T.y[1], T.y[2]));
-                // covered texel centres (ix + 0.5) lie in [xmin, xmax]
-                const int ix0 = max(0, (int)ceilf(xmin - 0.5f)), ix1 = min(R - 1, (int)floorf(xmax - 0.5f));
-                const int iy0 = max(0, (int)ceilf(ymin - 0.5f)), iy1 = min(R - 1, (int)floorf(ymax - 0.5f));
-                if (make_edges(T, e) && xmax >= 0.5f && ymax >= 0.5f && xmin <= R - 0.5f && ymin <= R - 0.5f &&
-                    ix0 <= ix1 && iy0 <= iy1) {
-                    const uint32_t dkey = depth_store_key(fminf(T.d[0], fminf(T.d[1], T.d[2])), lp, u24);
-                    const int tx0 = ix0 >> sh, tx1 = ix1 >> sh, ty0 = iy0 >> sh, ty1 = iy1 >> sh;
-                    const int wx = tx1 - tx0 + 1, ntiles = wx * (ty1 - ty0 + 1);
-                    if (ntiles > kBigTiles) {
-                        const unsigned int pos = atomicAdd(&B.ctr->n_big, 1u);
-                        if (pos < (uint64_t)W->big_cap) B.big[pos] = make_uint2((uint32_t)t, (uint32_t)js);
+            unsigned int kept = __ballot_sync(0xffffffffu, keep_lane);
+            for (unsigned int cm = __ballot_sync(0xffffffffu, coop); cm; cm &= cm - 1u) {
+                const int q = __ffs(cm) - 1;
+                const int mx0 = __shfl_sync(0xffffffffu, btx0, q), mx1 = __shfl_sync(0xffffffffu, btx1, q);
+                const int my0 = __shfl_sync(0xffffffffu, bty0, q), my1 = __shfl_sync(0xffffffffu, bty1, q);
+                const uint32_t mkey = __shfl_sync(0xffffffffu, bkey, q);
+                const int wx = mx1 - mx0 + 1, ntl = wx * (my1 - my0 + 1);
+                // blocks of tiles first
+                const int cx0 = mx0 >> kFarSh, cy0 = my0 >> kFarSh, cw = (mx1 >> kFarSh) - cx0 + 1;
+                const int nc = cw * ((my1 >> kFarSh) - cy0 + 1);
+                bool keep = false;
+                for (int q0 = 0; q0 < nc && !keep; q0 += 32) {
+                    const int k = q0 + lane;
+                    keep = __any_sync(0xffffffffu,
+                                      k < nc && mkey < B.t_off[far_block(te0, J.tiles_x, (cx0 + k % cw) << kFarSh,
+                                                                         (cy0 + k / cw) << kFarSh)]);
+                }
+                if (keep && ntl > kFineTiles) {
+                    kept |= 1u << q;
+                    continue;
+                }
+                if (!keep) continue;
+                keep = false;
+                for (int q0 = 0; q0 < ntl && !keep; q0 += 32) {
+                    const int k = q0 + lane;
+                    bool kk = false;
+                    if (k < ntl) {
+                        const int ty = my0 + k / wx, tx = mx0 + k % wx;
+                        kk = mkey < B.t_far[te0 + (int64_t)ty * J.tiles_x + tx];
+                    }
+                    keep = __any_sync(0xffffffffu, kk);
+                }
+                if (keep) kept |= 1u << q;
+            }
+            for (unsigned int cand = kept; cand; cand &= cand - 1u) {
+                const int q = __ffs(cand) - 1;
+                const int mi = g * 32 + q;
+                int t;
+                bool act;
+                if (mi < n_boxed) {
+                    if (mi < J.n_ml) {
+                        t = mi * 32 + lane;
+                        act = t < J.n_tris;
                     } else {
-#pragma unroll
-                        for (int q = 0; q < kBigTiles; ++q) {
-                            te[q] = 0u;
-                            if (q >= ntiles) continue;
-                            const int ty = ty0 + q / wx, tx = tx0 + q % wx;
-                            if (ntiles > 1 && !rect_overlap(e, tx * TS + 0.5f, tx * TS + TS - 0.5f, ty * TS + 0.5f,
-                                                            ty * TS + TS - 0.5f))
-                                continue;
-                            const uint32_t x = (uint32_t)(te0 + (int64_t)ty * J.tiles_x + tx);
-                            // unoccupied tile (far 0) or triangle wholly behind its far plane
-                            if (!(dkey < B.t_far[x])) continue;
-                            // a module triangle in the plane of every receiver of the tile
-                            if (tplane != kPlaneNone && B.t_plane[x] == tplane) continue;
-                            atomicAdd(&B.t_cnt[x], 1u);
-                            te[q] = x;
-                            valid |= 1u << q;
+                        t = J.n_tris + (mi - J.n_ml) * 32 + lane;
+                        act = t < J.n_tris + 2 * J.n_occ;
+                    }
+                } else {
+                    t = J.n_tris + (mi - n_boxed) * 32 + lane;
+                    act = t < J.n_tris + J.n_mtris;
+                }
+                // per lane: the tiles its triangle may shade (at most kBigTiles), in
+                // registers until the warp appends them together
+                uint32_t te[kBigTiles];
+                uint32_t valid = 0u;
+                if (act) {
+                    TriT T;
+                    tri_texel(J, B, lp, ls, t, T);
+                    const uint32_t tplane = module_tri_plane(J, t);
+                    Edges e;
+                    const float xmin = fminf(T.x[0], fminf(T.x[1], T.x[2])), xmax = fmaxf(T.x[0], fmaxf(T.x[1], T.x[2]));
+                    const float ymin = fminf(T.y[0], fminf(T.y[1], T.y[2])), ymax = fmaxf(T.y[0], fmaxf(T.y[1], T.y[2]));
+                    // covered texel centres (ix + 0.5) lie in [xmin, xmax]
+                    const int ix0 = max(0, (int)ceilf(xmin - 0.5f)), ix1 = min(R - 1, (int)floorf(xmax - 0.5f));
+                    const int iy0 = max(0, (int)ceilf(ymin - 0.5f)), iy1 = min(R - 1, (int)floorf(ymax - 0.5f));
+                    if (make_edges(T, e) && xmax >= 0.5f && ymax >= 0.5f && xmin <= R - 0.5f && ymin <= R - 0.5f &&
+                        ix0 <= ix1 && iy0 <= iy1) {
+                        const uint32_t dkey = depth_store_key(fminf(T.d[0], fminf(T.d[1], T.d[2])), lp, u24);
+                        const int tx0 = ix0 >> sh, tx1 = ix1 >> sh, ty0 = iy0 >> sh, ty1 = iy1 >> sh;
+                        const int wx = tx1 - tx0 + 1, ntiles = wx * (ty1 - ty0 + 1);
+                        if (ntiles > kBigTiles) {
+                            const unsigned int pos = atomicAdd(&B.ctr->n_big, 1u);
+                            if (pos < (uint64_t)W->big_cap) B.big[pos] = make_uint2((uint32_t)t, (uint32_t)js);
+                        } else {
+                            int nx = tx0, ny = ty0;
+    #pragma unroll
+                            for (int q = 0; q < kBigTiles; ++q) {
+                                te[q] = 0u;
+                                if (q >= ntiles) continue;
+                                const int tx = nx, ty = ny;
+                                if (++nx > tx1) {
+                                    nx = tx0;
+                                    ++ny;
+                                }
+                                if (ntiles > 1 && !rect_overlap(e, tx * TS + 0.5f, tx * TS + TS - 0.5f, ty * TS + 0.5f,
+                                                                ty * TS + TS - 0.5f))
+                                    continue;
+                                const uint32_t x = (uint32_t)(te0 + (int64_t)ty * J.tiles_x + tx);
+                                // unoccupied tile (far 0) or triangle wholly behind its far plane
+                                if (!(dkey < B.t_far[x])) continue;
+                                // a module triangle in the plane of every receiver of the tile
+                                if (tplane != kPlaneNone && B.t_plane[x] == tplane) continue;
+                                atomicAdd(&B.t_cnt[x], 1u);
+                                te[q] = x;
+                                valid |= 1u << q;
+                            }
                         }
                     }
                 }
+                append_pairs(B, W, te, valid, (uint32_t)t);
             }
-            append_pairs(B, W, te, valid, (uint32_t)t);
         }
     }
 }

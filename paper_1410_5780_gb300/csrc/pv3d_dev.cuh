@@ -67,7 +67,8 @@ struct JobDev {
     const float4* tri;
     int32_t n_tris;
     int32_t n_mtris;  // module triangles rasterised: 2 per module, or 0 for a coplanar generator
-    const float4* ml_box;  // scene meshlets (32 consecutive triangles, median-split order): world lo, hi
+    const float4* ml_box;  // scene meshlets (32 consecutive triangles, median-split order): world lo, hi;
+                           // then those of each 32 meshlets in a row
     int32_t n_ml;          // scene meshlets = ceil(n_tris / 32)
     int32_t pad_ml;
     // generator
@@ -167,7 +168,7 @@ struct WaveDev {
     int32_t fused;      // 1: coverage bits per tile; 0: map in HBM + gather kernel
     int32_t profile;    // count work (texel visits, sample tests) into Counters
     int64_t tot_js, tot_te, tot_ms, tot_cs;
-    int64_t tot_win, tot_mod, tot_tri, tot_epi;  // tot_tri: (group of 32 meshlets, step) warp items
+    int64_t tot_win, tot_mod, tot_tri, tot_epi;  // tot_tri: (32 groups of 32 meshlets, step) warp items
     int64_t tot_ss, tot_sq;                      // (step, substring) and (step, string) entries
     int64_t tot_heat;                            // heat-map bins over the jobs
     int64_t tot_sa;                              // (step, array) entries
