@@ -2511,6 +2511,14 @@ __device__ __forceinline__ void draw_tris(DrawSm& D, const TriWork& w, uint32_t 
                 const int word = iy * WPR + q;
                 uint32_t c = f0 <= f1 && q >= (f0 >> 5) && q <= (f1 >> 5) ? span_word(f0, f1, q) : 0u, o = 0u;
                 uint32_t r = span_word(c0, c1, q) & ~c & ~cov[l * NW + word];
+                if (!(bk < FLT_MAX)) {  // no plane to compare with: open
+                    o = r;
+                    for (r = TILE ? r : 0u; r; r &= r - 1u) {
+                        const int x = 32 * q + __ffs((int)r) - 1;
+                        if (PROF) ++writes;
+                        atomicMin(&tile[iy * TS + x], depth_store_key(depth_px((float)x + 0.5f), lp, u24));
+                    }
+                }
 #pragma unroll 1
                 for (; r; r &= r - 1u) {
                     const int x = __ffs((int)r) - 1;
