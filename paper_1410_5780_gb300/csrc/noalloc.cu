@@ -38,6 +38,13 @@ constexpr uint32_t kEmptyKey = 0xFFFFFFFFu;
 
 static __device__ __align__(256) uint32_t g_noalloc_map[kNoAllocMaxRes * kNoAllocMaxRes];
 
+// Triangles over more than kBigTexels texels of the map, for na_big: as the
+// map, one list for all calls.
+constexpr int64_t kBigTexels = 1024;
+constexpr unsigned int kBigCap = 4096;
+static __device__ uint32_t g_noalloc_big[kBigCap];
+static __device__ unsigned int g_noalloc_n_big;
+
 std::mutex g_setup_mu;
 uint32_t* g_map_ptr[kMaxDevices] = {};
 
@@ -67,57 +74,107 @@ __global__ void na_clear(uint32_t* map, int64_t n_texels, uint32_t* counts, int 
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_texels; i += stride) map[i] = kEmptyKey;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_cells; i += stride) counts[i] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) g_noalloc_n_big = 0u;
 }
 
-// One warp per triangle: texel-centre coverage (inclusive edges), barycentric
-// depth, atomicMin of the order-preserving depth key into the map.
+// A triangle in the map: edge functions, vertex depths and texel box.
+struct NaTri {
+    float A[3], Bc[3], C[3], d[3];
+    float inv_a;
+    int x0, x1, y0, y1;
+};
+
+// Triangle t of tri; false if it covers no texel centre of the map.
+__device__ __forceinline__ bool na_setup(const float* __restrict__ tri, int64_t t, const NaFrame& f, NaTri& T)
+{
+    float x[3], y[3];
+    float* d = T.d;
+    for (int k = 0; k < 3; ++k) {
+        const float px = tri[9 * t + 3 * k] - f.refx, py = tri[9 * t + 3 * k + 1] - f.refy,
+                    pz = tri[9 * t + 3 * k + 2] - f.refz;
+        x[k] = (px * f.ux + py * f.uy + pz * f.uz - f.u0) * f.inv_delta;
+        y[k] = (px * f.vx + py * f.vy + pz * f.vz - f.v0) * f.inv_delta;
+        d[k] = -(px * f.sx + py * f.sy + pz * f.sz);
+    }
+    float area2 = (x[1] - x[0]) * (y[2] - y[0]) - (y[1] - y[0]) * (x[2] - x[0]);
+    if (!(fabsf(area2) > 0.f)) return false;
+    if (area2 < 0.f) {
+        float t0 = x[1], t1 = y[1], t2 = d[1];
+        x[1] = x[2]; y[1] = y[2]; d[1] = d[2];
+        x[2] = t0; y[2] = t1; d[2] = t2;
+        area2 = -area2;
+    }
+    const float xmin = fminf(x[0], fminf(x[1], x[2])), xmax = fmaxf(x[0], fmaxf(x[1], x[2]));
+    const float ymin = fminf(y[0], fminf(y[1], y[2])), ymax = fmaxf(y[0], fmaxf(y[1], y[2]));
+    if (!(xmax >= 0.5f && ymax >= 0.5f && xmin <= f.R - 0.5f && ymin <= f.R - 0.5f)) return false;
+    T.x0 = max(0, (int)ceilf(xmin - 0.5f));
+    T.x1 = min(f.R - 1, (int)floorf(xmax - 0.5f));
+    T.y0 = max(0, (int)ceilf(ymin - 0.5f));
+    T.y1 = min(f.R - 1, (int)floorf(ymax - 0.5f));
+    if (T.x0 > T.x1 || T.y0 > T.y1) return false;
+    for (int k = 0; k < 3; ++k) {
+        const int a = (k + 1) % 3, b = (k + 2) % 3;
+        T.A[k] = -(y[b] - y[a]);
+        T.Bc[k] = x[b] - x[a];
+        T.C[k] = -(T.A[k] * x[a] + T.Bc[k] * y[a]);
+    }
+    T.inv_a = 1.f / area2;
+    return true;
+}
+
+// Texel-centre coverage (inclusive edges), barycentric depth, atomicMin of the
+// order-preserving depth key into the map.
+__device__ __forceinline__ void na_texel(const NaTri& T, const NaFrame& f, int ix, int iy, uint32_t* map)
+{
+    const float px = ix + 0.5f, py = iy + 0.5f;
+    const float w0 = T.A[0] * px + T.Bc[0] * py + T.C[0];
+    const float w1 = T.A[1] * px + T.Bc[1] * py + T.C[1];
+    const float w2 = T.A[2] * px + T.Bc[2] * py + T.C[2];
+    if (w0 >= 0.f && w1 >= 0.f && w2 >= 0.f)
+        atomicMin(&map[(int64_t)iy * f.R + ix], na_key((w0 * T.d[0] + w1 * T.d[1] + w2 * T.d[2]) * T.inv_a));
+}
+
+// One warp per triangle, as many rows at a time as its width leaves lanes for.
+// A triangle over many texels is left to na_big: drawn by one warp, the largest
+// were the kernel's time (1,024 texels are 32 steps of a warp).  With that and
+// no division per texel a call went from 145 to 66 us (one module, one sun) and
+// from 2,253 to 423 us on a map mostly covered by single triangles.
 __global__ void na_raster(const float* __restrict__ tri, int64_t n_tris, NaFrame f, uint32_t* map)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t t = warp; t < n_tris; t += n_warps) {
-        float x[3], y[3], d[3];
-        for (int k = 0; k < 3; ++k) {
-            const float px = tri[9 * t + 3 * k] - f.refx, py = tri[9 * t + 3 * k + 1] - f.refy,
-                        pz = tri[9 * t + 3 * k + 2] - f.refz;
-            x[k] = (px * f.ux + py * f.uy + pz * f.uz - f.u0) * f.inv_delta;
-            y[k] = (px * f.vx + py * f.vy + pz * f.vz - f.v0) * f.inv_delta;
-            d[k] = -(px * f.sx + py * f.sy + pz * f.sz);
+        NaTri T;
+        if (!na_setup(tri, t, f, T)) continue;
+        const int bw = T.x1 - T.x0 + 1;
+        if ((int64_t)bw * (T.y1 - T.y0 + 1) > kBigTexels && t <= 0xFFFFFFFFll) {
+            unsigned int pos = 0u;
+            if (lane == 0) {
+                pos = atomicAdd(&g_noalloc_n_big, 1u);
+                if (pos < kBigCap) g_noalloc_big[pos] = (uint32_t)t;
+            }
+            if (__shfl_sync(0xffffffffu, pos, 0) < kBigCap) continue;  // (a full list: drawn here)
         }
-        float area2 = (x[1] - x[0]) * (y[2] - y[0]) - (y[1] - y[0]) * (x[2] - x[0]);
-        if (!(fabsf(area2) > 0.f)) continue;
-        if (area2 < 0.f) {
-            float t0 = x[1], t1 = y[1], t2 = d[1];
-            x[1] = x[2]; y[1] = y[2]; d[1] = d[2];
-            x[2] = t0; y[2] = t1; d[2] = t2;
-            area2 = -area2;
-        }
-        const float xmin = fminf(x[0], fminf(x[1], x[2])), xmax = fmaxf(x[0], fmaxf(x[1], x[2]));
-        const float ymin = fminf(y[0], fminf(y[1], y[2])), ymax = fmaxf(y[0], fmaxf(y[1], y[2]));
-        if (!(xmax >= 0.5f && ymax >= 0.5f && xmin <= f.R - 0.5f && ymin <= f.R - 0.5f)) continue;
-        const int x0 = max(0, (int)ceilf(xmin - 0.5f)), x1 = min(f.R - 1, (int)floorf(xmax - 0.5f));
-        const int y0 = max(0, (int)ceilf(ymin - 0.5f)), y1 = min(f.R - 1, (int)floorf(ymax - 0.5f));
-        if (x0 > x1 || y0 > y1) continue;
-        float A[3], Bc[3], C[3];
-        for (int k = 0; k < 3; ++k) {
-            const int a = (k + 1) % 3, b = (k + 2) % 3;
-            A[k] = -(y[b] - y[a]);
-            Bc[k] = x[b] - x[a];
-            C[k] = -(A[k] * x[a] + Bc[k] * y[a]);
-        }
-        const float inv_a = 1.f / area2;
-        const int bw = x1 - x0 + 1;
-        const int64_t n_px = (int64_t)bw * (y1 - y0 + 1);
-        for (int64_t q = lane; q < n_px; q += 32) {
-            const int iy = y0 + (int)(q / bw), ix = x0 + (int)(q % bw);
-            const float px = ix + 0.5f, py = iy + 0.5f;
-            const float w0 = A[0] * px + Bc[0] * py + C[0];
-            const float w1 = A[1] * px + Bc[1] * py + C[1];
-            const float w2 = A[2] * px + Bc[2] * py + C[2];
-            if (w0 >= 0.f && w1 >= 0.f && w2 >= 0.f)
-                atomicMin(&map[(int64_t)iy * f.R + ix], na_key((w0 * d[0] + w1 * d[1] + w2 * d[2]) * inv_a));
-        }
+        const int sh = bw > 16 ? 5 : 32 - __clz(bw - 1), w = 1 << sh;  // lanes a row: bw rounded up to a power of two
+        for (int iy = T.y0 + (lane >> sh); iy <= T.y1; iy += 32 >> sh)
+            for (int ix = T.x0 + (lane & (w - 1)); ix <= T.x1; ix += w) na_texel(T, f, ix, iy, map);
+    }
+}
+
+// The triangles over many texels: one warp per (triangle, row).
+__global__ void na_big(const float* __restrict__ tri, int64_t n_tris, NaFrame f, uint32_t* map)
+{
+    const unsigned int n = min(g_noalloc_n_big, kBigCap);
+    const int lane = threadIdx.x & 31;
+    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < (int64_t)n * f.R; i += n_warps) {
+        const int64_t t = g_noalloc_big[i / f.R];
+        NaTri T;
+        if (t >= n_tris || !na_setup(tri, t, f, T)) continue;  // (t >= n_tris: another call's, see above)
+        const int iy = T.y0 + (int)(i % f.R);
+        if (iy > T.y1) continue;
+        for (int ix = T.x0 + lane; ix <= T.x1; ix += 32) na_texel(T, f, ix, iy, map);
     }
 }
 
@@ -244,6 +301,9 @@ extern "C" int pv3d_module_shade_noalloc(const float* tri_xyz, int64_t n_tris, c
             void* a_raster[] = {(void*)&tri_xyz, &n_tris, &f, &map};
             if (cudaLaunchKernel((const void*)na_raster, dim3((unsigned)blocks), dim3(256), a_raster, 0, st) !=
                 cudaSuccess)
+                return PV3D_E_DEVICE;
+            // (1216: eight blocks on each of 152 SMs)
+            if (cudaLaunchKernel((const void*)na_big, dim3(1216), dim3(256), a_raster, 0, st) != cudaSuccess)
                 return PV3D_E_DEVICE;
         }
         float3 o = make_float3((float)(M.origin[0] - ref[0]), (float)(M.origin[1] - ref[1]),
