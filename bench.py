@@ -507,10 +507,12 @@ def tile_kernel_rooflines(work, stages_ms, tile, n_waves, hbm_gbs, alu_tops, ras
     * bytes (the HBM byte model of a depth-map design restricted to the
       kernel's tiles): 4 B per texel of every tile it takes (the depth tile
       written once) + 4 B per sample it tests (the texel gather);
-    * lane-ops: 12 per fragment (a kept triangle covering a texel a sample
-      reads: 3 edge functions, barycentric depth, key and minimum) + 14 per
-      sample test (position, projection, texel, compare);
-    * fragments F (k_raster_test: depth atomicMin writes into the shared tile).
+    * lane-ops: 12 per fragment (a triangle in front of or across a receiver
+      plane covering a texel: 3 edge functions, barycentric depth, key and
+      minimum) + 14 per sample test (position, projection, texel, compare);
+    * fragments F against the atomicMin rate of the same writes.
+    The kernels do less: a fragment is a bit of a row's span, and the samples
+    are looked up in k_cells (the PV stage).
     """
     nw = max(n_waves, 1)
     heavy = {"tiles": work["heavy_tiles"], "samples": work["heavy_sample_tests"],
