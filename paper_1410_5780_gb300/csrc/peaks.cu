@@ -1,7 +1,7 @@
 // peaks.cu -- pv3d_raster_peak: the measured throughput of shared-memory
 // atomicMin on 32-bit depth keys, the second roofline of the rasterising
 // kernels (the first is HBM bandwidth).  Each block holds a 32 x 32 tile of
-// keys in shared memory, as k_raster_test does, and its warps draw strips of
+// keys in shared memory, as k_raster_map does, and its warps draw strips of
 // 32 consecutive texels (one per lane, a chunk of a triangle's texel visits)
 // with atomicMin of a varying key; the tile is folded into one word per block
 // at the end so that no update can be optimised away.

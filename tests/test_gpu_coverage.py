@@ -68,7 +68,7 @@ def _grazing_suns(tilt, degrees):
 
 
 CASES = {
-    # more planes in a tile than levels (12, 4 and 2): the last level is shared
+    # more planes in a tile than levels (12, 8 and 4): the last level is shared
     "planes_32": lambda: _rows(40, (4, 5), 3, 4, 64),
     "planes_32_fine": lambda: _rows(24, (6, 10), 4, 3, 512),
     # the sun within a degree of the modules' plane, on it, and behind it
