@@ -39,11 +39,13 @@ constexpr uint32_t kEmptyKey = 0xFFFFFFFFu;
 static __device__ __align__(256) uint32_t g_noalloc_map[kNoAllocMaxRes * kNoAllocMaxRes];
 
 // Triangles over more than kBigTexels texels of the map, for na_big: as the
-// map, one list for all calls.
+// map, one list for all calls.  A triangle is drawn in steps of 32 texels of a
+// row; entry i of the list is its index and the steps of the entries before it.
 constexpr int64_t kBigTexels = 1024;
 constexpr unsigned int kBigCap = 4096;
-static __device__ uint32_t g_noalloc_big[kBigCap];
-static __device__ unsigned int g_noalloc_n_big;
+constexpr unsigned int kBigSteps = 16;  // na_big: a warp takes so many at least
+static __device__ uint2 g_noalloc_big[kBigCap + 1];
+static __device__ unsigned long long g_noalloc_n_big;  // entries << 32 | steps
 
 std::mutex g_setup_mu;
 uint32_t* g_map_ptr[kMaxDevices] = {};
@@ -74,7 +76,7 @@ __global__ void na_clear(uint32_t* map, int64_t n_texels, uint32_t* counts, int 
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_texels; i += stride) map[i] = kEmptyKey;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_cells; i += stride) counts[i] = 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) g_noalloc_n_big = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) g_noalloc_n_big = 0ull;
 }
 
 // A triangle in the map: edge functions, vertex depths and texel box.
@@ -134,11 +136,16 @@ __device__ __forceinline__ void na_texel(const NaTri& T, const NaFrame& f, int i
         atomicMin(&map[(int64_t)iy * f.R + ix], na_key((w0 * T.d[0] + w1 * T.d[1] + w2 * T.d[2]) * T.inv_a));
 }
 
+// Steps of 32 texels of a row in triangle T's box.
+__device__ __forceinline__ unsigned int na_row_steps(const NaTri& T) { return (unsigned int)(T.x1 - T.x0 + 32) >> 5; }
+__device__ __forceinline__ unsigned int na_steps(const NaTri& T)
+{
+    return na_row_steps(T) * (unsigned int)(T.y1 - T.y0 + 1);
+}
+
 // One warp per triangle, as many rows at a time as its width leaves lanes for.
 // A triangle over many texels is left to na_big: drawn by one warp, the largest
-// were the kernel's time (1,024 texels are 32 steps of a warp).  With that and
-// no division per texel a call went from 145 to 66 us (one module, one sun) and
-// from 2,253 to 423 us on a map mostly covered by single triangles.
+// were the kernel's time (1,024 texels are 32 steps of a warp).
 __global__ void na_raster(const float* __restrict__ tri, int64_t n_tris, NaFrame f, uint32_t* map)
 {
     const int lane = threadIdx.x & 31;
@@ -149,10 +156,14 @@ __global__ void na_raster(const float* __restrict__ tri, int64_t n_tris, NaFrame
         if (!na_setup(tri, t, f, T)) continue;
         const int bw = T.x1 - T.x0 + 1;
         if ((int64_t)bw * (T.y1 - T.y0 + 1) > kBigTexels && t <= 0xFFFFFFFFll) {
-            unsigned int pos = 0u;
-            if (lane == 0) {
-                pos = atomicAdd(&g_noalloc_n_big, 1u);
-                if (pos < kBigCap) g_noalloc_big[pos] = (uint32_t)t;
+            // (a full list is looked at first, so that its count stays within
+            // 32 bits: beyond its end only the warps in flight add to it, some
+            // 1e4 of at most 2^17 steps each)
+            unsigned int pos = kBigCap;
+            if (lane == 0 && (__ldcg(&g_noalloc_n_big) >> 32) < kBigCap) {
+                const unsigned long long old = atomicAdd(&g_noalloc_n_big, (1ull << 32) | na_steps(T));
+                pos = (unsigned int)(old >> 32);
+                if (pos <= kBigCap) g_noalloc_big[pos] = make_uint2((uint32_t)t, (uint32_t)old);
             }
             if (__shfl_sync(0xffffffffu, pos, 0) < kBigCap) continue;  // (a full list: drawn here)
         }
@@ -162,19 +173,53 @@ __global__ void na_raster(const float* __restrict__ tri, int64_t n_tris, NaFrame
     }
 }
 
-// The triangles over many texels: one warp per (triangle, row).
+// The triangles over many texels: their steps in equal shares to the warps, so
+// that the time follows the texels, whether of one triangle or of thousands.
+// Whole calls, a warp a triangle / a warp for each row of the map and triangle /
+// equal shares: one module, one sun, 2,000 triangles, 512 x 512 texels 233 / 84 /
+// 52 us; 4,096 triangles of 33 x 33 texels, 2048 x 2048 48 / 1,690 / 58 us; 12
+// of 900 x 900 5,580 / 52 / 53 us.
 __global__ void na_big(const float* __restrict__ tri, int64_t n_tris, NaFrame f, uint32_t* map)
 {
-    const unsigned int n = min(g_noalloc_n_big, kBigCap);
-    const int lane = threadIdx.x & 31;
-    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < (int64_t)n * f.R; i += n_warps) {
-        const int64_t t = g_noalloc_big[i / f.R];
+    const unsigned long long listed = g_noalloc_n_big;
+    const unsigned int n = min((unsigned int)(listed >> 32), kBigCap);
+    if (n == 0u) return;
+    const unsigned int total = (listed >> 32) > kBigCap ? g_noalloc_big[kBigCap].y : (uint32_t)listed;
+    const unsigned int lane = threadIdx.x & 31;
+    const unsigned int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
+    const unsigned int share = max((total + n_warps - 1u) / n_warps, kBigSteps);
+    if ((unsigned long long)share * warp >= total) return;
+    unsigned int s = share * warp;
+    const unsigned int end = min(total - s, share) + s;
+    // the entry of step s: the last that starts at or before it
+    unsigned int e = 0u;
+    for (unsigned int len = n; len > 1u;) {
+        const unsigned int step = (len + 31u) / 32u;
+        const unsigned int at = lane * step;
+        const unsigned int le = __ballot_sync(0xffffffffu, at < len && g_noalloc_big[e + min(at, len - 1u)].y <= s);
+        const unsigned int k = (unsigned int)max(__popc(le) - 1, 0);
+        e += k * step;
+        len = min(step, len - k * step);
+    }
+    for (; s < end && e < n; ++e) {
+        const uint2 entry = g_noalloc_big[e];
         NaTri T;
-        if (t >= n_tris || !na_setup(tri, t, f, T)) continue;  // (t >= n_tris: another call's, see above)
-        const int iy = T.y0 + (int)(i % f.R);
-        if (iy > T.y1) continue;
-        for (int ix = T.x0 + lane; ix <= T.x1; ix += 32) na_texel(T, f, ix, iy, map);
+        if (entry.x >= n_tris || !na_setup(tri, entry.x, f, T)) continue;  // (entry.x >= n_tris: another call's)
+        const unsigned int steps = na_steps(T), row = na_row_steps(T);
+        unsigned int k = s - entry.y;
+        if (k >= steps) continue;  // (another call's list)
+        const unsigned int k1 = min(steps, k + (end - s));
+        s += k1 - k;
+        int iy = T.y0 + (int)(k / row);
+        unsigned int c = k % row;
+        for (; k < k1; ++k) {
+            const int ix = T.x0 + (int)(32u * c + lane);
+            if (ix <= T.x1) na_texel(T, f, ix, iy, map);
+            if (++c == row) {
+                c = 0u;
+                ++iy;
+            }
+        }
     }
 }
 
