@@ -86,19 +86,28 @@ struct NaTri {
     int x0, x1, y0, y1;
 };
 
-// Triangle t of tri; false if it covers no texel centre of the map.
+// a dx + b dy + c dz, the roundings written out.
+__device__ __forceinline__ float na_dot(float a, float b, float c, float dx, float dy, float dz)
+{
+    return __fmaf_rn(c, dz, __fmaf_rn(a, dx, __fmul_rn(b, dy)));
+}
+
+// Triangle t of tri; false if it covers no texel centre of the map.  Two
+// kernels draw triangles, and which of them draws one must not change a texel:
+// so the roundings here and in na_texel are written out, not the compiler's.
 __device__ __forceinline__ bool na_setup(const float* __restrict__ tri, int64_t t, const NaFrame& f, NaTri& T)
 {
     float x[3], y[3];
     float* d = T.d;
     for (int k = 0; k < 3; ++k) {
-        const float px = tri[9 * t + 3 * k] - f.refx, py = tri[9 * t + 3 * k + 1] - f.refy,
-                    pz = tri[9 * t + 3 * k + 2] - f.refz;
-        x[k] = (px * f.ux + py * f.uy + pz * f.uz - f.u0) * f.inv_delta;
-        y[k] = (px * f.vx + py * f.vy + pz * f.vz - f.v0) * f.inv_delta;
-        d[k] = -(px * f.sx + py * f.sy + pz * f.sz);
+        const float px = __fsub_rn(tri[9 * t + 3 * k], f.refx), py = __fsub_rn(tri[9 * t + 3 * k + 1], f.refy),
+                    pz = __fsub_rn(tri[9 * t + 3 * k + 2], f.refz);
+        x[k] = __fmul_rn(__fsub_rn(na_dot(px, py, pz, f.ux, f.uy, f.uz), f.u0), f.inv_delta);
+        y[k] = __fmul_rn(__fsub_rn(na_dot(px, py, pz, f.vx, f.vy, f.vz), f.v0), f.inv_delta);
+        d[k] = -na_dot(px, py, pz, f.sx, f.sy, f.sz);
     }
-    float area2 = (x[1] - x[0]) * (y[2] - y[0]) - (y[1] - y[0]) * (x[2] - x[0]);
+    float area2 = __fmaf_rn(__fsub_rn(x[1], x[0]), __fsub_rn(y[2], y[0]),
+                            -__fmul_rn(__fsub_rn(y[1], y[0]), __fsub_rn(x[2], x[0])));
     if (!(fabsf(area2) > 0.f)) return false;
     if (area2 < 0.f) {
         float t0 = x[1], t1 = y[1], t2 = d[1];
@@ -116,11 +125,11 @@ __device__ __forceinline__ bool na_setup(const float* __restrict__ tri, int64_t 
     if (T.x0 > T.x1 || T.y0 > T.y1) return false;
     for (int k = 0; k < 3; ++k) {
         const int a = (k + 1) % 3, b = (k + 2) % 3;
-        T.A[k] = -(y[b] - y[a]);
-        T.Bc[k] = x[b] - x[a];
-        T.C[k] = -(T.A[k] * x[a] + T.Bc[k] * y[a]);
+        T.A[k] = -__fsub_rn(y[b], y[a]);
+        T.Bc[k] = __fsub_rn(x[b], x[a]);
+        T.C[k] = -__fmaf_rn(T.Bc[k], y[a], __fmul_rn(T.A[k], x[a]));
     }
-    T.inv_a = 1.f / area2;
+    T.inv_a = __fdiv_rn(1.f, area2);
     return true;
 }
 
@@ -129,11 +138,12 @@ __device__ __forceinline__ bool na_setup(const float* __restrict__ tri, int64_t 
 __device__ __forceinline__ void na_texel(const NaTri& T, const NaFrame& f, int ix, int iy, uint32_t* map)
 {
     const float px = ix + 0.5f, py = iy + 0.5f;
-    const float w0 = T.A[0] * px + T.Bc[0] * py + T.C[0];
-    const float w1 = T.A[1] * px + T.Bc[1] * py + T.C[1];
-    const float w2 = T.A[2] * px + T.Bc[2] * py + T.C[2];
-    if (w0 >= 0.f && w1 >= 0.f && w2 >= 0.f)
-        atomicMin(&map[(int64_t)iy * f.R + ix], na_key((w0 * T.d[0] + w1 * T.d[1] + w2 * T.d[2]) * T.inv_a));
+    float w[3];
+    for (int k = 0; k < 3; ++k) w[k] = __fadd_rn(__fmaf_rn(T.Bc[k], py, __fmul_rn(T.A[k], px)), T.C[k]);
+    if (w[0] >= 0.f && w[1] >= 0.f && w[2] >= 0.f) {
+        const float d = __fmaf_rn(w[2], T.d[2], __fmaf_rn(w[1], T.d[1], __fmul_rn(w[0], T.d[0])));
+        atomicMin(&map[(int64_t)iy * f.R + ix], na_key(__fmul_rn(d, T.inv_a)));
+    }
 }
 
 // Steps of 32 texels of a row in triangle T's box.
