@@ -2681,7 +2681,17 @@ constexpr int kWarpOpen = 32;
 constexpr int kWarpKept = 80;
 constexpr int kWarpRecv = 16;
 constexpr int kTileWarps = 4;  // warps per block
-constexpr int kTileBlocks = 8; // blocks per SM (64 registers a thread)
+
+// Blocks an SM: as many as its shared memory holds.  (A bound of 8 for every
+// tile side kept 64 registers a thread and spilled 60 of them for blocks that
+// could not be resident; with 6 for 64 and 128 texels, 80 registers and no
+// spills, this kernel's share of the facade's year went from 2.82 to 2.70 ms,
+// of its report from 3.00 to 2.71, of the diffuse month from 419 to 362 us.)
+template <int TS>
+struct TileBlocks {
+    static constexpr int n = TS == 32 ? 8 : 6;
+};
+constexpr size_t kSmShared = 228 * 1024, kBlockShared = 1024;  // of an SM; taken by the system for each block
 
 template <int TS>
 __device__ constexpr uint32_t warp_bins() { return TS == 32 ? 256u : (TS == 64 ? 512u : 96u); }
@@ -2698,10 +2708,11 @@ static_assert(offsetof(WarpSm<64>, cov) % 16 == 0 && sizeof(WarpSm<64>) % 16 == 
               offsetof(WarpSm<128>, cov) % 16 == 0 && sizeof(WarpSm<128>) % 16 == 0, "rows are read as vectors");
 
 template <int TS, bool PROF>
-__global__ void __launch_bounds__(kTileWarps * 32, kTileBlocks) k_tile_warp(const WaveDev* __restrict__ W,
+__global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_warp(const WaveDev* __restrict__ W,
                                                                   const JobDev* __restrict__ jobs, Buffers B)
 {
     extern __shared__ __align__(16) unsigned char tile_smem[];  // kTileWarps WarpSm, set at launch
+    static_assert(TileBlocks<TS>::n * (kTileWarps * sizeof(WarpSm<TS>) + kBlockShared) <= kSmShared, "blocks an SM");
     constexpr int NW = TS * TS / 32;
     unsigned int p_visits = 0, p_writes = 0, p_culled = 0, p_tiles = 0, p_stiles = 0, p_hr = 0, p_hb = 0, p_ht = 0;
     const int lane = threadIdx.x & 31;
@@ -2860,7 +2871,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, kTileBlocks) k_tile_warp(cons
 template <int TS>
 struct HeavyCfg {
     static constexpr int threads = TS == 32 ? 128 : 256;
-    static constexpr int min_blocks = TS == 32 ? 8 : (TS == 64 ? 4 : 3);
+    static constexpr int min_blocks = TS == 32 ? 8 : (TS == 64 ? 4 : 2);
 };
 
 template <int TS>
@@ -2882,6 +2893,7 @@ __global__ void __launch_bounds__(HeavyCfg<TS>::threads, HeavyCfg<TS>::min_block
 {
     constexpr int NW = TS * TS / 32, kWarps = HeavyCfg<TS>::threads / 32;
     extern __shared__ __align__(16) unsigned char tile_smem[];  // HeavySm, set at launch
+    static_assert(HeavyCfg<TS>::min_blocks * (sizeof(HeavySm<TS>) + kBlockShared) <= kSmShared, "blocks an SM");
     HeavySm<TS>& sm = *reinterpret_cast<HeavySm<TS>*>(tile_smem);
     unsigned int p_visits = 0, p_writes = 0, p_culled = 0, p_tiles = 0;
     // incomplete bins (pool overflow, the wave is rerun): nothing to read
@@ -4308,7 +4320,7 @@ static void launch_tile_kernels(const WaveDev* W, const JobDev* d_jobs, const Bu
 {
     const int sm = cfg.sm_count;
     if (cfg.fused) {
-        k_tile_warp<TS, PROF><<<sm * kTileBlocks, kTileWarps * 32, kTileWarps * sizeof(WarpSm<TS>), cfg.stream>>>(
+        k_tile_warp<TS, PROF><<<sm * TileBlocks<TS>::n, kTileWarps * 32, kTileWarps * sizeof(WarpSm<TS>), cfg.stream>>>(
             W, d_jobs, b);
         if (cfg.ev) cudaEventRecord(cfg.ev[3], cfg.stream);
         k_raster_test<TS, PROF><<<sm * HeavyCfg<TS>::min_blocks, HeavyCfg<TS>::threads, sizeof(HeavySm<TS>),
