@@ -178,7 +178,8 @@ typedef struct pv3d_profile {
     int64_t heavy_tiles;       /* tiles with many receivers or triangles, taken one per block (stage 3) */
     int64_t heavy_sample_tests;   /* their share of sample_tests */
     int64_t heavy_texel_writes;   /* their share of texel_writes */
-    int64_t heavy_why[3];      /* heavy tiles by cause: too many receivers, binned triangles, kept or open triangles */
+    int64_t heavy_why[3];      /* heavy tiles by cause: too many receivers; too many binned triangles; else (kept or open
+                                  triangles, planes, or one of the largest of a wave of few tiles) */
 } pv3d_profile;
 
 /*

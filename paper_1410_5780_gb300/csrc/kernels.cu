@@ -243,6 +243,9 @@ __device__ __forceinline__ bool behind_key(float d, float bias, uint32_t key, fl
 // The largest far plane of each block of kFarBlock x kFarBlock tiles lies at
 // the start of the step's stretch of t_off, which has no other use until the
 // scan fills it.
+constexpr unsigned int kSmallWave = 4096;      // fused path: up to so many tiles those over share_bins are counted
+constexpr int kShareSteps = 3;
+__host__ __device__ constexpr unsigned int share_bins(int q) { return 8u << q; }
 constexpr int kFarSh = 3, kFarBlock = 1 << kFarSh;
 __device__ __forceinline__ int64_t far_block(int64_t te0, int tiles_x, int tx, int ty)
 {
@@ -298,6 +301,7 @@ __global__ void k_clear(const WaveDev* __restrict__ W, const JobDev* __restrict_
         B.ctr->n_touch = 0u;
         B.ctr->n_first = 0u;
         B.ctr->n_rest = 0u;
+        for (int q = 0; q < kShareSteps; ++q) B.ctr->n_over[q] = 0u;
         B.ctr->heavy_next = 0u;
     }
     const int64_t nw = 4 * W->tot_js, nt = W->tot_te;
@@ -1193,6 +1197,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_c(const WaveDev* __restri
 {
     const int64_t tot = W->tot_te;
     const int64_t n_tiles = (tot + kScanTile - 1) / kScanTile;
+    const bool small = W->fused && B.ctr->n_nonempty <= kSmallWave;
     for (int64_t st = blockIdx.x; st < n_tiles; st += gridDim.x) {
         unsigned long long x[kScanPer][3];
         unsigned long long v[3] = {0, 0, 0};
@@ -1237,6 +1242,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_c(const WaveDev* __restri
                 const unsigned int below = (1u << lane) - 1u;
                 if (first) B.nonempty[pf + __popc(bf & below)] = (uint32_t)i;
                 else if (ne) B.nonempty[tot - 1 - (int64_t)(pr + __popc(br & below))] = (uint32_t)i;
+                if (small && (bf | br)) {
+#pragma unroll
+                    for (int p = 0; p < kShareSteps; ++p) {
+                        const unsigned int bo = __ballot_sync(0xffffffffu, ne && x[q][0] > share_bins(p));
+                        if (lane == 0 && bo) atomicAdd(&B.ctr->n_over[p], (unsigned int)__popc(bo));
+                    }
+                }
             }
         }
     }
@@ -2099,18 +2111,24 @@ __global__ void __launch_bounds__(256) k_raster_map(const WaveDev* __restrict__ 
 // of each loop, none unrolled that is not short and hot.
 // ---------------------------------------------------------------------------
 
-// Planes of a tile with bits of their own; further ones share the last.
-template <int TS>
-struct Levels {
-    static constexpr int n = TS == 32 ? 12 : (TS == 64 ? 8 : 4);
-};
-
-// Of these, the ones a warp of k_tile_warp keeps (k_raster_test keeps all): the
-// less shared memory a warp takes, the more of them an SM holds.
+// Planes that a warp of k_tile_warp keeps bits of; tiles of more go to
+// k_raster_test.  The less shared memory a warp takes, the more of them an SM
+// holds.
 template <int TS>
 struct WarpLevels {
     static constexpr int n = TS == 32 ? 12 : (TS == 64 ? 8 : 1);
 };
+
+// Planes that k_raster_test keeps bits of at a time (its blocks an SM stay
+// what they are without), and in all: a tile of more of them has them drawn in
+// turns.  In a tile of more than kMaxLevels the last of a single turn stands
+// for every plane without bits of its own.
+template <int TS>
+struct PassLevels {
+    static constexpr int n = TS == 32 ? 32 : (TS == 64 ? 28 : 10);
+};
+constexpr int kMaxLevels = 64;
+static_assert(kMaxLevels >= kRecvChunk, "a tile that culls by all planes (Level::cull) has all of them in its list");
 
 template <int TS>
 struct TileSh {  // log2 of the tile side
@@ -2134,19 +2152,24 @@ struct Level {
 // tile that shades every sample of every receiver, or 1 + the 16-byte offset
 // of the tile's record in the pool B.cov:
 //   word 0      levels | kRecOpen | kRecDepth | kRecHeavy | open triangles << 16
-//   words 1-12  plane group of each level
-//   words 13-24 box of each level's covered and open texels, x0 | x1 << 8 | y0
-//               << 16 | y1 << 24 (kBoxNone: none)
-//   word 28 ... TS * TS / 32 words of coverage bits per level (bit x & 31 of
+//   word 4 ...  plane group of each level, as many words as a multiple of four
+//               holds (kNoPlane in the others)
+//   then        box of each level's covered and open texels, x0 | x1 << 8 | y0
+//               << 16 | y1 << 24 (kBoxNone: none), as many words
+//   then        TS * TS / 32 words of coverage bits per level (bit x & 31 of
 //               word y * TS / 32 + x / 32)
 // and, with kRecOpen, as many words of open texels, then the open triangles
 // (TriS, 12 words each) or, with kRecDepth, TS * TS depth keys.
 constexpr uint32_t kTileLit = 0u;
 constexpr uint32_t kTileFull = 0xFFFFFFFFu, kTileFullHeavy = 0xFFFFFFFEu;  // (heavy: k_raster_test's, for the counters)
 constexpr uint32_t kRecLevels = 0xFFu, kRecOpen = 1u << 8, kRecDepth = 1u << 9, kRecHeavy = 1u << 10;
-constexpr int kRecHead = 28, kRecBox = 13;
+constexpr int kRecPlane = 4;
+constexpr uint32_t kNoPlane = 0xFFFFFFFEu;
 constexpr uint32_t kBoxNone = 0x000000FFu;
-static_assert(Levels<32>::n <= 12 && Levels<64>::n <= 12 && Levels<128>::n <= 12, "record header");
+__device__ __forceinline__ int rec_planes(int nl) { return (nl + 3) & ~3; }
+__device__ __forceinline__ int rec_box(int nl) { return kRecPlane + rec_planes(nl); }
+__device__ __forceinline__ int rec_head(int nl) { return kRecPlane + 2 * rec_planes(nl); }
+static_assert(kMaxLevels <= (int)kRecLevels, "record header");
 
 // A triangle set up for the sample-driven test (48 bytes, three 16-byte loads):
 // edge functions k = 0..2 in tile-local texel coordinates and depths scaled by
@@ -2240,14 +2263,13 @@ __device__ __forceinline__ bool order_levels(Level* lv, int nl)
     return __all_sync(0xffffffffu, ok);
 }
 
-// The levels of tile te, for one full warp; returns their number, and whether
-// they are nested (order_levels).  A tile of one plane group takes the plane
-// from any of its modules (t_roff), others go through the receiver list.
+// The levels of tile te, at most `cap`, for one full warp; returns their
+// number, or cap + 1 if there are more.  A tile of one plane group takes the
+// plane from any of its modules (t_roff), others go through the receiver list.
 template <int TS>
-__device__ __forceinline__ int build_levels(Level* lv, const JobDev& J, const Buffers& B, const WaveDev* W, uint32_t te,
-                                            int ls, int tx, int ty, uint32_t plane, bool& nested)
+__device__ __forceinline__ int build_levels(Level* lv, int cap, const JobDev& J, const Buffers& B, const WaveDev* W,
+                                            uint32_t te, int ls, int tx, int ty, uint32_t plane)
 {
-    nested = false;
     const int lane = threadIdx.x & 31;
     const ModStep* ms = B.ms + J.ms_base + (int64_t)ls * J.n_mods;
     const uint32_t r0 = B.t_roff[te];
@@ -2270,25 +2292,15 @@ __device__ __forceinline__ int build_levels(Level* lv, const JobDev& J, const Bu
         unsigned int todo = __ballot_sync(0xffffffffu, !known);
 #pragma unroll 1
         while (todo) {
+            if (nl == cap) return cap + 1;
             const int lead = __ffs((int)todo) - 1;
             const int p = __shfl_sync(0xffffffffu, pl, lead);
             todo &= ~__ballot_sync(0xffffffffu, have && pl == p);
-            if (lane == lead) {
-                if (nl < Levels<TS>::n) {
-                    fill_level<TS>(lv[nl], ms[m], pl, tx, ty, cull);
-                } else {
-                    Level& L = lv[Levels<TS>::n - 1];
-                    L.pa = L.pb = L.pc = 0.f;
-                    L.front = L.back = INFINITY;
-                    L.cull = -1.f;
-                    L.plane = -1;
-                }
-            }
-            if (nl < Levels<TS>::n) ++nl;
+            if (lane == lead) fill_level<TS>(lv[nl], ms[m], pl, tx, ty, cull);
+            ++nl;
             __syncwarp();
         }
     }
-    if (nl > 1) nested = order_levels<TS>(lv, nl);
     return nl;
 }
 
@@ -2304,9 +2316,10 @@ struct TriWork {
     bool whole;            // covers every texel centre of the tile
 };
 
-// Set up binned triangle t of tile (ox, oy); front = deep = 0 if it covers no
-// texel centre of the tile or is behind every level, or lies in or behind the
-// planes of all.
+// Set up binned triangle t of tile (ox, oy) for levels [s0, s0 + np) of nl (bit
+// l of front and deep: level s0 + l); front = deep = 0 if it covers no texel
+// centre of the tile or is behind every level, or lies in or behind the planes
+// of all nl.
 //
 // The triangle's depth less a plane's is linear, so over the tile it lies
 // between its values at the vertices, up to what rounding makes of the depth
@@ -2320,8 +2333,8 @@ struct TriWork {
 // Twice that is allowed for, and 1e-5 of the plane's terms at the vertices.
 template <int TS, bool PROF>
 __device__ __forceinline__ void classify_tri(const JobDev& J, const Buffers& B, const LightParams& lp, int ls, int t,
-                                             float ox, float oy, const Level* lv, int nl, TriWork& w,
-                                             unsigned int& culled)
+                                             float ox, float oy, const Level* lv, int nl, int s0, int np,
+                                             TriWork& w, unsigned int& culled)
 {
     tri_texel(J, B, lp, ls, t, w.T);
     TriT& T = w.T;
@@ -2349,11 +2362,12 @@ __device__ __forceinline__ void classify_tri(const JobDev& J, const Buffers& B, 
         }
         const float tol = err + 1e-5f * (fabsf(pa) * xm + fabsf(pb) * ym);
         keep = keep || lv[l].cull < 0.f || !(lo >= -lv[l].cull);
-        if (hi + tol < -lv[l].front) w.front |= 1u << l;
-        else if (!(lo - tol >= lv[l].back)) w.deep |= 1u << l;
+        const uint32_t bit = l >= s0 && l < s0 + np ? 1u << (l - s0) : 0u;
+        if (hi + tol < -lv[l].front) w.front |= bit;
+        else if (!(lo - tol >= lv[l].back)) w.deep |= bit;
     }
     if (!keep) w.deep = 0u;  // (front none)
-    if (PROF && !(w.front | w.deep)) ++culled;
+    if (PROF && s0 == 0 && !(w.front | w.deep)) ++culled;
     // each edge at the texel centre farthest outside it (edge_at is monotone
     // in px and py)
     if (w.x0 == 0 && w.y0 == 0 && w.x1 == TS - 1 && w.y1 == TS - 1) {
@@ -2416,13 +2430,29 @@ __device__ __forceinline__ bool below(float ga, float gb, float T, float margin,
 // triangles share the warp.  (128 texels, the facade year: 4.7 -> 3.9 ms for
 // k_tile_warp; 64 texels, 45 suns over 13 modules: 68 -> 53 us.)
 //
+// k_raster_test: threads of a block, blocks an SM.
+template <int TS>
+struct HeavyCfg {
+    static constexpr int threads = TS == 32 ? 128 : 256;
+    static constexpr int stride = TS + 1;  // of a row of depths: the lanes' rows lie in different banks
+    static constexpr int min_blocks = TS == 32 ? 8 : (TS == 64 ? 4 : 2);
+};
+
+// A row's texels between those in front of a plane and those behind it are
+// compared one by one up to so many, above that as a span.  (A steep plane's
+// band may be as wide as the tile: with this, and the depths of a row's open
+// texels drawn once in place of once a level, k_raster_test took 117 us in
+// place of 158 for 25 modules of all orientations, 47 suns, R = 512.)
+constexpr float kBandTexels = 6.f;
+
 // Draw the warp's triangles (w, one per lane; `full`: the levels covered
 // everywhere, neither drawn nor compared any more): row spans into the coverage bits of the levels they are in
 // front of (cov, TS * TS / 32 words each; nested levels: of the first of them
 // only, finish_words adds the bits to the levels after it), and for the levels
-// they cross, each texel compared with the plane: in front, a coverage bit; in
-// the band, open.  `open` (level-free): the open texels' bits; with TILE, their nearest depth in
-// `tile` too.  D.open receives the triangles that left a texel open.
+// they cross, the texels in front of the plane as coverage bits and those in
+// the band as open.  `open` (level-free): the open texels' bits; with TILE,
+// their nearest depth in `tile` too.  D.open receives the triangles that left
+// a texel open.
 template <int TS, bool TILE, bool PROF>
 __device__ __forceinline__ void draw_tris(DrawSm& D, const TriWork& w, uint32_t full, bool nested, const Level* lv,
                                           uint32_t* cov,
@@ -2493,49 +2523,70 @@ __device__ __forceinline__ void draw_tris(DrawSm& D, const TriWork& w, uint32_t 
             return depth_at(__fmaf_rn(A0, px, tk[0]), __fmaf_rn(A1, px, tk[1]), __fmaf_rn(A2, px, tk[2]), e0, e1, e2);
         };
         const float pl = a + 0.5f, ph = b + 0.5f, dl = depth_px(pl), dh = depth_px(ph), err2 = 2.f * S.err;
+        uint32_t left[TILE ? WPR : 1] = {};  // the row's open texels
 #pragma unroll 1
         for (; m; m &= m - 1u) {
             const int l = __ffs((int)m) - 1;
             const float pa = lv[l].pa, base = __fmaf_rn(lv[l].pb, py, lv[l].pc);
             const float fr = -lv[l].front, bk = lv[l].back;
             // the gap is linear along the row, up to the depths' rounding: its
-            // ends tell which texels are in front and which are behind, but
+            // ends tell which texels are in front and which are behind, and
+            // where there are many others which of them are in the band, but
             // for those about the roots
             const float ga = dl - __fmaf_rn(pa, pl, base), gb = dh - __fmaf_rn(pa, ph, base);
-            float fa = a, fb = b, ca = a, cb = b;
+            float fa = a, fb = b, ca = a, cb = b;          // in front; not behind
+            float ia = a, ib = a - 1.f, ja = a, jb = a - 1.f;  // in the band: [ia, ib] less [ja, jb]
             if (!below(ga, gb, fr - err2, -0.02f, fa, fb)) fb = fa - 1.f;
             if (!below(ga, gb, bk + err2, 0.02f, ca, cb)) continue;
+            if ((cb - ca) - (fb - fa) > kBandTexels) {
+                ib = jb = b;
+                if (!below(ga, gb, bk - err2, -0.02f, ia, ib)) ib = ia - 1.f;
+                if (!below(ga, gb, fr + err2, 0.02f, ja, jb)) jb = ja - 1.f;
+            }
             const int f0 = (int)fa, f1 = (int)fb, c0 = (int)ca, c1 = (int)cb;
+            const int i0 = (int)ia, i1 = (int)ib, j0 = (int)ja, j1 = (int)jb;
 #pragma unroll 1
             for (int q = c0 >> 5; q <= (c1 >> 5); ++q) {
                 const int word = iy * WPR + q;
-                uint32_t c = f0 <= f1 && q >= (f0 >> 5) && q <= (f1 >> 5) ? span_word(f0, f1, q) : 0u, o = 0u;
+                uint32_t c = span_word(f0, f1, q);
                 uint32_t r = span_word(c0, c1, q) & ~c & ~cov[l * NW + word];
-                if (!(bk < FLT_MAX)) {  // no plane to compare with: open
-                    o = r;
-                    for (r = TILE ? r : 0u; r; r &= r - 1u) {
-                        const int x = 32 * q + __ffs((int)r) - 1;
-                        if (PROF) ++writes;
-                        atomicMin(&tile[iy * TS + x], depth_store_key(depth_px((float)x + 0.5f), lp, u24));
-                    }
-                }
+                uint32_t o = r & span_word(i0, i1, q) & ~span_word(j0, j1, q);
 #pragma unroll 1
-                for (; r; r &= r - 1u) {
+                for (r &= ~o; r; r &= r - 1u) {
                     const int x = __ffs((int)r) - 1;
                     const float px = (float)(32 * q + x) + 0.5f;
-                    const float depth = depth_px(px), gap = depth - __fmaf_rn(pa, px, base);
+                    const float gap = depth_px(px) - __fmaf_rn(pa, px, base);
                     if (PROF) ++writes;
-                    if (gap < fr) {
-                        c |= 1u << x;
-                    } else if (!(gap >= bk)) {
-                        o |= 1u << x;
-                        if (TILE) atomicMin(&tile[iy * TS + 32 * q + x], depth_store_key(depth, lp, u24));
-                    }
+                    if (gap < fr) c |= 1u << x;
+                    else if (!(gap >= bk)) o |= 1u << x;
                 }
                 if (c) atomicOr(&cov[l * NW + word], c);
                 if (o) {
                     atomicOr(&open[word], o);
                     atomicOr(&D.open, 1u << t);
+                    if (TILE) {
+#pragma unroll
+                        for (int k = 0; k < WPR; ++k) left[k] |= k == q ? o : 0u;
+                    }
+                }
+            }
+        }
+        // the depths of the row's open texels, of all levels together (each a
+        // chain of 25 dependent instructions: four at a time, 25 modules of all
+        // orientations on 128-texel tiles, 47 suns, went from 805 to 600 us)
+        if constexpr (TILE) {
+#pragma unroll 1
+            for (int q = lo >> 5; q <= (hi >> 5); ++q) {
+                uint32_t r = 0u;
+#pragma unroll
+                for (int k = 0; k < WPR; ++k) r |= k == q ? left[k] : 0u;
+                if (r == 0u) continue;
+                const int x0 = __ffs((int)r) - 1, x1 = 31 - __clz((int)r);
+                uint32_t* dst = &tile[iy * HeavyCfg<TS>::stride + 32 * q];
+#pragma unroll 4
+                for (int x = x0; x <= x1; ++x) {
+                    const uint32_t key = depth_store_key(depth_px((float)(32 * q + x) + 0.5f), lp, u24);
+                    if ((r >> x) & 1u) atomicMin(&dst[x], key);
                 }
             }
         }
@@ -2594,7 +2645,7 @@ __device__ __forceinline__ void for_levels(const uint32_t* cov, int nl, bool nes
 template <int TS>
 __device__ __forceinline__ uint32_t full_levels(const uint32_t* cov, int nl, bool nested, uint32_t full)
 {
-    uint32_t ok = (1u << nl) - 1u;
+    uint32_t ok = (2u << (nl - 1)) - 1u;
 #pragma unroll 1
     for (int q = threadIdx.x & 31; q < TS * TS / 32; q += 32)
         for_levels<TS>(cov, nl, nested, full, q, [&](int l, uint32_t c) {
@@ -2660,7 +2711,8 @@ __device__ __forceinline__ uint32_t texel_box(const uint32_t* cov, const uint32_
 
 // ---------------------------------------------------------------------------
 // k_tile_warp: fused path -- one warp per non-empty tile: the tile's coverage
-// bits.  A tile with more than warp_bins() binned triangles or more than
+// bits.  A tile of more planes than WarpLevels, with more than warp_bins()
+// binned triangles (fewer in waves of few tiles, see below) or more than
 // kWarpOpen that leave texels open, and a 64-texel tile with more than
 // kWarpRecv receivers or more than kWarpKept triangles in front of or across a
 // level, is listed for k_raster_test.  A tile is a small
@@ -2700,7 +2752,7 @@ template <int TS>
 struct __align__(16) WarpSm {
     TriS tri[kWarpOpen];
     DrawSm d;
-    Level lv[Levels<TS>::n];
+    Level lv[WarpLevels<TS>::n];
     __align__(16) uint32_t cov[WarpLevels<TS>::n * TS * TS / 32];  // draw_tris takes a row at once
     uint32_t open[TS * TS / 32];
 };
@@ -2725,10 +2777,24 @@ __global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_war
     const unsigned int n_first = B.ctr->n_first, last = (unsigned int)(W->tot_te - 1);
     const int nj = W->n_jobs;
     const int u24 = W->depth_u24;
-    // with a tile or less for each resident warp the largest tile is the
-    // kernel's time: 32 triangles of up to 128 rows are enough for a warp
-    // (77 facade modules, 72 suns: both tile kernels 353 us with 96, 240 with 32)
-    const uint32_t most = TS == 128 && n_ne <= gridDim.x * (unsigned int)kTileWarps ? 32u : warp_bins<TS>();
+    // with few tiles the largest is the kernel's time.  128 texels, a tile or
+    // less for each resident warp: 32 triangles of up to 128 rows are enough
+    // for a warp (77 facade modules, 72 suns: both tile kernels 353 us with 96,
+    // 240 with 32).  Smaller tiles: where some are large, as many of the
+    // largest as k_raster_test's blocks take in two rounds go to a block's eight
+    // warps (25 modules on planes of their own, R = 512, 47 suns, 652 tiles of
+    // up to 163 triangles: both 452 us, now 140; the call 641, now 345.  With
+    // one round for the limit 50 modules, 100 suns, took 1 to 15 % longer; tiles
+    // of at most 48 triangles are a warp's in any case: their blocks cost as
+    // much as they save)
+    uint32_t most = warp_bins<TS>();
+    if (TS == 128) {
+        if (n_ne <= gridDim.x * (unsigned int)kTileWarps) most = 32u;
+    } else if (n_ne <= kSmallWave && n_first > 0u) {
+        const unsigned int blocks = gridDim.x / TileBlocks<TS>::n * HeavyCfg<TS>::min_blocks;
+        for (int q = kShareSteps; q-- > 0;)
+            if (B.ctr->n_over[q] <= 2u * blocks) most = share_bins(q);
+    }
     unsigned int next = 0;
     if (lane == 0) next = atomicAdd(&B.ctr->raster_next, 1u);
     next = __shfl_sync(0xffffffffu, next, 0);
@@ -2747,13 +2813,14 @@ __global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_war
         bool heavy = crowd || cnt > most;
         if (PROF && lane == 0) {
             if (crowd) ++p_hr;
-            else if (heavy) ++p_hb;
+            else if (heavy && cnt > warp_bins<TS>()) ++p_hb;
+            else if (heavy) ++p_ht;
         }
         if (!heavy) {
             const LightParams& lp = B.lp[J.js_base + ls];
-            bool nested;
-            const int nl = build_levels<TS>(sm.lv, J, B, W, te, ls, tx, ty, plane, nested);
+            const int nl = build_levels<TS>(sm.lv, WarpLevels<TS>::n, J, B, W, te, ls, tx, ty, plane);
             heavy = nl > WarpLevels<TS>::n;
+            const bool nested = !heavy && nl > 1 && order_levels<TS>(sm.lv, nl);
 #pragma unroll 4
             for (int q = lane; q < (heavy ? 0 : nl * NW); q += 32) sm.cov[q] = 0u;
 #pragma unroll 4
@@ -2769,7 +2836,8 @@ __global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_war
                 w.front = w.deep = 0u;
                 w.whole = false;
                 if (b0 + lane < cnt)
-                    classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, w, p_culled);
+                    classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, 0, nl, w,
+                                           p_culled);
                 full = full_after(full | __reduce_or_sync(0xffffffffu, w.whole ? w.front : 0u), nested, all);
                 const unsigned int use = __ballot_sync(0xffffffffu, (w.front | w.deep) != 0u);
                 kept += __popc(use);
@@ -2809,19 +2877,20 @@ __global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_war
                     } else if (n == 0 && !__any_sync(0xffffffffu, some != 0u)) {
                         state = kTileLit;
                     } else {
-                        const uint32_t words = (uint32_t)(kRecHead + nl * NW + (n ? NW + 12 * n : 0));
+                        const uint32_t words = (uint32_t)(rec_head(nl) + nl * NW + (n ? NW + 12 * n : 0));
                         if (lane == 0) state = alloc_record(B, W, words);
                         state = __shfl_sync(0xffffffffu, state, 0);
                         if (state) {
                             uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
                             if (lane == 0) rec[0] = (uint32_t)nl | (n ? kRecOpen | ((uint32_t)n << 16) : 0u);
-                            else if (lane <= nl) rec[lane] = (uint32_t)sm.lv[lane - 1].plane;
+                            if (lane < rec_planes(nl))
+                                rec[kRecPlane + lane] = lane < nl ? (uint32_t)sm.lv[lane].plane : kNoPlane;
 #pragma unroll 1
                             for (int l = 0; l < nl; ++l) {
                                 const uint32_t box = texel_box<TS>(sm.cov + l * NW, sm.open);
-                                if (lane == 0) rec[kRecBox + l] = box;
+                                if (lane == 0) rec[rec_box(nl) + l] = box;
                             }
-                            uint32_t* dst = rec + kRecHead;
+                            uint32_t* dst = rec + rec_head(nl);
                             for (int q = lane; q < nl * NW; q += 32) dst[q] = sm.cov[q];
                             if (n) {
                                 dst += nl * NW;
@@ -2865,22 +2934,19 @@ __global__ void __launch_bounds__(kTileWarps * 32, TileBlocks<TS>::n) k_tile_war
 // tile, its warps taking up to 32 triangles at a time by themselves (as many
 // each: with 32 for some and none for others the facade year's share of this
 // kernel was 0.96 ms, now 0.63); texels left open keep their nearest depth in
-// a shared tile that goes to the record.  Bound by the longest tile: there are
+// a shared tile that goes to the record.  Tiles of more planes than have bits
+// at a time are drawn in turns: 50 modules on planes of their own, 128-texel
+// tiles, 100 suns: the call 1,045 us with all but three planes left open
+// throughout, 660 with ten at a time.  Bound by the longest tile: there are
 // fewer than blocks in most waves.
 // ---------------------------------------------------------------------------
 template <int TS>
-struct HeavyCfg {
-    static constexpr int threads = TS == 32 ? 128 : 256;
-    static constexpr int min_blocks = TS == 32 ? 8 : (TS == 64 ? 4 : 2);
-};
-
-template <int TS>
 struct __align__(16) HeavySm {
-    uint32_t tile[TS * TS];  // nearest depth keys of open texels
-    uint32_t cov[Levels<TS>::n * TS * TS / 32];
+    uint32_t tile[TS * HeavyCfg<TS>::stride];  // nearest depth keys of open texels
+    uint32_t cov[PassLevels<TS>::n * TS * TS / 32];
     uint32_t open[TS * TS / 32];
     DrawSm d[HeavyCfg<TS>::threads / 32];
-    Level lv[Levels<TS>::n];
+    Level lv[kMaxLevels];
     int nl;
     int nested;
     uint32_t full, state;
@@ -2918,80 +2984,113 @@ __global__ void __launch_bounds__(HeavyCfg<TS>::threads, HeavyCfg<TS>::min_block
         const JobDev& J = jobs[j];
         const LightParams& lp = B.lp[J.js_base + ls];
         if (warp == 0) {
-            bool nested;
-            const int nl = build_levels<TS>(sm.lv, J, B, W, te, ls, tx, ty, B.t_plane[te], nested);
-            if (lane == 0) {
-                sm.nl = nl;
-                sm.nested = nested;
-                sm.full = 0u;
+            int nl = build_levels<TS>(sm.lv, kMaxLevels, J, B, W, te, ls, tx, ty, B.t_plane[te]);
+            if (nl > kMaxLevels) {
+                nl = PassLevels<TS>::n;
+                if (lane == 0) {
+                    Level& L = sm.lv[nl - 1];
+                    L.pa = L.pb = L.pc = 0.f;
+                    L.front = L.back = INFINITY;
+                    L.cull = -1.f;
+                    L.plane = -1;
+                }
             }
+            if (lane == 0) sm.nl = nl;
         }
         uint4* t4 = reinterpret_cast<uint4*>(sm.tile);
-        for (int q = tid; q < TS * TS / 4; q += bd) t4[q] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
-        for (int q = tid; q < Levels<TS>::n * NW; q += bd) sm.cov[q] = 0u;
+        for (int q = tid; q < TS * HeavyCfg<TS>::stride / 4; q += bd) t4[q] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
         for (int q = tid; q < NW; q += bd) sm.open[q] = 0u;
         if (PROF && tid == 0) ++p_tiles;
         __syncthreads();
         const int nl = sm.nl;
-        const bool nested = sm.nested != 0;
-        const uint32_t all = (1u << nl) - 1u;
         const float ox = (float)(tx * TS), oy = (float)(ty * TS);
-        uint32_t full = 0u;
-        // up to 32 triangles a warp and turn, the same number for each
-        const uint32_t turns = (cnt + 32u * kWarps - 1u) / (32u * kWarps);
-        const uint32_t share = (cnt + kWarps * turns - 1u) / (kWarps * turns);
+        // turns of as many levels each; up to 32 triangles a warp and round, the
+        // same number for each
+        const int n_turns = (nl + PassLevels<TS>::n - 1) / PassLevels<TS>::n, per = (nl + n_turns - 1) / max(n_turns, 1);
+        const uint32_t rounds = (cnt + 32u * kWarps - 1u) / (32u * kWarps);
+        const uint32_t share = (cnt + kWarps * rounds - 1u) / (kWarps * rounds);
+        bool any_hole = false, any_open = false, any_some = false;
+        uint32_t state = kTileLit;
+        uint32_t* rec = nullptr;
 #pragma unroll 1
-        for (uint32_t b0 = share * warp; b0 < cnt; b0 += share * kWarps) {
-            full |= *(volatile uint32_t*)&sm.full;
-            full = __reduce_or_sync(0xffffffffu, full);
-            if (full == all) break;  // every sample of the tile is shaded
-            TriWork w;
-            w.front = w.deep = 0u;
-            w.whole = false;
-            if ((uint32_t)lane < share && b0 + lane < cnt)
-                classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, w, p_culled);
-            const uint32_t f = full_after(__reduce_or_sync(0xffffffffu, w.whole ? w.front : 0u), nested, all);
-            if (f & ~full) {
-                full |= f;
-                if (lane == 0) atomicOr(&sm.full, f);
+        for (int s0 = 0; s0 < nl; s0 += per) {
+            const int np = min(per, nl - s0);
+            if (warp == 0) {
+                const bool nested = np > 1 && order_levels<TS>(sm.lv + s0, np);
+                if (lane == 0) {
+                    sm.nested = nested;
+                    sm.full = 0u;
+                }
             }
-            if (full == all || !__any_sync(0xffffffffu, (w.front | w.deep) != 0u)) continue;
-            draw_tris<TS, true, PROF>(sm.d[warp], w, full, nested, sm.lv, sm.cov, sm.open, sm.tile, lp, u24, p_visits,
-                                      p_writes);
-            if (b0 + share * kWarps < cnt) full = full_levels<TS>(sm.cov, nl, nested, full);
-        }
-        __syncthreads();
-        full = sm.full;
-        uint32_t some = 0u, hole = 0u, op = 0u;
-        finish_words<TS>(sm.cov, nl, nested, full, tid, bd, some, hole);
-        for (int q = tid; q < NW; q += bd) op |= sm.open[q];
-        const bool any_hole = __syncthreads_or(hole != 0u), any_open = __syncthreads_or(op != 0u),
-                   any_some = __syncthreads_or(some != 0u);
-        uint32_t state = !any_hole ? kTileFullHeavy : kTileLit;
-        if (any_hole && (any_some || any_open)) {
-            const uint32_t words = (uint32_t)(kRecHead + nl * NW + (any_open ? NW + TS * TS : 0));
-            if (tid == 0) sm.state = alloc_record(B, W, words);
+            for (int q = tid; q < np * NW; q += bd) sm.cov[q] = 0u;
             __syncthreads();
-            state = sm.state;
-            if (state) {
-                uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
-                if (tid == 0) rec[0] = (uint32_t)nl | kRecHeavy | (any_open ? kRecOpen | kRecDepth : 0u);
-                else if (tid <= nl) rec[tid] = (uint32_t)sm.lv[tid - 1].plane;
+            const Level* lv = sm.lv + s0;
+            const bool nested = sm.nested != 0;
+            const uint32_t all = (2u << (np - 1)) - 1u;
+            uint32_t full = 0u;
 #pragma unroll 1
-                for (int l = warp; l < nl; l += kWarps) {
+            for (uint32_t b0 = share * warp; b0 < cnt; b0 += share * kWarps) {
+                full |= *(volatile uint32_t*)&sm.full;
+                full = __reduce_or_sync(0xffffffffu, full);
+                if (full == all) break;  // every sample of these levels is shaded
+                TriWork w;
+                w.front = w.deep = 0u;
+                w.whole = false;
+                if ((uint32_t)lane < share && b0 + lane < cnt)
+                    classify_tri<TS, PROF>(J, B, lp, ls, (int)B.bins[off + b0 + lane], ox, oy, sm.lv, nl, s0, np, w,
+                                           p_culled);
+                const uint32_t f = full_after(__reduce_or_sync(0xffffffffu, w.whole ? w.front : 0u), nested, all);
+                if (f & ~full) {
+                    full |= f;
+                    if (lane == 0) atomicOr(&sm.full, f);
+                }
+                if (full == all || !__any_sync(0xffffffffu, (w.front | w.deep) != 0u)) continue;
+                draw_tris<TS, true, PROF>(sm.d[warp], w, full, nested, lv, sm.cov, sm.open, sm.tile, lp, u24, p_visits,
+                                          p_writes);
+                if (b0 + share * kWarps < cnt) full = full_levels<TS>(sm.cov, np, nested, full);
+            }
+            __syncthreads();
+            full = sm.full;
+            uint32_t some = 0u, hole = 0u, op = 0u;
+            finish_words<TS>(sm.cov, np, nested, full, tid, bd, some, hole);
+            if (s0 + per >= nl)
+                for (int q = tid; q < NW; q += bd) op |= sm.open[q];
+            any_hole |= __syncthreads_or(hole != 0u) != 0;
+            any_open |= __syncthreads_or(op != 0u) != 0;
+            any_some |= __syncthreads_or(some != 0u) != 0;
+            // the record: once it is known to be needed, or before the bits of
+            // the first of several turns are replaced
+            if (s0 == 0 && (n_turns > 1 || (any_hole && (any_some || any_open)))) {
+                const uint32_t words = (uint32_t)(rec_head(nl) + nl * NW + (any_open || n_turns > 1 ? NW + TS * TS : 0));
+                if (tid == 0) sm.state = alloc_record(B, W, words);
+                __syncthreads();
+                state = sm.state;
+                if (state) rec = B.cov + 4 * (size_t)(state - 1u);
+            }
+            if (rec) {
+#pragma unroll 1
+                for (int l = warp; l < np; l += kWarps) {
                     const uint32_t box = texel_box<TS>(sm.cov + l * NW, sm.open);
-                    if (lane == 0) rec[kRecBox + l] = box;
+                    if (lane == 0) rec[rec_box(nl) + s0 + l] = box;
                 }
-                uint32_t* dst = rec + kRecHead;
-                for (int q = tid; q < nl * NW; q += bd) dst[q] = sm.cov[q];
-                if (any_open) {
-                    dst += nl * NW;
-                    for (int q = tid; q < NW; q += bd) dst[q] = sm.open[q];
-                    dst += NW;
-                    for (int q = tid; q < TS * TS; q += bd) dst[q] = sm.tile[q];
-                }
+                if (tid < np) rec[kRecPlane + s0 + tid] = (uint32_t)lv[tid].plane;
+                uint32_t* dst = rec + rec_head(nl) + s0 * NW;
+                for (int q = tid; q < np * NW; q += bd) dst[q] = sm.cov[q];
+            }
+            __syncthreads();  // the bits may be replaced
+        }
+        if (rec) {
+            if (tid == 0) rec[0] = (uint32_t)nl | kRecHeavy | (any_open ? kRecOpen | kRecDepth : 0u);
+            if (nl + tid < rec_planes(nl)) rec[kRecPlane + nl + tid] = kNoPlane;
+            if (any_open) {
+                uint32_t* dst = rec + rec_head(nl) + nl * NW;
+                for (int q = tid; q < NW; q += bd) dst[q] = sm.open[q];
+                dst += NW;
+                for (int q = tid; q < TS * TS; q += bd) dst[q] = sm.tile[q + q / TS * (HeavyCfg<TS>::stride - TS)];
             }
         }
+        if (!any_hole) state = kTileFullHeavy;
+        else if (!any_some && !any_open) state = kTileLit;
         if (tid == 0) B.t_cnt[te] = state;
         __syncthreads();  // the tile's shared memory may be reused
     }
@@ -3101,14 +3200,20 @@ constexpr int kCellWarps = 8, kCellBlocks = 4;  // warps a block, blocks an SM
 __device__ __forceinline__ int level_of(const uint32_t* rec, uint32_t h, int plane)
 {
     const int nl = (int)(h & kRecLevels);
-    int l = 0;
+    const uint4* p = reinterpret_cast<const uint4*>(rec + kRecPlane);
 #pragma unroll 1
-    while (l < nl - 1 && (int)rec[1 + l] != plane) ++l;  // the last level takes every other plane
-    return l;
+    for (int l = 0; l < nl - 1; l += 4) {
+        const uint4 v = p[l >> 2];
+        if (v.x == (uint32_t)plane) return l;
+        if (v.y == (uint32_t)plane) return l + 1;
+        if (v.z == (uint32_t)plane) return l + 2;
+        if (v.w == (uint32_t)plane) return l + 3;
+    }
+    return nl - 1;  // the last level takes every other plane
 }
 __device__ __forceinline__ const uint32_t* level_words(const uint32_t* rec, uint32_t h, int plane, int words)
 {
-    return rec + kRecHead + level_of(rec, h, plane) * words;
+    return rec + rec_head((int)(h & kRecLevels)) + level_of(rec, h, plane) * words;
 }
 
 // The words of a row of TS / 32 coverage words, together.
@@ -3153,7 +3258,7 @@ __device__ __forceinline__ bool sample_shaded(const Buffers& B, const uint32_t* 
     const int lx = ix & (TS - 1), ly = iy & (TS - 1), word = ly * WPR + (lx >> 5);
     if ((level_words(rec, h, plane, NW)[word] >> (lx & 31)) & 1u) return true;
     if (!(h & kRecOpen)) return false;
-    const uint32_t* open = rec + kRecHead + (int)(h & kRecLevels) * NW;
+    const uint32_t* open = rec + rec_head((int)(h & kRecLevels)) + (int)(h & kRecLevels) * NW;
     if (!((open[word] >> (lx & 31)) & 1u)) return false;
     if (h & kRecDepth) {
         const uint32_t key = open[NW + ly * TS + lx];
@@ -3277,7 +3382,8 @@ __device__ __forceinline__ int cell_shaded(const Buffers& B, const JobDev& J, co
                     const uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
                     const uint32_t h = rec[0];
                     w = level_words(rec, h, plane, NW);
-                    if (h & kRecOpen) o = (int)(rec + kRecHead + (int)(h & kRecLevels) * NW - w);
+                    const int nl = (int)(h & kRecLevels);
+                    if (h & kRecOpen) o = (int)(rec + rec_head(nl) + nl * NW - w);
                 }
                 if (!big) {
                     const int q = lx0 >> 5, col = (tx << SH) + lx0 - x0, row = (ty << SH) + ly0 - y0;
@@ -3469,7 +3575,8 @@ __device__ __forceinline__ void add_tile_box(const Buffers& B, const JobDev& J, 
     uint32_t box = (uint32_t)side << 8 | (uint32_t)side << 24;
     if (state < kTileFullHeavy) {
         const uint32_t* rec = B.cov + 4 * (size_t)(state - 1u);
-        box = rec[kRecBox + level_of(rec, rec[0], J.mods[m].plane)];
+        const uint32_t h = rec[0];
+        box = rec[rec_box((int)(h & kRecLevels)) + level_of(rec, h, J.mods[m].plane)];
     }
     if (box == kBoxNone) return;
     x0 = min(x0, (tx << sh) + (int)(box & 255u));

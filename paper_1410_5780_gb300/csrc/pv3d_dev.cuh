@@ -186,6 +186,7 @@ struct Counters {
     unsigned int heavy_next;  // k_raster_test's work counter
     unsigned int n_touch;     // modules listed for k_cells
     unsigned int n_first, n_rest;  // fused path: tiles listed from the front and from the end of nonempty
+    unsigned int n_over[3];        // fused path, few tiles: tiles of more than share_bins() triangles
     unsigned long long tot_bins;
     unsigned long long tot_recv;
     unsigned long long need_recv;
@@ -211,7 +212,7 @@ struct Counters {
     unsigned long long prof_h_samples;  // of prof_samples, prof_writes and prof_tiles: the share of the
     unsigned long long prof_h_writes;   //   kernel that takes the heavy tiles (one block per tile)
     unsigned long long prof_h_tiles;
-    unsigned long long prof_heavy_why[3];  // heavy because of: receivers, binned triangles, kept or open triangles
+    unsigned long long prof_heavy_why[3];  // heavy because of: receivers, binned triangles, else
 };
 
 // Scratch and pools, sized by the host for the largest wave.
