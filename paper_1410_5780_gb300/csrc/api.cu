@@ -1151,6 +1151,10 @@ static WaveDev pack_wave(std::vector<JobDev>& jobs, size_t first, size_t last, i
     return W;
 }
 
+constexpr int64_t kMaxCov = 0xFFFFFFF0ll;  // tile records lie at 32-bit offsets, of 16 bytes
+
+static int64_t grown_cov(const Counters& hc) { return std::min<int64_t>((int64_t)(hc.need_cov * 5 / 4 + 4096), kMaxCov); }
+
 static int ensure_workspace(pv3d_ctx* c, int64_t js, int64_t te, int64_t ms, int64_t cs, int tile, bool fused,
                             int64_t ss = 0, int64_t sq = 0, int64_t sa = 0)
 {
@@ -1176,9 +1180,12 @@ static int ensure_workspace(pv3d_ctx* c, int64_t js, int64_t te, int64_t ms, int
     if (fused) {
         // tile records (one plane's bits and a header each, 16-byte units): one
         // for every tile, or 256 MiB, or one for every second module of a
-        // wave, whichever is the least that holds; grown on overflow
+        // wave, whichever is the least that holds, but no more than a quarter of
+        // the context's memory; grown on overflow
         const int64_t rec = (int64_t)tile * tile / 128 + 8;
-        c->cov_cap = std::max<int64_t>(c->cov_cap, std::min<int64_t>(te * rec + 4096, std::max<int64_t>(ms * rec / 2, 1 << 24)));
+        const int64_t first = std::min<int64_t>(te * rec + 4096, std::max<int64_t>(ms * rec / 2, 1 << 24));
+        const int64_t share = std::max<int64_t>(c->opts.hbm_budget_bytes / 64, 1 << 16);
+        c->cov_cap = std::max<int64_t>(c->cov_cap, std::min<int64_t>(std::min(first, share), kMaxCov));
         if ((rc = ensure(c, c->cov, (size_t)c->cov_cap * 16)) || (rc = ensure(c, c->touch, ms * 16))) return rc;
     }
     if (c->bin_cap == 0) c->bin_cap = 1 << 22;
@@ -1534,7 +1541,7 @@ static int evaluate_plain(pv3d_ctx* c, uint32_t gen_id, const pv3d_eval_opts* o,
         if (hc.overflow & 2u) c->map_cap_tiles = (int64_t)(hc.need_tiles * 5 / 4 + 16);
         if (hc.overflow & 4u) c->big_cap = (int64_t)(hc.need_big * 5 / 4 + 1024);
         if (hc.overflow & 8u) c->recv_cap = (int64_t)(hc.need_recv * 5 / 4 + 1024);
-        if (hc.overflow & 16u) c->cov_cap = (int64_t)(hc.need_cov * 5 / 4 + 4096);
+        if (hc.overflow & 16u) c->cov_cap = grown_cov(hc);
     }
     float ms = 0;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
@@ -2061,7 +2068,9 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
             if (hc.overflow & 1u) c->bin_cap = (int64_t)(hc.need_bins * 5 / 4 + 1024);
             if (hc.overflow & 4u) c->big_cap = (int64_t)(hc.need_big * 5 / 4 + 1024);
             if (hc.overflow & 8u) c->recv_cap = (int64_t)(hc.need_recv * 5 / 4 + 1024);
-            if (hc.overflow & 16u) c->cov_cap = (int64_t)(hc.need_cov * 5 / 4 + 4096);
+            if ((hc.overflow & 16u) && c->cov_cap == kMaxCov)
+                rc = fail(c, PV3D_E_OVERFLOW, "a wave needs more tile records than can be addressed");
+            if (hc.overflow & 16u) c->cov_cap = grown_cov(hc);
             for (auto* r : in_wave) {
                 const GenH& g = c->gens.at(r->gen_id);
                 cudaMemsetAsync(r->kmod.p, 0, (size_t)g.M * 2 * sizeof(float2), st);
