@@ -1800,6 +1800,21 @@ struct pv3d_ctx::Request {
     std::chrono::steady_clock::time_point t_submit, t_done;
 };
 
+// Scratch bytes of one step of a request: as ensure_workspace takes them, with
+// tile records for half of the modules, ...
+static int64_t wave_step_bytes(const GenH& g, const EvalSetup& es)
+{
+    const int64_t tiles = (int64_t)(es.R / es.tile) * (es.R / es.tile);
+    const int64_t rec = (int64_t)es.tile * es.tile / 128 + 8;
+    int64_t b = tiles * 4 * 11 + (int64_t)g.C + (int64_t)g.M * (sizeof(ModStep) + 12 + 16) + sizeof(LightParams) + 28;
+    b += std::min<int64_t>(tiles, (g.M + 1) / 2) * rec * 16;
+    if (es.strings) b += (int64_t)g.M * 4 + (int64_t)g.n_sub_tot * 4 + (int64_t)g.str_ids.size() * 8;
+    if (es.arrays) b += (int64_t)g.arr_ids.size() * 8;
+    return b;
+}
+
+// ... and as a request is admitted by: an upper bound for any but the smallest
+// modules, without the pools that grow.
 static int64_t per_step_scratch(const GenH& g, const EvalSetup& es)
 {
     const int64_t tiles = (int64_t)(es.R / es.tile) * (es.R / es.tile);
@@ -2023,7 +2038,7 @@ static int serve_wave(pv3d_ctx* c, std::unique_lock<std::mutex>& lk)
         const GenH& g = c->gens.at(r.gen_id);
         const SceneH& sc = c->scenes.at(g.scene_id);
         int k = (int)std::min<int64_t>(r.es.K, r.es.e - r.next);
-        const int64_t per_step = per_step_scratch(g, r.es);
+        const int64_t per_step = wave_step_bytes(g, r.es);
         if (jobs.empty()) k = (int)std::max<int64_t>(1, std::min<int64_t>(k, scratch_cap / std::max<int64_t>(per_step, 1)));
         const int64_t need = per_step * k;
         if (!jobs.empty() && scratch + need > scratch_cap) break;

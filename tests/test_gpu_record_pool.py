@@ -75,3 +75,21 @@ def test_overflow_restarts_served_requests():
         torch.cuda.synchronize()
         for k in OUTS:
             np.testing.assert_array_equal(arrays[k].cpu().numpy().view(big[k].dtype), big[k], err_msg=k)
+
+
+def test_served_waves_use_their_scratch():
+    """A served wave takes as many steps as wave_scratch_mb holds of what a step
+    really takes: a byte a cell, 96 a module, 44 a tile and at most one record a
+    tile."""
+    w = S.make_tracker(seed=24, n=2, map_res=512, grid=(6, 5), terrain_n=48, spacing=3.0, n_pylons=1, step_h=1.0,
+                       days=np.array([100, 280]))
+    tiles = (512 // 64) ** 2
+    step = w.gen.n_cells + 96 * w.gen.n_modules + tiles * (44 + 16 * (64 * 64 // 128 + 8)) + 512
+    steps = w.sun.n_steps
+    per_wave = (1 << 20) // step
+    assert 2 <= per_wave < steps
+    with pv3d.Context(device=0, tile=64, wave_scratch_mb=1) as c:
+        gid = pv3d.load_workload(c, w)
+        rid, got = c.submit(gid, n=w.n, map_res=w.map_res, outputs=("energy",))
+        assert c.poll(rid, timeout_ms=-1) == pv3d.PV3D_OK
+    assert got["waves"] <= -(-steps // per_wave)
