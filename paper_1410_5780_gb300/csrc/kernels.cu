@@ -2086,7 +2086,10 @@ __global__ void __launch_bounds__(256) k_raster_map(const WaveDev* __restrict__ 
         for (int q = tid; q < TS * TS / 4; q += bd) dst[q] = t4[q];
         __syncthreads();
     }
-    if (PROF) flush_profile(B, 0u, p_visits, p_writes, p_culled);
+    if (PROF) {
+        flush_profile(B, 0u, p_visits, p_writes, p_culled);
+        flush_profile2(B, p_cand, 0u, p_dense, 0u, 0u);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -3848,6 +3851,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_cells(const Wa
 // k_sample: map path -- per (step, module) texel gathers from the HBM map,
 // depth tests, warp-ballot cell tallies, then the PV model
 // ---------------------------------------------------------------------------
+template <bool PROF>
 __global__ void __launch_bounds__(kPvThreads) k_sample(const WaveDev* __restrict__ W,
                                                        const JobDev* __restrict__ jobs, Buffers B)
 {
@@ -3861,6 +3865,7 @@ __global__ void __launch_bounds__(kPvThreads) k_sample(const WaveDev* __restrict
     const int64_t map_cap = W->map_cap_tiles;
     const int u24 = W->depth_u24;
     const int lane = threadIdx.x & 31;
+    unsigned int p_samples = 0;
     for (int64_t item = blockIdx.x; item < tot; item += gridDim.x) {
         int j = job_of(nj, item, [&](int q) { return jobs[q].it_mod; });
         const JobDev& J = jobs[j];
@@ -3901,6 +3906,7 @@ __global__ void __launch_bounds__(kPvThreads) k_sample(const WaveDev* __restrict
                 if (J.tiles_x > 0 && B.t_cnt[te] != 0u) {
                     const uint32_t slot = B.t_slot[te];
                     if (slot < map_cap) {
+                        if (PROF) ++p_samples;
                         const uint32_t key = B.map[((size_t)slot << (2 * sh)) + ((iy & tmask) << sh) + (ix & tmask)];
                         if (key != kEmpty) shaded = behind_key(d, s.bias, key, lp.dnear, lp.qscale, u24);
                     }
@@ -3931,6 +3937,7 @@ __global__ void __launch_bounds__(kPvThreads) k_sample(const WaveDev* __restrict
         module_pv(J, M, s, lp, s_cnt, s_imin, B, msi);
         __syncthreads();
     }
+    if (PROF) flush_profile(B, p_samples, 0u, 0u, 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -4441,7 +4448,7 @@ static void launch_tile_kernels(const WaveDev* W, const JobDev* d_jobs, const Bu
             cudaEventRecord(cfg.ev[3], cfg.stream);
             cudaEventRecord(cfg.ev[4], cfg.stream);
         }
-        k_sample<<<sm * 16, kPvThreads, 0, cfg.stream>>>(W, d_jobs, b);
+        k_sample<PROF><<<sm * 16, kPvThreads, 0, cfg.stream>>>(W, d_jobs, b);
     }
 }
 
