@@ -1295,7 +1295,7 @@ static int wave_graph(pv3d_ctx* c, const LaunchCfg& cfg0, int max_jobs, cudaGrap
     cfg.stream = c->cap_stream;
     cfg.ev = nullptr;
     CUDA_TRY(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t le = launch_wave((const WaveDev*)c->wave_slot.p, (const JobDev*)c->jobs_slot.p, buffers_of(c), cfg, 0);
+    cudaError_t le = launch_wave((const WaveDev*)c->wave_slot.p, (const JobDev*)c->jobs_slot.p, buffers_of(c), cfg);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
     if (le != cudaSuccess || ee != cudaSuccess || !g) {
@@ -1362,7 +1362,7 @@ static int run_waves(pv3d_ctx* c, const std::vector<WaveDev>& waves, cudaStream_
             CUDA_TRY(c, cudaGraphLaunch(exec, st));
         } else {
             if (profile) cfg.ev = &c->prof_ev[w * (kStages + 1)];
-            CUDA_TRY(c, launch_wave((const WaveDev*)c->wave_slot.p, (const JobDev*)c->jobs_slot.p, B, cfg, W.tot_te));
+            CUDA_TRY(c, launch_wave((const WaveDev*)c->wave_slot.p, (const JobDev*)c->jobs_slot.p, B, cfg));
         }
         job0 += (size_t)W.n_jobs;
     }

@@ -1348,11 +1348,6 @@ struct RecvSm {
     int item_pref;             // (row, cell column) items of the receivers staged before this one
 };
 
-template <int TS>
-struct RasterSm {
-    uint32_t tile[TS * TS];  // depth keys of the tile
-};
-
 static_assert(SubGrid<32>::blocks == 64 && SubGrid<64>::blocks == 64 && SubGrid<128>::blocks == 64,
               "a triangle's sub-block set is one 64-bit mask");
 
@@ -1364,9 +1359,7 @@ struct SubInfo {
 
 template <int TS>
 struct TileSm {
-    struct {
-        RasterSm<TS> r;
-    } u;
+    uint32_t tile[TS * TS];          // depth keys of the tile
     float dlim[SubGrid<TS>::blocks]; // per sub-block depth limit (sub_limits)
     SubInfo si;                      // their summary (sub_summary)
     uint32_t mask[TS * TS / 32];     // texels read by some sample (sparse tiles)
@@ -1374,7 +1367,6 @@ struct TileSm {
     RecvSm recv[kRecvChunk];
     int n_recv;                      // receivers staged
     int total_items;                 // (sample row, cell column) items over the staged receivers
-    int any_write;                   // some texel of the tile received a depth
     TriSetup tri[kTriBatchMax];      // a batch of set-up triangles, one per thread
     int row_pref[kTriBatchMax + 1];  // prefix of their rows
 };
@@ -1801,7 +1793,7 @@ __device__ __forceinline__ int setup_raster_tri(const JobDev& J, const Buffers& 
 template <int TS, bool PROF>
 __device__ __forceinline__ void draw_rows(const TriSetup* tri, const int* row_pref, int nb, int u_beg, int u_end,
                                           const uint32_t* mask, uint32_t* tile, const LightParams& lp, int u24,
-                                          bool& wrote, unsigned int& visits, unsigned int& writes)
+                                          unsigned int& visits, unsigned int& writes)
 {
     constexpr int WPR = TS / 32;
     constexpr int SWS = (TS == 128 ? 7 : (TS == 64 ? 6 : 5)) - 3;
@@ -1853,7 +1845,6 @@ __device__ __forceinline__ void draw_rows(const TriSetup* tri, const int* row_pr
                 const float w1 = __fmaf_rn(A1, px, t1);
                 const float w2 = __fmaf_rn(A2, px, t2);
                 atomicMin(&tile[iy * TS + ix], depth_store_key(depth_at(w0, w1, w2, e0, e1, e2), lp, u24));
-                wrote = true;
                 if (PROF) { ++visits; ++writes; }
             }
         }
@@ -1877,7 +1868,7 @@ __device__ __forceinline__ void tile_limits(TileSm<TS>& sm, const LightParams& l
     __syncthreads();
 }
 
-// Rasterise the tile's triangles into sm.u.r.tile.  Sparse tiles (fewer samples
+// Rasterise the tile's triangles into sm.tile.  Sparse tiles (fewer samples
 // than two per texel) are rasterised only at the texels their samples read.
 // A triangle is drawn only in the sub-blocks where it may shade a sample
 // (tri_sub_mask with the sub-block depth limits): the stored nearest depth
@@ -1887,11 +1878,10 @@ __device__ __forceinline__ void tile_limits(TileSm<TS>& sm, const LightParams& l
 // (triangle, row) goes to one lane, which visits only the texels of the row
 // inside all three edges (edge_span), of the triangle's sub-blocks and, in
 // sparse tiles, marked.  Receivers [r0, r0 + nrecv) must be staged (the
-// first kRecvChunk of them) on entry.  Returns 0 if no sample reads the tile
-// or nothing was drawn at a texel a sample reads.
+// first kRecvChunk of them) on entry.
 template <int TS, bool PROF>
-__device__ int tile_raster(TileSm<TS>& sm, const JobDev& J, const Buffers& B, const WaveDev* W, int ls, int tx,
-                           int ty, int64_t te, uint64_t r0, int nrecv, bool limits_ready, unsigned int& visits,
+__device__ void tile_raster(TileSm<TS>& sm, const JobDev& J, const Buffers& B, const WaveDev* W, int ls, int tx,
+                           int ty, int64_t te, uint64_t r0, int nrecv, unsigned int& visits,
                            unsigned int& writes, unsigned int& culled, unsigned int& cand, unsigned int& dense_n)
 {
     constexpr int WPR = TS / 32;
@@ -1908,7 +1898,7 @@ __device__ int tile_raster(TileSm<TS>& sm, const JobDev& J, const Buffers& B, co
     // the texels that samples read
     const bool dense = est >= 2 * TS * TS;
     if (PROF && threadIdx.x == 0 && dense) ++dense_n;
-    if (!limits_ready) tile_limits<TS>(sm, lp, u24, cull_ok);
+    tile_limits<TS>(sm, lp, u24, cull_ok);
     int n_need = TS * TS;
     if (!dense) {
         for (int q = tid; q < TS * WPR; q += bd) sm.mask[q] = 0u;
@@ -1933,12 +1923,10 @@ __device__ int tile_raster(TileSm<TS>& sm, const JobDev& J, const Buffers& B, co
         __syncthreads();
         n_need = sm.n_need;
     }
-    uint4* t4 = reinterpret_cast<uint4*>(sm.u.r.tile);
+    uint4* t4 = reinterpret_cast<uint4*>(sm.tile);
     for (int q = tid; q < TS * TS / 4; q += bd) t4[q] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
-    if (tid == 0) sm.any_write = 0;
     __syncthreads();
-    if (n_need == 0) return 0;
-    bool wrote = false;
+    if (n_need == 0) return;
     const float ox = (float)(tx * TS), oy = (float)(ty * TS);
     const uint64_t off = B.t_off[te];
     uint64_t cnt = B.t_cnt[te];
@@ -1958,16 +1946,11 @@ __device__ int tile_raster(TileSm<TS>& sm, const JobDev& J, const Buffers& B, co
         // each warp takes a contiguous range of the batch's rows
         const int n_rows = sm.row_pref[nb];
         draw_rows<TS, PROF>(sm.tri, sm.row_pref, nb, (int)(((int64_t)n_rows * warp) / n_warps),
-                            (int)(((int64_t)n_rows * (warp + 1)) / n_warps), dense ? nullptr : sm.mask, sm.u.r.tile,
-                            lp, u24, wrote, visits, writes);
+                            (int)(((int64_t)n_rows * (warp + 1)) / n_warps), dense ? nullptr : sm.mask, sm.tile,
+                            lp, u24, visits, writes);
         __syncthreads();
     }
-    if (wrote) sm.any_write = 1;
-    __syncthreads();
-    // no triangle reaches a texel that a sample reads: every sample is lit
-    return sm.any_write ? n_need : 0;
 }
-
 // Add per-thread work counters to the global profile counters (warp-reduced).
 __device__ __forceinline__ void flush_profile(const Buffers& B, unsigned int samples, unsigned int visits,
                                               unsigned int writes, unsigned int culled)
@@ -2079,9 +2062,9 @@ __global__ void __launch_bounds__(256) k_raster_map(const WaveDev* __restrict__ 
         tile_receivers(B, W, te, r0, nrecv);
         stage_receivers<TS>(sm, J, B, ls, tx, ty, r0, min(nrecv, kRecvChunk));
         // the tile is stored even when nothing was drawn: its samples read it
-        tile_raster<TS, PROF>(sm, J, B, W, ls, tx, ty, te, r0, nrecv, false, p_visits, p_writes, p_culled, p_cand,
+        tile_raster<TS, PROF>(sm, J, B, W, ls, tx, ty, te, r0, nrecv, p_visits, p_writes, p_culled, p_cand,
                               p_dense);
-        const uint4* t4 = reinterpret_cast<const uint4*>(sm.u.r.tile);
+        const uint4* t4 = reinterpret_cast<const uint4*>(sm.tile);
         uint4* dst = reinterpret_cast<uint4*>(B.map + ((size_t)item * (TS * TS)));
         for (int q = tid; q < TS * TS / 4; q += bd) dst[q] = t4[q];
         __syncthreads();
@@ -4452,13 +4435,11 @@ static void launch_tile_kernels(const WaveDev* W, const JobDev* d_jobs, const Bu
     }
 }
 
-cudaError_t launch_wave(const WaveDev* d_wave, const JobDev* d_jobs, const Buffers& b, const LaunchCfg& cfg,
-                        int64_t tot_te_host)
+cudaError_t launch_wave(const WaveDev* d_wave, const JobDev* d_jobs, const Buffers& b, const LaunchCfg& cfg)
 {
     const WaveDev* W = d_wave;
     cudaStream_t st = cfg.stream;
     const int sm = cfg.sm_count;
-    (void)tot_te_host;
     if (cfg.ev) cudaEventRecord(cfg.ev[0], st);
     k_clear<<<sm * 8, 256, 0, st>>>(W, d_jobs, b);
     k_window<<<sm * 8, kWinPerItem, 0, st>>>(W, d_jobs, b);

@@ -275,7 +275,7 @@ constexpr int kMaxArraySub = 512;        // bypass substrings an array of parall
 // once per context, before any launch: the block-per-tile kernels' dynamic shared tile
 cudaError_t prepare_tile_kernels();
 cudaError_t launch_wave(const WaveDev* d_wave, const JobDev* d_jobs, const Buffers& b,
-                        const LaunchCfg& cfg, int64_t tot_te_host);
+                        const LaunchCfg& cfg);
 cudaError_t launch_finalize_pairs(const float2* kmod, int n_mods, const float2* kcell, int n_cells,
                                   double* energy, double* energy_u, double* cell_loss, cudaStream_t stream);
 // clear-sky sun table: steps k * step_h (k < per_day) of n / per_day days from day_first;
