@@ -64,3 +64,37 @@ def test_every_plane_has_bits(tile):
         p = c.last_profile()
     assert p["texel_visits"] > 0
     assert p["texel_writes"] - p["texel_visits"] < 0.1 * p["texel_visits"], p
+
+
+@pytest.mark.parametrize("tile", [32, 64, 128])
+@pytest.mark.parametrize("n", [1, 2, 5])
+def test_few_samples_in_large_cells(n, tile):
+    """Cells of some 26 x 26 texels: 27 texels a sample for n = 5, where a
+    cell's samples are looked up without a look at its box, and up to 680."""
+    w = _stack(12, n, 1024, True)
+    outputs = ("cell_counts", "sample_bits", "power")
+    with pv3d.Context(device=0, tile=tile) as c:
+        gid = pv3d.load_workload(c, w)
+        f = run_gpu(c, gid, w, outputs=outputs)
+        m = run_gpu(c, gid, w, outputs=outputs, path=pv3d.PV3D_PATH_MAP)
+    for k in outputs:
+        np.testing.assert_array_equal(f[k], m[k], err_msg=f"n {n}, tile {tile}: {k}")
+    assert 0 < f["cell_counts"].sum() < f["cell_counts"].size * n * n
+
+
+@pytest.mark.parametrize("tile", [32, 64, 128])
+def test_suns_along_the_plane_shade_some_and_light_some(tile):
+    """The steps with the sun within a degree of the modules' plane (no plane to
+    compare with), taken by themselves."""
+    from test_gpu_coverage import CASES
+    w = CASES["grazing"]()
+    w.map_res = max(w.map_res, tile)
+    normal = np.cross(w.gen.u[0], w.gen.v[0]).astype(np.float64)
+    near = np.abs(w.sun.xyz @ normal) < math.sin(math.radians(1.0))
+    assert near.sum() >= 5
+    with pv3d.Context(device=0, tile=tile) as c:
+        gid = pv3d.load_workload(c, w)
+        f = run_gpu(c, gid, w, outputs=("cell_counts",))["cell_counts"][near].astype(np.int64)
+        m = run_gpu(c, gid, w, outputs=("cell_counts",), path=pv3d.PV3D_PATH_MAP)["cell_counts"][near]
+    np.testing.assert_array_equal(f, m)
+    assert 0 < f.sum() < f.size * w.n * w.n
