@@ -39,16 +39,6 @@ METRIC = "shadow sample tests/sec (sun steps x cell samples) at 1 GB300"
 UNIT = "tests/s"
 L2_FLUSH_BYTES = 512 << 20  # > 129 MB L2
 
-# algorithmic ALU work of the tile kernel (the roofline numerator).  The
-# method's depth map must hold, at every texel a sample reads, the nearest of
-# the triangles covering the texel centre: each such (texel, triangle)
-# fragment costs 3 edge functions (2 FMA each) + barycentric depth (3 FMA) +
-# key conversion and minimum (3) = 12 lane-ops; a sample test costs its
-# position (2), projection to texel space and depth (6), floor/clamp/tile
-# check (4), depth compare (2) = 14 lane-ops.
-OPS_PER_TEXEL_WRITE = 12
-OPS_PER_SAMPLE_TEST = 14
-
 
 def parse():
     ap = argparse.ArgumentParser()
@@ -500,45 +490,29 @@ def measured_peaks() -> dict:
         return {}
 
 
-def tile_kernel_rooflines(work, stages_ms, tile, n_waves, hbm_gbs, alu_tops, raster_peak, workload):
-    """Roofline figures of the two tile kernels per launch (one launch a wave).
+def tile_kernel_rooflines(work, stages_ms, tile, n_waves, hbm_gbs, workload):
+    """The two tile kernels together against the copy bandwidth, per wave.
 
-    Algorithmic work per launch, from the work counters of one evaluation:
-    * bytes (the HBM byte model of a depth-map design restricted to the
-      kernel's tiles): 4 B per texel of every tile it takes (the depth tile
-      written once) + 4 B per sample it tests (the texel gather);
-    * lane-ops: 12 per fragment (a triangle in front of or across a receiver
-      plane covering a texel: 3 edge functions, barycentric depth, key and
-      minimum) + 14 per sample test (position, projection, texel, compare);
-    * fragments F against the atomicMin rate of the same writes.
-    The kernels do less: a fragment is a bit of a row's span, and the samples
-    are looked up in k_cells (the PV stage).
+    Bytes a wave's tile kernels cannot do without, from the work counters of
+    one evaluation: of every (triangle, tile) pair its id and three vertices
+    (4 + 48 B), and of every non-empty tile its entries in six lists (24 B) and
+    one plane's coverage bits (an eighth of a byte a texel).
     """
     nw = max(n_waves, 1)
-    heavy = {"tiles": work["heavy_tiles"], "samples": work["heavy_sample_tests"],
-             "fragments": work["heavy_texel_writes"], "ms": stages_ms["heavy"]}
-    warp = {"tiles": work["nonempty_tiles"] - work["heavy_tiles"],
-            "samples": work["sample_tests"] - work["heavy_sample_tests"],
-            "fragments": work["texel_writes"] - work["heavy_texel_writes"], "ms": stages_ms["raster"]}
-    out = {}
-    for name, k in (("k_tile_warp", warp), ("k_raster_test", heavy)):
-        launch_ms = k["ms"] / nw
-        t = max(launch_ms * 1e-3, 1e-12)
-        byts = (4.0 * tile * tile * k["tiles"] + 4.0 * k["samples"]) / nw
-        ops = (OPS_PER_TEXEL_WRITE * k["fragments"] + OPS_PER_SAMPLE_TEST * k["samples"]) / nw
-        gbs = byts / t / 1e9
-        tops = ops / t / 1e12
-        d = {"avg_launch_ms": launch_ms, "ms_per_step": k["ms"],
-             "per_launch": {"tiles": k["tiles"] / nw, "sample_tests": k["samples"] / nw,
-                            "fragments": k["fragments"] / nw, "algorithmic_bytes": byts, "lane_ops": ops},
-             "hbm": {"achieved": gbs, "peak": hbm_gbs, "unit": "GB/s", "frac": gbs / hbm_gbs},
-             "alu": {"achieved": tops, "peak": alu_tops, "unit": "T lane-ops/s", "frac": tops / alu_tops},
-             "traffic": profiled_traffic(workload, tile, name)}
-        if name == "k_raster_test" and raster_peak:
-            fr = k["fragments"] / nw / t / 1e9
-            d["raster"] = {"achieved": fr, "peak": raster_peak, "unit": "G atomicMin/s", "frac": fr / raster_peak}
-        out[name] = d
-    return out
+    ms = stages_ms["raster"] + stages_ms["heavy"]
+    byts = (52.0 * work["binned_tris"] + (24.0 + tile * tile / 8.0) * work["nonempty_tiles"]) / nw
+    gbs = byts / max(ms / nw * 1e-3, 1e-12) / 1e9
+    heavy = work["heavy_tiles"]
+    return {"achieved": gbs, "frac": gbs / hbm_gbs, "ms_per_step": ms, "avg_wave_ms": ms / nw,
+            "per_wave": {"pairs": work["binned_tris"] / nw, "tiles": work["nonempty_tiles"] / nw,
+                         "algorithmic_bytes": byts},
+            "kernels": {
+                "k_tile_warp": {"ms_per_step": stages_ms["raster"], "tiles": (work["nonempty_tiles"] - heavy) / nw,
+                                "texels_drawn": (work["texel_writes"] - work["heavy_texel_writes"]) / nw,
+                                "traffic": profiled_traffic(workload, tile, "k_tile_warp")},
+                "k_raster_test": {"ms_per_step": stages_ms["heavy"], "tiles": heavy / nw,
+                                  "texels_drawn": work["heavy_texel_writes"] / nw,
+                                  "traffic": profiled_traffic(workload, tile, "k_raster_test")}}}
 
 
 def path_byte_model(w, work, tile, chunk, n_steps_lit, t_ms_per_step):
@@ -623,19 +597,9 @@ def measure(args, name, dev, dist, rank, world, steps, warmup, tile=0, chunk=0):
     if rank != 0:
         return out
     peaks = measured_peaks()
-    sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     hbm = float(peaks.get("hbm_gbs", 6800.0))
-    props = torch.cuda.get_device_properties(dev)
-    alu_peak = props.multi_processor_count * 128 * sm_max * 1e6 / 1e12  # T lane-ops/s
     stages = {s_: float(prof[f"{s_}_ms"]) for s_ in pv3d.STAGES}
-    raster_peak = None
-    try:
-        raster_peak = pv3d.raster_peak(dev)["g_atomics_per_s"]
-    except (AttributeError, pv3d.PV3DError, OSError):
-        raster_peak = None
-    kern = tile_kernel_rooflines(work, stages, tuned["tile"], prof["waves"], hbm, alu_peak, raster_peak, name)
-    dom = max(kern, key=lambda k: kern[k]["ms_per_step"])
-    kd = kern[dom]
+    kern = tile_kernel_rooflines(work, stages, tuned["tile"], prof["waves"], hbm, name)
     lit = int(results[-1]["steps_lit"])
     t_step = t_ms / steps
     model = path_byte_model(w, work, tuned["tile"], chunk, lit, t_step / max(world, 1) * max(world, 1))
@@ -646,17 +610,15 @@ def measure(args, name, dev, dist, rank, world, steps, warmup, tile=0, chunk=0):
                        waves_per_step=int(prof["waves"]), annual_loss_pct=round(e_loss, 4),
                        timed_path="production: each wave a replayed CUDA graph, no stage events",
                        autotuned={"tile": tuned["tile"], "chunk_steps": chunk, "bin_capacity": tuned["bin_capacity"]}),
-        "roofline": {"bound": "hbm", "kernel": dom, "achieved": kd["hbm"]["achieved"], "peak": hbm, "unit": "GB/s",
-                     "frac": kd["hbm"]["frac"], "traffic": kd["traffic"],
+        "roofline": {"bound": "instruction issue (the fraction is of the copy bandwidth)",
+                     "kernel": "k_tile_warp + k_raster_test", "peak": hbm, "unit": "GB/s",
                      "peak_source": "hbm_gbs of MEASURED_PEAKS.json (measured copy bandwidth)",
-                     "algorithmic": "4 B per texel of each tile the kernel takes (depth tile written once) + 4 B per "
-                                    "sample it tests (texel gather), per launch (one wave), over its average launch "
-                                    "time (stage events of an untimed run of the same evaluation)",
-                     "traffic_source": f"DRAM read+write bytes of one launch, ncu capture in profiles/{dom}_{name}*.md "
+                     "algorithmic": "52 B per (triangle, tile) pair + 24 B and one plane's coverage bits per non-empty "
+                                    "tile, over the time of both kernels (stage events of an untimed run of the same "
+                                    "evaluation)",
+                     "traffic_source": f"DRAM read+write bytes of one launch, ncu captures in profiles/*_{name}*.md "
                                        "taken with the same tile side (null if the code of kernels.cu changed since)",
-                     "alu": kd["alu"], "per_launch": kd["per_launch"], "avg_launch_ms": kd["avg_launch_ms"],
-                     "alu_peak_source": f"{props.multi_processor_count} SMs x 128 FP32 lanes x {sm_max:.0f} MHz",
-                     "kernels": kern, "path_byte_model": model},
+                     **kern, "path_byte_model": model},
         "work_per_step": {"sample_tests_in_tested_tiles": work["sample_tests"] / max(lit, 1),
                           "fragments": work["texel_writes"] / max(lit, 1),
                           "nonempty_tiles": work["nonempty_tiles"] / max(lit, 1),
