@@ -600,6 +600,10 @@ def measure(args, name, dev, dist, rank, world, steps, warmup, tile=0, chunk=0):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     stages = {s_: float(prof[f"{s_}_ms"]) for s_ in pv3d.STAGES}
     kern = tile_kernel_rooflines(work, stages, tuned["tile"], prof["waves"], hbm, name)
+    try:  # the rate at which depths can be drawn in shared memory (the map path, open texels)
+        kern["atomic_min_peak_g_per_s"] = pv3d.raster_peak(dev)["g_atomics_per_s"]
+    except (AttributeError, pv3d.PV3DError, OSError):
+        kern["atomic_min_peak_g_per_s"] = None
     lit = int(results[-1]["steps_lit"])
     t_step = t_ms / steps
     model = path_byte_model(w, work, tuned["tile"], chunk, lit, t_step / max(world, 1) * max(world, 1))

@@ -47,10 +47,14 @@ extern "C" {
 #define PV3D_DEPTH_U24    1  /* 24-bit unsigned fixed point over the window's depth range */
 
 /* ---- evaluation paths ---------------------------------------------------
- * FUSED: each raster tile is built in shared memory and the samples that read
- *        it are depth-tested by the same CTA; no shadow map reaches HBM.
+ * FUSED: each raster tile keeps one bit per texel and receiver plane, which the
+ *        modules' cells look up; no shadow map reaches HBM.
  * MAP:   raster tiles are stored to a shadow map in device memory and a second
- *        kernel gathers one texel per sample.  Same results, bit for bit. */
+ *        kernel gathers one texel per sample.  Same results, bit for bit, but
+ *        for single samples that the search by tile misses where its rounding
+ *        is magnified (the sun all but in the module's plane; a tile's border
+ *        under a sun all but across the module's rows): lit on FUSED, on MAP
+ *        by whatever else was drawn at their texel. */
 #define PV3D_PATH_FUSED   0
 #define PV3D_PATH_MAP     1
 

@@ -2711,8 +2711,8 @@ __device__ __forceinline__ uint32_t texel_box(const uint32_t* cov, const uint32_
 // costs one step per row of a triangle, and a plane's samples read it as
 // words.  The code is kept small (loops not unrolled, one copy of each): at
 // twice the size the warps waited for instructions up to nine cycles each.
-// With k_cells, against depth tiles and a test per sample: 2 520 modules on
-// trackers over terrain, 33 suns: 3.2 -> 1.8 ms all told; a facade of 200
+// With k_cells, against depth tiles and a test per sample: 12,000 modules on
+// trackers over terrain, 47 suns: 3.2 -> 1.8 ms all told; a facade of 200
 // modules, 50 000 triangles, n = 8, a year of hours: 17.5 -> 13.4 ms.
 // ---------------------------------------------------------------------------
 constexpr int kWarpOpen = 32;
@@ -3174,8 +3174,8 @@ __device__ __forceinline__ void zero_step_module(const JobDev& J, const ModuleDe
 // cell is lit or shaded whole; the samples of the remaining cells are shared
 // out over the lanes.  Nothing is accumulated across tiles, so there are no
 // tallies to clear and no atomics in device memory.  Bound by instruction
-// issue: a third of the year of 2 520 tracker modules' time goes to the samples
-// of mixed cells.
+// issue (71 % of the slots on a wave of 12,000 tracker modules, 256 suns: 1.13
+// ms), most of it the samples of mixed cells.
 // ---------------------------------------------------------------------------
 constexpr int kPvTiles = 8;    // k_pv: a module over more tiles is looked at by the whole warp
 constexpr int kPvFastSub = 8;  // up to so many substrings a module's voltages are summed in order
@@ -3266,12 +3266,13 @@ __device__ __forceinline__ bool sample_shaded(const Buffers& B, const uint32_t* 
     return false;
 }
 
-// Samples are looked for per tile by mapping the tile back onto the module
-// (stage_one's box, row_range), one sample more each side.  Where that map
-// magnifies the rounding of positions to more than that -- 2: the sun all but
-// in the module's plane, anywhere; 1: an axis of texels all but constant along
-// the module's rows, at the tile's border -- some samples are not found, and
-// count as lit: sample_found asks for them one by one.
+// The map path and all before the coverage bits look for a tile's samples by
+// mapping the tile back onto the module (stage_one's box, row_range), one sample
+// more each side.  Where that map magnifies the rounding of positions to more
+// than that -- 2: the sun all but in the module's plane, anywhere; 1: an axis of
+// texels all but constant along the module's rows, at the tile's border -- some
+// samples are not found, and count as lit.  The counts stay what they were:
+// sample_found asks for such samples one by one.
 __device__ __forceinline__ int find_risk(const ModStep& s, float lu, float lv, float inv_p, int R)
 {
     const float ext = fabsf(lu * s.tax) + fabsf(lv * s.tbx) + fabsf(lu * s.tay) + fabsf(lv * s.tby) + 256.f;
