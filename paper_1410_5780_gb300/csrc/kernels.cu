@@ -2524,7 +2524,9 @@ __device__ __forceinline__ void draw_tris(DrawSm& D, const TriWork& w, uint32_t 
             float ia = a, ib = a - 1.f, ja = a, jb = a - 1.f;  // in the band: [ia, ib] less [ja, jb]
             if (!below(ga, gb, fr - err2, -0.02f, fa, fb)) fb = fa - 1.f;
             if (!below(ga, gb, bk + err2, 0.02f, ca, cb)) continue;
-            if ((cb - ca) - (fb - fa) > kBandTexels) {
+            if (!(bk < FLT_MAX)) {  // no plane to compare with
+                ib = b;
+            } else if ((cb - ca) - (fb - fa) > kBandTexels) {
                 ib = jb = b;
                 if (!below(ga, gb, bk - err2, -0.02f, ia, ib)) ib = ia - 1.f;
                 if (!below(ga, gb, fr + err2, 0.02f, ja, jb)) jb = ja - 1.f;
